@@ -358,11 +358,30 @@ __device__ __forceinline__ float scaled_rest_sum(const float* v)
     }
 }
 
+// The flow part of the macros: u*, the fluid-solid force, the corrected
+// velocity and the pressure of Eq. (26) from the nine flow deviations (in units
+// of 1/SF) and m.p1, m.Fx, m.Fy, which the caller has set.
+template <int SF>
+__device__ __forceinline__ void flow_macros(const float* h, Macro& m)
+{
+    constexpr float iF = 1.0f / SF;
+    float jx = (h[1] - h[3] + h[5] - h[6] - h[7] + h[8]) * iF;
+    float jy = (h[2] - h[4] + h[5] + h[6] - h[7] - h[8]) * iF;
+    float rest = (h[1] + h[2] + h[3] + h[4] + h[5] + h[6] + h[7] + h[8]) * iF;
+    float usx = jx + 0.5f * m.Fx, usy = jy + 0.5f * m.Fy;   // u*
+    float qt = 1.0f - 0.5f * m.p1;                         // q~ = (1 - phi)/2
+    m.fsx = -usx;
+    m.fsy = -usy;
+    m.ux = usx + 0.5f * (1.0f - qt) * m.fsx;
+    m.uy = usy + 0.5f * (1.0f - qt) * m.fsy;
+    // p = cs^2/(1 - w0) (sum_{i!=0} h_i - w0 |u|^2/(2 cs^2)) with w0 = 4/9
+    m.p = 0.6f * (rest - (2.0f / 3.0f) * (m.ux * m.ux + m.uy * m.uy));
+}
+
 template <int SN = 1, int SF = 1>
 __device__ __forceinline__ Macro node_macros(const float* f, const float* n, const float* g, const float* h,
                                              const StepParams& P)
 {
-    constexpr float iF = 1.0f / SF;
     Macro m;
     m.p1 = f[0] + f[1] + f[2] + f[3] + f[4];
     m.phi = m.p1 - 1.0f;
@@ -375,17 +394,7 @@ __device__ __forceinline__ Macro node_macros(const float* f, const float* n, con
     m.U = U_of(m.dC, m.p1, P.k);
     m.Fx = P.Fx;
     m.Fy = P.Fy + P.gbT * m.dth + P.gbC * (m.dC + P.dC_ref);
-    float jx = (h[1] - h[3] + h[5] - h[6] - h[7] + h[8]) * iF;
-    float jy = (h[2] - h[4] + h[5] + h[6] - h[7] - h[8]) * iF;
-    float rest = (h[1] + h[2] + h[3] + h[4] + h[5] + h[6] + h[7] + h[8]) * iF;
-    float usx = jx + 0.5f * m.Fx, usy = jy + 0.5f * m.Fy;   // u*
-    float qt = 1.0f - 0.5f * m.p1;                         // q~ = (1 - phi)/2
-    m.fsx = -usx;
-    m.fsy = -usy;
-    m.ux = usx + 0.5f * (1.0f - qt) * m.fsx;
-    m.uy = usy + 0.5f * (1.0f - qt) * m.fsy;
-    // p = cs^2/(1 - w0) (sum_{i!=0} h_i - w0 |u|^2/(2 cs^2)) with w0 = 4/9
-    m.p = 0.6f * (rest - (2.0f / 3.0f) * (m.ux * m.ux + m.uy * m.uy));
+    flow_macros<SF>(h, m);
     return m;
 }
 

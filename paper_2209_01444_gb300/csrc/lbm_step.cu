@@ -477,117 +477,118 @@ __global__ void __launch_bounds__(TX* TYV, (LBM_BATCH_WARPS / TYV > 0 ? LBM_BATC
     }
 }
 
-// v as a store to flow plane q and a load would return it (16-bit storage
-// rounds; FP32 keeps v).
-template <class Store>
-__device__ __forceinline__ float stored_flow(int q, float v)
-{
-    if constexpr (std::is_same<Store, StoreF32>::value) {
-        return v;
-    } else {
-        return Conv<typename Store::T>::to(Conv<typename Store::T>::from(v * Store::scale(q))) * Store::inv_scale(q);
-    }
-}
-
 // Flow populations the flow-only wall pass gives a wall node of `side` (axis
-// 0: left/right columns, 1: bottom/top rows) from its interior node at offset
-// oi, whose flow populations are hi: extrapolation with that node's macros,
-// its scalar populations read from sc.
-template <class Store>
-__device__ __forceinline__ void flow_wall_from(const StepParams& P, const void* __restrict__ sc, int axis, int side,
-                                               long long oi, const float (&hi)[9], float (&hb)[9])
+// 0: left/right columns, 1: bottom/top rows) from its interior node, whose flow
+// populations are hi and whose phi + 1 and F_y (from its scalar populations)
+// are sc.x and sc.y.
+__device__ __forceinline__ void flow_wall_from(const StepParams& P, int axis, int side, float2 sc,
+                                               const float (&hi)[9], float (&hb)[9])
 {
-    float fi[5], ni[5], gi[5], nb[5], gb[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) fi[i] = Store::load(sc, nullptr, kF + i, oi, P);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) ni[i] = Store::load(sc, nullptr, kN + i, oi, P);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) gi[i] = Store::load(sc, nullptr, kG + i, oi, P);
-    const Macro m = node_macros(fi, ni, gi, hi, P);
-    wall_rest(P, axis, P.bc[side], m, ni, gi, hi, nb, gb, hb, 1);
+    Macro m;
+    m.p1 = sc.x;
+    m.Fx = P.Fx;
+    m.Fy = sc.y;
+    flow_macros<1>(hi, m);
+    const float none[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    float nb[5], gb[5];
+    wall_rest(P, axis, P.bc[side], m, none, none, hi, nb, gb, hb, 1);
 }
 
-// The flow populations the flow-only wall pass (rows, then columns) would
-// have left at wall node (x, y) after the previous flow step, which skipped
-// it: a row node from its interior node; a column node from its interior
-// node; a corner from the row node beside it as the row pass leaves it.
+// phi + 1 and F_y of the node at offset o, from its scalar populations.
 template <class Store>
-__device__ __forceinline__ void flow_wall_repair(const StepParams& P, const void* __restrict__ sc,
-                                              const void* __restrict__ src, int x, int y, bool wx, bool wy,
-                                              float (&h)[9])
+__device__ __forceinline__ float2 flow_wall_scalars(const StepParams& P, const void* __restrict__ sc, long long o)
 {
-    const int xi = x == 0 ? 1 : P.nx - 2, yi = y == 0 ? 1 : P.ny - 2;
-    const int row_side = y == 0 ? 2 : 3, col_side = x == 0 ? 0 : 1;
-    float hi[9];
-    if (!wx) {
-        const long long oi = (long long)yi * P.pitch + x;
+    float f[5], n[5], g[5];
+    const float h[9] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-        for (int i = 0; i < 9; ++i) hi[i] = Store::load(nullptr, src, kH + i, oi, P);
-        flow_wall_from<Store>(P, sc, 1, row_side, oi, hi, h);
-    } else {
-        const long long oc = (long long)y * P.pitch + xi;
-        if (wy) {
-            const long long oi = (long long)yi * P.pitch + xi;
-            float hr[9];
+    for (int i = 0; i < 5; ++i) f[i] = Store::load(sc, nullptr, kF + i, o, P);
 #pragma unroll
-            for (int i = 0; i < 9; ++i) hr[i] = Store::load(nullptr, src, kH + i, oi, P);
-            flow_wall_from<Store>(P, sc, 1, row_side, oi, hr, hi);
+    for (int i = 0; i < 5; ++i) n[i] = Store::load(sc, nullptr, kN + i, o, P);
 #pragma unroll
-            for (int i = 0; i < 9; ++i) hi[i] = stored_flow<Store>(kH + i, hi[i]);  // as the row pass stores it
-        } else {
-#pragma unroll
-            for (int i = 0; i < 9; ++i) hi[i] = Store::load(nullptr, src, kH + i, oc, P);
-        }
-        flow_wall_from<Store>(P, sc, 0, col_side, oc, hi, h);
-    }
-    // as the wall pass would store them and this step's load return them
-#pragma unroll
-    for (int i = 0; i < 9; ++i) h[i] = stored_flow<Store>(kH + i, h[i]);
+    for (int i = 0; i < 5; ++i) g[i] = Store::load(sc, nullptr, kG + i, o, P);
+    const Macro m = node_macros(f, n, g, h, P);
+    return make_float2(m.p1, m.Fy);
 }
 
-// Flow sub-step (two-time-scaling of Sec. 4): collide and stream h with phi
-// and the force frozen at time n.  repair: the previous flow step skipped the
-// flow-only wall pass, so wall nodes first take the populations it would have
-// given them (flow_wall_repair; sc holds the newest scalar populations, whose
-// macros the wall scheme uses).
+// Collision of one flow step at a node: phi and the body force F_y frozen, h
+// the node's populations; ho in units of 1/Store::kSF (as a store takes them).
+template <class Store>
+__device__ __forceinline__ void flow_collide(const StepParams& P, float phi, float fy, const float (&h)[9],
+                                             float (&ho)[9])
+{
+    Macro m;
+    m.phi = phi;
+    m.p1 = m.phi + 1.0f;
+    m.Fx = P.Fx;
+    m.Fy = fy;
+    flow_macros<1>(h, m);
+    collide_flow<1, Store::kSF>(h, m, P.s2u, ho);
+}
+
+// The same for two nodes at once, in packed FP32 (one instruction for both):
+// the operations and their order are those of flow_macros and collide_flow.
+struct F2 {
+    float2 v;
+};
+__device__ __forceinline__ F2 f2(float a) { return {make_float2(a, a)}; }
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) { return {__ffma2_rn(a.v, b.v, c.v)}; }
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) { return {__fadd2_rn(a.v, b.v)}; }
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return fma2(b, f2(-1.0f), a); }
+__device__ __forceinline__ F2 operator*(F2 a, F2 b) { return {__fmul2_rn(a.v, b.v)}; }
+
+template <class Store>
+__device__ __forceinline__ void flow_collide2(const StepParams& P, F2 phi, F2 Fy, const F2 (&h)[9], F2 (&out)[9])
+{
+    const F2 half = f2(0.5f), third = f2(1.0f / 3.0f), Fx = f2(P.Fx);
+    const F2 ns2 = f2(-P.s2u);
+    const F2 jx = h[1] - h[3] + h[5] - h[6] - h[7] + h[8];
+    const F2 jy = h[2] - h[4] + h[5] + h[6] - h[7] - h[8];
+    const F2 rest = h[1] + h[2] + h[3] + h[4] + h[5] + h[6] + h[7] + h[8];
+    const F2 usx = fma2(half, Fx, jx), usy = fma2(half, Fy, jy);
+    const F2 nw = fma2(f2(-0.5f), phi + f2(1.0f), f2(1.0f)) + f2(-1.0f);  // q~ - 1
+    const F2 nt = nw * half;
+    const F2 u = fma2(nt, usx, usx), v = fma2(nt, usy, usy);
+    const F2 p = f2(0.6f) * fma2(f2(-(2.0f / 3.0f)), fma2(u, u, v * v), rest);
+    const F2 Fpx = fma2(nw, usx, Fx), Fpy = fma2(nw, usy, Fy);
+    const F2 mxx = h[1] + h[3] + h[5] + h[6] + h[7] + h[8];
+    const F2 myy = h[2] + h[4] + h[5] + h[6] + h[7] + h[8];
+    const F2 mxy = h[5] - h[6] + h[7] - h[8];
+    const F2 r1 = fma2(half, Fpx, u), r2 = fma2(half, Fpy, v);
+    const F2 pu = fma2(u, u, p);
+    const F2 r3 = fma2(ns2, mxx - pu, mxx);
+    const F2 r4 = fma2(ns2, myy - fma2(v, v, p), myy);
+    const F2 r5 = fma2(ns2, fma2(u * f2(-1.0f), v, mxy), mxy);
+    const F2 r6 = r2 * third, r7 = r1 * third, r8 = fma2(v, v, pu) * third;
+    const F2 hO = f2(0.5f * Store::kSF), qO = f2(0.25f * Store::kSF);
+    out[0] = r8 - (r3 + r4);
+    if (Store::kSF != 1) out[0] = out[0] * f2((float)Store::kSF);
+    out[1] = hO * (r1 + r3 - r7 - r8);
+    out[3] = hO * (r3 - r1 + r7 - r8);
+    out[2] = hO * (r2 + r4 - r6 - r8);
+    out[4] = hO * (r4 - r2 + r6 - r8);
+    out[5] = qO * (r5 + r6 + r7 + r8);
+    out[6] = qO * (r6 - r5 - r7 + r8);
+    out[7] = qO * (r5 - r6 - r7 + r8);
+    out[8] = qO * (r7 - (r5 + r6) + r8);
+}
+
+// One flow sub-step (two-time-scaling of Sec. 4): collide and stream h with phi
+// and the force frozen at time n.
 // phi: plane 0 of a node-block array of phi_np planes (the history, or the
 // frozen phi of flow-only steps, phi_np = 1: a plain plane).
 template <class Store>
 __global__ void __launch_bounds__(256, 8) k_flow_substep(const StepParams P, const void* __restrict__ src,
                                                       void* __restrict__ dst, const float* __restrict__ phi,
-                                                      int phi_np, const float* __restrict__ fb,
-                                                      const void* __restrict__ sc, int repair)
+                                                      int phi_np, const float* __restrict__ fb)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (x >= P.nx || y >= P.ny) return;
     const long long o = (long long)y * P.pitch + x;
-    float h[9];
+    float h[9], ho[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) h[i] = Store::load(nullptr, src, kH + i, o, P);
-    if (repair) {
-        const bool wx = !P.periodic_x && (x == 0 || x == P.nx - 1);
-        const bool wy = !P.periodic_y && (y == 0 || y == P.ny - 1);
-        if (wx || wy) flow_wall_repair<Store>(P, sc, src, x, y, wx, wy, h);
-    }
-    Macro m;
-    m.phi = phi[block_index(o, phi_np)];
-    m.p1 = m.phi + 1.0f;
-    m.Fx = P.Fx;
-    m.Fy = fb[o];
-    float jx = h[1] - h[3] + h[5] - h[6] - h[7] + h[8];
-    float jy = h[2] - h[4] + h[5] + h[6] - h[7] - h[8];
-    float rest = h[1] + h[2] + h[3] + h[4] + h[5] + h[6] + h[7] + h[8];
-    float usx = jx + 0.5f * m.Fx, usy = jy + 0.5f * m.Fy;
-    float qt = 1.0f - 0.5f * m.p1;
-    m.fsx = -usx;
-    m.fsy = -usy;
-    m.ux = usx + 0.5f * (1.0f - qt) * m.fsx;
-    m.uy = usy + 0.5f * (1.0f - qt) * m.fsy;
-    m.p = 0.6f * (rest - (2.0f / 3.0f) * (m.ux * m.ux + m.uy * m.uy));
-    float ho[9];
-    collide_flow<1, Store::kSF>(h, m, P.s2u, ho);
+    flow_collide<Store>(P, phi[block_index(o, phi_np)], fb[o], h, ho);
     const int xp = (x + 1 == P.nx) ? 0 : x + 1, xm = (x == 0) ? P.nx - 1 : x - 1;
     const int yp = (y + 1 == P.ny) ? 0 : y + 1, ym = (y == 0) ? P.ny - 1 : y - 1;
     const long long rY = Store::flow_row(y, P), rP = Store::flow_row(yp, P), rM = Store::flow_row(ym, P);
@@ -595,6 +596,244 @@ __global__ void __launch_bounds__(256, 8) k_flow_substep(const StepParams P, con
     const long long d9[9] = {rY + c0, rY + cP, rP + c0, rY + cM, rM + c0, rP + cP, rP + cM, rM + cM, rM + cP};
 #pragma unroll
     for (int i = 0; i < 9; ++i) Store::store_flow(dst, i, d9[i], ho[i]);
+}
+
+// Several flow steps in one launch.  A step alone moves 80 bytes per node
+// (FP32) for some 130 operations, so a step per launch is bound by L2 or HBM;
+// here a CTA takes a region of kFmW x kFmH nodes and keeps its flow populations
+// in shared memory for `ks` <= K steps.  The outermost nodes lose one ring per
+// step (their neighbours are not in the region), so the CTA writes the inner
+// (kFmW - 2 K) x (kFmH - 2 K) nodes, which are exact.
+// Per step and node, each thread reads its own populations, collides (its rows
+// in pairs, packed FP32), and after a barrier pushes them to the neighbours'
+// places, in the storage type (16-bit storage rounds at every step as a store
+// to memory would).  Wall nodes take the values of the flow-only wall pass
+// (rows, then columns) at the start of every step but the first (there when
+// `repair` is set: the launch before left them out); the last step leaves them
+// to the next launch or the pass.
+constexpr int kFmW = 64;   // region width: two warps
+constexpr int kFmY = 8;    // rows of threads
+constexpr int kFmR = 4;    // rows per thread
+constexpr int kFmH = kFmY * kFmR;
+
+// A flow population in shared memory: the storage type, in units of 1/kSF.
+template <class Store>
+__device__ __forceinline__ typename Store::T flow_enc(float vs)
+{
+    if constexpr (std::is_same<Store, StoreF32>::value)
+        return vs;
+    else
+        return Conv<typename Store::T>::from(vs);
+}
+template <class Store>
+__device__ __forceinline__ float flow_dec(typename Store::T v)
+{
+    if constexpr (std::is_same<Store, StoreF32>::value)
+        return v;
+    else
+        return Conv<typename Store::T>::to(v) * (1.0f / Store::kSF);
+}
+
+// Region with its border, then two rows and two columns of wall scalars.
+template <class Store>
+constexpr int flow_multi_smem()
+{
+    return 9 * (kFmW + 2) * (kFmH + 2) * (int)sizeof(typename Store::T) + 2 * (kFmW + kFmH) * (int)sizeof(float2);
+}
+
+template <class Store, int K>
+__global__ void __launch_bounds__(kFmW* kFmY, 2)
+    k_flow_multi(const StepParams P, const void* __restrict__ src, void* __restrict__ dst,
+                 const float* __restrict__ phi, int phi_np, const float* __restrict__ fb, const void* __restrict__ sc,
+                 int ks, int repair)
+{
+    static_assert(kFmR % 2 == 0, "rows in pairs");
+    static_assert(kFmH > 2 * K && kFmW > 2 * K, "region size");
+    using T = typename Store::T;
+    constexpr int NR = kFmR, RH = kFmH;
+    // a border of one node around the region takes what leaves it (never read),
+    // so that every push is one store at a constant offset from the node
+    constexpr int PW = kFmW + 2, PP = PW * (RH + 2), PJ = kFmY * PW;
+    constexpr int kPush[9] = {0, 1, PW, -1, -PW, PW + 1, PW - 1, -PW - 1, -PW + 1};
+    extern __shared__ float2 fm_smem[];
+    float2* rowS = fm_smem;              // [2][kFmW] scalars of the row walls' interior nodes
+    float2* colS = rowS + 2 * kFmW;      // [2][RH] and of the column walls'
+    T* s = (T*)(colS + 2 * RH);          // [9][RH + 2][PW]
+
+    const int lx = threadIdx.x, ty = threadIdx.y, t = ty * kFmW + lx;
+    const int rx0 = blockIdx.x * (kFmW - 2 * K) - K, ry0 = blockIdx.y * (RH - 2 * K) - K;
+    // node of this thread's column and rows; outside a wall there is none
+    int gx = rx0 + lx;
+    bool colx = true;
+    if (P.periodic_x)
+        gx = (gx < 0 || gx >= P.nx) ? wrap(gx, P.nx) : gx;
+    else
+        colx = gx >= 0 && gx < P.nx;
+    const int margin = K - ks;  // rings the region has in excess
+    T* const own = s + (ty + 1) * PW + lx + 1;  // row ty + kFmY j is PJ j further
+    const bool walls = (!P.periodic_x && (rx0 <= 0 || rx0 + kFmW >= P.nx)) ||
+                       (!P.periodic_y && (ry0 <= 0 || ry0 + RH >= P.ny));
+
+    float ph[NR], fy[NR];
+    bool on[NR];
+#pragma unroll
+    for (int j = 0; j < NR; ++j) {
+        const int ly = ty + kFmY * j;
+        int gy = ry0 + ly;
+        bool rowy = true;
+        if (P.periodic_y)
+            gy = (gy < 0 || gy >= P.ny) ? wrap(gy, P.ny) : gy;
+        else
+            rowy = gy >= 0 && gy < P.ny;
+        on[j] = colx && rowy && ly >= margin && ly < RH - margin;
+        const long long o = on[j] ? (long long)gy * P.pitch + gx : 0;
+        const T* e = (const T*)src + block_index(o, 9);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) own[i * PP + PJ * j] = e[32 * i];
+        ph[j] = phi[block_index(o, phi_np)];
+        fy[j] = fb[o];
+    }
+    // thread t's wall nodes in the wall pass: t < 2 kFmW a row wall's node in
+    // this thread's column (the corners belong to the columns), the next 2 RH
+    // threads a column wall's node
+    int wrow = -1, wcol = -1;  // position of the node (row wall), of the node (column wall), or -1
+    int wside = 0, win = 0;    // wall side; offset of the interior node
+    if (walls) {
+        if (!P.periodic_y && t < 2 * kFmW) {
+            const int side = t / kFmW, ly = (side ? P.ny - 1 : 0) - ry0;
+            if (ly >= 0 && ly < RH && colx && (P.periodic_x || (gx > 0 && gx < P.nx - 1))) {
+                wrow = (ly + 1) * PW + lx + 1;
+                wside = 2 + side;
+                win = side ? -PW : PW;
+                rowS[t] = flow_wall_scalars<Store>(P, sc, (long long)(side ? P.ny - 2 : 1) * P.pitch + gx);
+            }
+        }
+        const int r = t - 2 * kFmW;
+        if (!P.periodic_x && r >= 0 && r < 2 * RH) {
+            const int side = r / RH, ly = r - side * RH, cx = (side ? P.nx - 1 : 0) - rx0;
+            int yy = ry0 + ly;
+            if (P.periodic_y) yy = wrap(yy, P.ny);
+            if (cx >= 0 && cx < kFmW && yy >= 0 && yy < P.ny) {
+                wcol = (ly + 1) * PW + cx + 1;
+                wside = side;
+                win = side ? -1 : 1;
+                colS[r] = flow_wall_scalars<Store>(P, sc, (long long)yy * P.pitch + (side ? P.nx - 2 : 1));
+            }
+        }
+    }
+    auto wall_pass = [&](int w, int axis, float2 scal) {
+        if (w < 0) return;
+        float hi[9], hb[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) hi[i] = flow_dec<Store>(s[i * PP + w + win]);
+        flow_wall_from(P, axis, wside, scal, hi, hb);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) s[i * PP + w] = flow_enc<Store>(hb[i] * Store::kSF);
+    };
+    __syncthreads();
+
+    for (int k = 0;; ++k) {
+        if (walls && (k > 0 || repair)) {
+            wall_pass(wrow, 1, wrow >= 0 ? rowS[t] : make_float2(0.0f, 0.0f));
+            __syncthreads();
+            wall_pass(wcol, 0, wcol >= 0 ? colS[t - 2 * kFmW] : make_float2(0.0f, 0.0f));
+            __syncthreads();
+        }
+        F2 ho[NR / 2][9];
+#pragma unroll
+        for (int j = 0; j < NR; j += 2) {
+            F2 h[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i)
+                h[i].v = make_float2(flow_dec<Store>(own[i * PP + PJ * j]), flow_dec<Store>(own[i * PP + PJ * (j + 1)]));
+            flow_collide2<Store>(P, {make_float2(ph[j], ph[j + 1])}, {make_float2(fy[j], fy[j + 1])}, h, ho[j / 2]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < NR; ++j) {
+            // rows whose populations are exact at this step
+            const int ly = ty + kFmY * j;
+            if (!on[j] || ly < margin + k || ly >= RH - margin - k) continue;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const float2 v = ho[j / 2][i].v;
+                own[i * PP + PJ * j + kPush[i]] = flow_enc<Store>(j & 1 ? v.y : v.x);
+            }
+        }
+        __syncthreads();
+        if (k + 1 == ks) break;
+    }
+    const bool outx = lx >= K && lx < kFmW - K && rx0 + lx < P.nx;
+#pragma unroll
+    for (int j = 0; j < NR; ++j) {
+        const int ly = ty + kFmY * j;
+        if (!outx || ly < K || ly >= RH - K || ry0 + ly >= P.ny) continue;
+        const long long e = block_index((long long)(ry0 + ly) * P.pitch + rx0 + lx, 9);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) ((T*)dst)[e + 32 * i] = own[i * PP + PJ * j];
+    }
+}
+
+template <class Store, int K>
+cudaError_t launch_flow_multi(const StepParams& P, const void* src, void* dst, const float* phi, int phi_np,
+                              const float* fb, const void* sc, int ks, int repair, cudaStream_t s)
+{
+    constexpr int ow = kFmW - 2 * K, oh = kFmH - 2 * K, smem = flow_multi_smem<Store>();
+    if (smem > 48 * 1024) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k_flow_multi<Store, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return e;
+    }
+    const dim3 grid((P.nx + ow - 1) / ow, (P.ny + oh - 1) / oh);
+    k_flow_multi<Store, K><<<grid, dim3(kFmW, kFmY), smem, s>>>(P, src, dst, phi, phi_np, fb, sc, ks, repair);
+    return cudaGetLastError();
+}
+
+// Steps per launch for n >= 2 flow steps: a launch costs about its steps plus
+// 8 of them for loading, the walls' scalars and storing (1.12 M nodes, FP32:
+// 49 us for 4 steps; one step per launch took 16 us), over the share of the
+// region that a ring of K nodes leaves to write.
+inline int flow_multi_k(int n)
+{
+    int best = 2;
+    double least = 0.0;
+    for (int K : {2, 4, 5}) {
+        const double cost = (8.0 * ((n + K - 1) / K) + n) / ((kFmW - 2 * K) * (kFmH - 2 * K));
+        if (least == 0.0 || cost < least) {
+            least = cost;
+            best = K;
+        }
+    }
+    return best;
+}
+
+// n flow steps from buffer fl[*cf] (parity updated), the flow-only wall pass
+// left out after the last.  A single step has no traffic to save and goes
+// node by node; more are shared out evenly over the fewest launches.
+template <class Store>
+cudaError_t flow_chain(const StepParams& P, int n, const void* sc, void* const fl[2], int* cf, const float* phi,
+                       int phi_np, const float* fb, cudaStream_t s)
+{
+    cudaError_t e = cudaSuccess;
+    if (n == 1) {
+        const dim3 block(64, 4), grid((P.nx + 63) / 64, (P.ny + 3) / 4);
+        k_flow_substep<Store><<<grid, block, 0, s>>>(P, fl[*cf], fl[1 - *cf], phi, phi_np, fb);
+        *cf = 1 - *cf;
+        return cudaGetLastError();
+    }
+    const int K = flow_multi_k(n);
+    int repair = 0;
+    for (int left = (n + K - 1) / K; left > 0 && e == cudaSuccess; --left) {
+        const int ks = (n + left - 1) / left;
+        const auto launch = K == 2   ? launch_flow_multi<Store, 2>
+                            : K == 4 ? launch_flow_multi<Store, 4>
+                                     : launch_flow_multi<Store, 5>;
+        e = launch(P, fl[*cf], fl[1 - *cf], phi, phi_np, fb, sc, ks, repair, s);
+        n -= ks;
+        repair = 1;
+        *cf = 1 - *cf;
+    }
+    return e;
 }
 
 template <class Store>
@@ -682,16 +921,11 @@ template <class Store>
 cudaError_t flow_steps_t(const StepParams& P, int n, void* sc, void* const fl[2], int* cf, const float* phi,
                          const float* fy, cudaStream_t s)
 {
-    const dim3 fblock(64, 4), fgrid((P.nx + 63) / 64, (P.ny + 3) / 4);
-    cudaError_t e = cudaSuccess;
-    for (int k = 0; k < n; ++k) {
-        // wall pass after the last step only; each later step repairs the wall
-        // nodes it loads instead
-        k_flow_substep<Store><<<fgrid, fblock, 0, s>>>(P, fl[*cf], fl[1 - *cf], phi, 1, fy, sc, k > 0);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (k + 1 == n && (e = walls<Store>(P, sc, fl[1 - *cf], 1, s)) != cudaSuccess) return e;
-        *cf = 1 - *cf;
-    }
+    // wall pass after the last step only; each later step repairs the wall
+    // nodes it loads instead
+    if (n < 1) return cudaSuccess;
+    cudaError_t e = flow_chain<Store>(P, n, sc, fl, cf, phi, 1, fy, s);
+    if (e == cudaSuccess) e = walls<Store>(P, sc, fl[*cf], 1, s);
     return e;
 }
 
@@ -731,19 +965,16 @@ cudaError_t coupled_step(const StepParams& P, int n_sub, StepBuffers& B, cudaStr
     if ((e = walls<Store>(P, dst, dstf, 0, s, !(xwall && skip_columns))) != cudaSuccess) return e;
     B.cs = 1 - B.cs;
     B.cf = 1 - B.cf;
-    const dim3 fblock(64, 4), fgrid((P.nx + 63) / 64, (P.ny + 3) / 4);
-    for (int sub = 1; sub < n_sub; ++sub) {
+    if (n_sub > 1) {
         // phi and the force of time n come from hist/fb; the wall scheme reads
         // the scalar macros of time n+1 from the newest scalar buffer.  The
         // flow-only wall pass runs after the last sub-step only: each later
         // sub-step repairs the wall nodes it loads instead.
-        if (sub == 1 && B.ev_begin && B.ev_substeps) cudaEventRecord(B.ev_begin, s);
-        k_flow_substep<Store><<<fgrid, fblock, 0, s>>>(P, B.fl[B.cf], B.fl[1 - B.cf], B.hist, kHist, B.fb,
-                                                       B.sc[B.cs], sub > 1);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if (sub + 1 == n_sub && B.ev_end && B.ev_substeps) cudaEventRecord(B.ev_end, s);
-        if (sub + 1 == n_sub && (e = walls<Store>(P, B.sc[B.cs], B.fl[1 - B.cf], 1, s)) != cudaSuccess) return e;
-        B.cf = 1 - B.cf;
+        if (B.ev_begin && B.ev_substeps) cudaEventRecord(B.ev_begin, s);
+        if ((e = flow_chain<Store>(P, n_sub - 1, B.sc[B.cs], B.fl, &B.cf, B.hist, kHist, B.fb, s)) != cudaSuccess)
+            return e;
+        if (B.ev_end && B.ev_substeps) cudaEventRecord(B.ev_end, s);
+        if ((e = walls<Store>(P, B.sc[B.cs], B.fl[B.cf], 1, s)) != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
