@@ -182,10 +182,11 @@ LBM_API int lbm_init_fields(lbm_handle* h, const double* fields, const double* o
 /* Queue `nsteps` coupled time steps (the fused stream-collide kernel of all
  * four models, then the wall kernels, then n_sub - 1 flow-only sub-steps) on
  * the handle's stream and return without waiting.  Long runs are replayed
- * from captured 16-step CUDA graphs; inside one (n_sub = 1) the
- * left/right walls of a step are updated by the next step as it loads them,
- * and the last step of the graph runs the wall kernels in full, so the state
- * seen between calls is always complete.  The graph is captured,
+ * from captured 16-step CUDA graphs; inside one, and inside the
+ * remainder of a call, walls (n_sub = 1; on grids of more than 2^20 nodes the
+ * left/right ones) are updated by the next step as it loads them, and the last
+ * step runs the wall kernels in full, so the state seen between calls is always
+ * complete.  The graph is captured,
  * instantiated and uploaded when a state is set (lbm_init_seeds,
  * lbm_init_fields, lbm_load_state), so the first lbm_step pays none of it. */
 LBM_API int lbm_step(lbm_handle* h, int nsteps);

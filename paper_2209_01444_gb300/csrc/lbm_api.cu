@@ -358,7 +358,9 @@ int run_steps_direct(lbm_handle* h, int n)
             h->B.ev_end = h->ev[h->ev_used++];
             h->B.ev_substeps = h->prof_substeps;
         }
-        cudaError_t e = lbm::launch_coupled_step(h->P, h->storage, h->prm.n_sub, h->B, h->stream);
+        // (a profiled step runs its wall passes: its fused kernel is timed alone)
+        cudaError_t e = lbm::launch_coupled_step(h->P, h->storage, h->prm.n_sub, h->B, h->stream,
+                                                 !h->profiling && i > 0, !h->profiling && i + 1 < n);
         h->B.ev_begin = h->B.ev_end = nullptr;
         if (e != cudaSuccess) return cuda_fail(h, e, "coupled step");
     }
@@ -379,9 +381,9 @@ int graph_for(lbm_handle* h, cudaGraphExec_t* out)
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        // the left/right walls of all but the last step are updated by the
-        // next step as it loads them (see launch_coupled_step); the graph's
-        // first step takes the state as stored and its last leaves it complete
+        // the walls of all but the last step are updated by the next step as
+        // it loads them (see launch_coupled_step); the graph's first step takes
+        // the state as stored and its last leaves it complete
         for (int i = 0; i < kGraphSteps && e == cudaSuccess; ++i)
             e = lbm::launch_coupled_step(h->P, h->storage, h->prm.n_sub, h->B, cap, i > 0, i + 1 < kGraphSteps);
         cudaError_t e2 = cudaStreamEndCapture(cap, &g);
@@ -1420,7 +1422,7 @@ int batch_graph(lbm_batch* b, cudaGraphExec_t* out)
     cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     int par = b->parity;
     for (int i = 0; i < kGraphSteps && e == cudaSuccess; ++i) {
-        // left/right walls as in the single-domain graphs
+        // walls as in the single-domain graphs
         e = lbm::launch_batch_step(T, b->storage, b->ty, b->run, par, b->ctas[tyk(b->ty)], cap, i > 0,
                                    i + 1 < kGraphSteps);
         par = 1 - par;
@@ -1480,7 +1482,8 @@ int batch_run_direct(lbm_batch* b, int n)
             T.ev_begin = b->ev[b->ev_used++];
             T.ev_end = b->ev[b->ev_used++];
         }
-        LBM_BCUDA(b, lbm::launch_batch_step(T, b->storage, b->ty, b->run, b->parity, b->ctas[tyk(b->ty)], b->stream));
+        LBM_BCUDA(b, lbm::launch_batch_step(T, b->storage, b->ty, b->run, b->parity, b->ctas[tyk(b->ty)], b->stream,
+                                            !b->profiling && i > 0, !b->profiling && i + 1 < n));
         b->parity = 1 - b->parity;
     }
     return LBM_OK;

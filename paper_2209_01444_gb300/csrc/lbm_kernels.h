@@ -31,13 +31,13 @@ struct StepBuffers {
     int ev_substeps = 0;   // 0: the events bracket the fused kernel; 1: the n_sub - 1 flow sub-step kernels
 };
 
-// One coupled step.  skip_columns: leave out the column pass of the left/right
-// walls (n_sub = 1 and walls in x; ignored otherwise);
-// the next step must then be launched with `repair`, which applies that
-// update to the wall cells as they are loaded.  A state read or kept between
-// launches must come from a step without skip_columns.
+// One coupled step.  skip_walls: leave out wall passes (n_sub = 1; ignored
+// otherwise): all of them on a grid of up to kFoldNodes nodes (lbm_step.cu), the
+// left/right walls' on a larger one; the next step must then be launched with
+// `repair`, which applies that update to the wall cells as they are loaded.  A
+// state read or kept between calls must come from a step without skip_walls.
 cudaError_t launch_coupled_step(const StepParams& P, int storage, int n_sub, StepBuffers& B, cudaStream_t s,
-                                int repair = 0, int skip_columns = 0);
+                                int repair = 0, int skip_walls = 0);
 
 // One domain of a batch as the batched kernels see it: its parameters and the
 // two parities of its population buffers (n_sub = 1).
@@ -68,10 +68,10 @@ struct BatchTables {
 
 // One coupled step of every domain: buffers `parity` -> 1 - parity, then walls.
 // ty: tile height 4, 8 or 16; run: tiles per CTA (0: persistent grid of
-// `ctas` CTAs, each taking one contiguous run).  repair, skip_columns: as for
+// `ctas` CTAs, each taking one contiguous run).  repair, skip_walls: as for
 // launch_coupled_step.
 cudaError_t launch_batch_step(const BatchTables& T, int storage, int ty, int run, int parity, int ctas,
-                              cudaStream_t s, int repair = 0, int skip_columns = 0);
+                              cudaStream_t s, int repair = 0, int skip_walls = 0);
 // CTAs of the persistent batched kernel that fit on the current device at once.
 int batch_resident_ctas(int storage, int ty);
 

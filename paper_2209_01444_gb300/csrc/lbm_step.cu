@@ -16,9 +16,8 @@
 //      backward time differences of the next step.
 // Periodic wrap is applied to every streaming destination; on non-periodic
 // sides the wrapped values land on wall nodes, which the wall scheme then
-// overwrites completely: the wall kernel after the step, or, for the left and
-// right walls of steps inside a captured step graph, the next step as it
-// loads them (coupled_tile).
+// overwrites completely: the wall kernels after the step, or the next step of
+// the same call as it loads them (coupled_tile).
 #include <cuda_runtime.h>
 #include <stddef.h>
 
@@ -114,6 +113,80 @@ __device__ __forceinline__ void wall_rest(const StepParams& P, int axis, int typ
     deq_H(m.dth, P.latent * m.hp1, m.H * m.ux * sc, m.H * m.uy * sc, ef);
 #pragma unroll
     for (int i = 0; i < 5; ++i) gb[i] = eb[i] + g[i] - ef[i];
+}
+
+// v as a store to plane q and a load would return it (16-bit storage rounds
+// its planes; FP32 keeps v).
+template <class Store>
+__device__ __forceinline__ float stored(int q, float v)
+{
+    if constexpr (std::is_same<Store, StoreF32>::value) {
+        return v;
+    } else {
+        if (Store::rest(q)) return v;
+        return Conv<typename Store::T>::to(Conv<typename Store::T>::from(v * Store::scale(q))) * Store::inv_scale(q);
+    }
+}
+
+// What the wall scheme gives the wall node (xw, yw) of a freshly streamed
+// state whose wall passes (rows, then columns) have not run: its n, g and h in
+// out[0..4], [5..9], [10..18], in the units the node update takes (rest
+// populations unscaled).  A row node follows from its interior node; a column
+// node from its interior node, which in a corner is itself a row node, as the
+// row pass would store it.  Row nodes are rounded as the row pass stores them.
+// ROWS: row walls may be among them.
+template <class Store, bool ROWS>
+__device__ __forceinline__ void wall_values(const StepParams& P, const void* __restrict__ src,
+                                            const void* __restrict__ srcf, int xw, int yw, bool column, bool row,
+                                            float* __restrict__ out)
+{
+    const int xi = !column ? xw : (xw == 0 ? 1 : P.nx - 2);
+    const int yi = !row ? yw : (yw == 0 ? 1 : P.ny - 2);
+    const long long oi = (long long)yi * P.pitch + xi;
+    float f[5], n[5], g[5], h[9], fb[5], nb[5], gb[5], hb[9];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) f[i] = Store::load(src, srcf, kF + i, oi, P);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) n[i] = Store::load(src, srcf, kN + i, oi, P);
+#pragma unroll
+    for (int i = 0; i < 5; ++i) g[i] = Store::load(src, srcf, kG + i, oi, P);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) h[i] = Store::load(src, srcf, kH + i, oi, P);
+    if constexpr (ROWS) {
+        // at most two extrapolations: the row's, then the column's
+#pragma unroll 1
+        for (int axis = row ? 1 : 0; axis >= (column ? 0 : 1); --axis) {
+            const int side = axis ? (yw == 0 ? 2 : 3) : (xw == 0 ? 0 : 1);
+            const Macro m = node_macros(f, n, g, h, P);
+            wall_phi(P, P.bc[side], f, m.p1, fb);
+            wall_rest(P, axis, P.bc[side], m, n, g, h, nb, gb, hb, 0);
+#pragma unroll
+            for (int i = 0; i < 5; ++i) f[i] = axis ? stored<Store>(kF + i, fb[i]) : fb[i];
+#pragma unroll
+            for (int i = 0; i < 5; ++i) n[i] = axis ? stored<Store>(kN + i, nb[i]) : nb[i];
+#pragma unroll
+            for (int i = 0; i < 5; ++i) g[i] = axis ? stored<Store>(kG + i, gb[i]) : gb[i];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) h[i] = axis ? stored<Store>(kH + i, hb[i]) : hb[i];
+        }
+    } else {
+        const Macro m = node_macros(f, n, g, h, P);
+        wall_rest(P, 0, P.bc[xw == 0 ? 0 : 1], m, n, g, h, nb, gb, hb, 0);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) n[i] = nb[i];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) g[i] = gb[i];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) h[i] = hb[i];
+    }
+    out[0] = n[0];
+    out[5] = g[0];
+#pragma unroll
+    for (int i = 1; i < 5; ++i) out[i] = n[i] * (float)Store::kSS;
+#pragma unroll
+    for (int i = 1; i < 5; ++i) out[5 + i] = g[i] * (float)Store::kSS;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) out[10 + i] = h[i] * (float)Store::kSF;
 }
 
 // Per-node part of the coupled step for node (x, y) = tile-local (lx - 1, ly - 1):
@@ -272,61 +345,52 @@ __device__ __forceinline__ void coupled_node(const StepParams& P, void* __restri
 // grain map (read when `grain` is not null).  All threads reach the barriers,
 // so callers may loop over tiles.
 //
-// XWALL with xfix set: the left and right walls of a domain that is not
-// periodic in x were not updated after the previous step (the wall scheme's
-// column pass was skipped); the tile applies that update to the wall cells it
-// loads instead.  Extrapolation depends on the first interior node alone, and
-// the tile holding a wall column also holds that node (x = 1 or nx - 2), so
-// the result is the column pass's, without its strided sweep over 24 planes.
-// Rows (bottom/top walls) are still updated by their own pass after each step,
-// before the columns, as the corners belong to the columns.
-template <class Store, bool GRAIN, bool WRITE_FB, int TYV, bool XWALL = false>
+// WALLS with wfix set: wall passes were left out after the previous step, and
+// the tile applies their update to the wall cells it loads instead: kColumns,
+// the left and right walls; kAllWalls, the bottom and top walls too (rows
+// first: the corners belong to the columns).  Extrapolation depends on the first
+// interior node alone, and the tile and its halo hold that node for every wall
+// cell they hold, so the result is the passes'.
+enum Walls { kNoWalls, kColumns, kAllWalls };
+template <class Store, bool GRAIN, bool WRITE_FB, int TYV, int WALLS = kNoWalls>
 __device__ __forceinline__ void coupled_tile(const StepParams& P, const void* __restrict__ src,
                                              const void* __restrict__ srcf, void* __restrict__ dst,
                                              void* __restrict__ dstf, float* __restrict__ hist,
                                              const uint8_t* __restrict__ grain, float* __restrict__ fb, int x0,
                                              int y0, float (&fs)[5][TYV + 2][TX + 2], float (&ps)[TYV + 2][TX + 2],
-                                             int xfix = 0)
+                                             int wfix = 0)
 {
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int x = x0 + tx, y = y0 + ty;
     const bool active = x < P.nx && y < P.ny;
-    // XWALL: C, H and flow populations of the tile's own wall nodes, computed
+    // WALLS: C, H and flow populations of the tile's own wall nodes, computed
     // first, while no other values are held in registers
-    const bool xwall_tile = XWALL && xfix && !P.periodic_x && (x0 == 0 || x0 + TX + 1 >= P.nx);
-    __shared__ float wnb[XWALL ? 2 : 1][XWALL ? TYV : 1][19];
-    if constexpr (XWALL) {
-        static_assert(2 * (TYV + 2) <= TX * TYV && 2 * TYV <= TX * TYV, "wall-repair thread ranges");
-        const int tid = ty * TX + tx;
-        if (xwall_tile && tid < 2 * TYV) {
-            const int side = tid / TYV, r = tid % TYV;
-            const int xw = side == 0 ? 0 : P.nx - 1, xi = side == 0 ? 1 : P.nx - 2;
-            const int yw = y0 + r;
-            if (xw >= x0 && xw < x0 + TX && yw < P.ny) {
-                const long long oi = (long long)yw * P.pitch + xi;
-                float fi[5], ni[5], gi[5], hi[9], nbw[5], gbw[5], hbw[9];
-#pragma unroll
-                for (int i = 0; i < 5; ++i) fi[i] = Store::load(src, srcf, kF + i, oi, P);
-#pragma unroll
-                for (int i = 0; i < 5; ++i) ni[i] = Store::load(src, srcf, kN + i, oi, P);
-#pragma unroll
-                for (int i = 0; i < 5; ++i) gi[i] = Store::load(src, srcf, kG + i, oi, P);
-#pragma unroll
-                for (int i = 0; i < 9; ++i) hi[i] = Store::load(src, srcf, kH + i, oi, P);
-                const Macro mi = node_macros(fi, ni, gi, hi, P);
-                wall_rest(P, 0, P.bc[side], mi, ni, gi, hi, nbw, gbw, hbw, 0);
-                // in the units the node update takes (rest populations unscaled)
-                wnb[side][r][0] = nbw[0];
-                wnb[side][r][5] = gbw[0];
-#pragma unroll
-                for (int i = 1; i < 5; ++i) wnb[side][r][i] = nbw[i] * (float)Store::kSS;
-#pragma unroll
-                for (int i = 1; i < 5; ++i) wnb[side][r][5 + i] = gbw[i] * (float)Store::kSS;
-#pragma unroll
-                for (int i = 0; i < 9; ++i) wnb[side][r][10 + i] = hbw[i] * (float)Store::kSF;
+    const bool xwall_tile = WALLS && wfix && !P.periodic_x && (x0 == 0 || x0 + TX + 1 >= P.nx);
+    const bool ywall_tile =
+        WALLS == kAllWalls && wfix && !P.periodic_y && (y0 == 0 || y0 + TYV + 1 >= P.ny);
+    constexpr bool ROWS = WALLS == kAllWalls;
+    __shared__ float wcol[WALLS ? 2 : 1][WALLS ? TYV : 1][19];  // left and right columns
+    __shared__ float wrow[ROWS ? 2 : 1][ROWS ? TX : 1][19];     // bottom and top rows, corners excepted
+    if constexpr (WALLS) {
+        static_assert(2 * TX + 2 * TYV <= TX * TYV && 2 * (TX + 2) <= TX * TYV && 2 * (TYV + 2) <= TX * TYV,
+                      "wall thread ranges");
+        if (xwall_tile || ywall_tile) {
+            const int tid = ty * TX + tx;
+            if (ROWS && ywall_tile && tid < 2 * TX) {
+                const int side = tid / TX, yw = side ? P.ny - 1 : 0;
+                if (yw >= y0 && yw < y0 + TYV && x < P.nx && (P.periodic_x || (x > 0 && x < P.nx - 1)))
+                    wall_values<Store, ROWS>(P, src, srcf, x, yw, false, true, wrow[side][tx]);
             }
+            constexpr int T0 = ROWS ? 2 * TX : 0;  // first of the columns' threads
+            if (xwall_tile && tid >= T0 && tid < T0 + 2 * TYV) {
+                const int side = (tid - T0) / TYV, r = (tid - T0) % TYV;
+                const int xw = side ? P.nx - 1 : 0, yw = y0 + r;
+                if (xw >= x0 && xw < x0 + TX && yw < P.ny)
+                    wall_values<Store, ROWS>(P, src, srcf, xw, yw, true,
+                                       ROWS && !P.periodic_y && (yw == 0 || yw == P.ny - 1), wcol[side][r]);
+            }
+            __syncthreads();  // keeps the loads below after the repair
         }
-        if (xwall_tile) __syncthreads();  // keeps the loads below after the repair
     }
     // own-node loads first, so that they are in flight while the halo loads.
     // Every thread loads its own tile cell (x, y), wrapped into the grid when
@@ -394,42 +458,56 @@ __device__ __forceinline__ void coupled_tile(const StepParams& P, const void* __
     }
     __syncthreads();
 
-    if constexpr (XWALL) {
-        if (xwall_tile) {
-            // (side, row) of each wall column the tile holds: x = 0 (side 0)
-            // at tile column 1 - x0, x = nx - 1 (side 1) at nx - x0
-            const int tid = ty * TX + tx;
-            if (tid < 2 * (TYV + 2)) {
-                // phase-field populations and phi of a wall cell of the tile or its halo rows
-                const int side = tid / (TYV + 2), hy = tid % (TYV + 2);
-                const int hx = side == 0 ? 1 - x0 : P.nx - x0;
-                if (hx >= 0 && hx <= TX + 1) {
-                    const int hf = side == 0 ? hx + 1 : hx - 1;  // the interior node, never a wall (nx >= 4)
-                    float ff[5], fbw[5];
+    if constexpr (WALLS) {
+        // phase-field populations and phi of the wall cells of the tile and its
+        // halo: rows (corners excepted), then columns
+        const int tid = ty * TX + tx;
+        auto phi_cell = [&](int side, int hy, int hx, int fy, int fx) {
+            float ff[5], fbw[5];
 #pragma unroll
-                    for (int i = 0; i < 5; ++i) ff[i] = fs[i][hy][hf];
-                    wall_phi(P, P.bc[side], ff, ff[0] + ff[1] + ff[2] + ff[3] + ff[4], fbw);
-                    float sum = 0.0f;
+            for (int i = 0; i < 5; ++i) ff[i] = fs[i][fy][fx];
+            wall_phi(P, P.bc[side], ff, ff[0] + ff[1] + ff[2] + ff[3] + ff[4], fbw);
+            float sum = 0.0f;
 #pragma unroll
-                    for (int i = 0; i < 5; ++i) {
-                        fs[i][hy][hx] = fbw[i];
-                        sum += fbw[i];
-                    }
-                    ps[hy][hx] = sum;
-                }
+            for (int i = 0; i < 5; ++i) {
+                const float v = side >= 2 ? stored<Store>(kF + i, fbw[i]) : fbw[i];
+                fs[i][hy][hx] = v;
+                sum += v;
+            }
+            ps[hy][hx] = sum;
+        };
+        if (ywall_tile) {
+            if (tid < 2 * (TX + 2)) {
+                const int side = tid / (TX + 2), hx = tid % (TX + 2);
+                const int hy = side == 0 ? 1 - y0 : P.ny - y0;  // tile row of y = 0, y = ny - 1
+                const int gx = x0 - 1 + hx;
+                const bool corner = !P.periodic_x && (gx <= 0 || gx >= P.nx - 1);
+                // the interior row is never a wall (ny >= 4)
+                if (hy >= 0 && hy <= TYV + 1 && !corner) phi_cell(2 + side, hy, hx, side == 0 ? hy + 1 : hy - 1, hx);
             }
             __syncthreads();
-            if (active && (x == 0 || x == P.nx - 1)) {
-                const int side = x == 0 ? 0 : 1;
-#pragma unroll
-                for (int i = 0; i < 5; ++i) f[i] = fs[i][ty + 1][tx + 1];  // as the repair left the tile
-#pragma unroll
-                for (int i = 0; i < 5; ++i) n[i] = wnb[side][ty][i];
-#pragma unroll
-                for (int i = 0; i < 5; ++i) g[i] = wnb[side][ty][5 + i];
-#pragma unroll
-                for (int i = 0; i < 9; ++i) h[i] = wnb[side][ty][10 + i];
+        }
+        if (xwall_tile) {
+            if (tid < 2 * (TYV + 2)) {
+                // x = 0 at tile column 1 - x0, x = nx - 1 at nx - x0
+                const int side = tid / (TYV + 2), hy = tid % (TYV + 2);
+                const int hx = side == 0 ? 1 - x0 : P.nx - x0;
+                if (hx >= 0 && hx <= TX + 1) phi_cell(side, hy, hx, hy, side == 0 ? hx + 1 : hx - 1);
             }
+            __syncthreads();
+        }
+        const bool on_col = xwall_tile && (x == 0 || x == P.nx - 1);
+        const bool on_row = ywall_tile && (y == 0 || y == P.ny - 1);
+        if (active && (on_col || on_row)) {
+            const float* w = on_col || !ROWS ? wcol[x == 0 ? 0 : 1][ty] : wrow[y == 0 ? 0 : 1][tx];
+#pragma unroll
+            for (int i = 0; i < 5; ++i) f[i] = fs[i][ty + 1][tx + 1];  // as the repair left the tile
+#pragma unroll
+            for (int i = 0; i < 5; ++i) n[i] = w[i];
+#pragma unroll
+            for (int i = 0; i < 5; ++i) g[i] = w[5 + i];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) h[i] = w[10 + i];
         }
     }
 
@@ -439,16 +517,20 @@ __device__ __forceinline__ void coupled_tile(const StepParams& P, const void* __
                                                           grain != nullptr, gid, fs, ps);
 }
 
-template <class Store, bool GRAIN, bool WRITE_FB, bool XWALL = false>
-__global__ void __launch_bounds__(TX* TY, LBM_STEP_MIN_BLOCKS)
+// Resident CTAs per SM: see LBM_STEP_MIN_BLOCKS; kAllWalls with FP32 storage
+// takes one less (64 registers), as its wall code spills at 56 (1024^2 forced
+// flow 43.8 against 43.0 us per step; in 16-bit storage nine stay the faster).
+template <class Store, bool GRAIN, bool WRITE_FB, int WALLS = kNoWalls>
+__global__ void __launch_bounds__(TX* TY, LBM_STEP_MIN_BLOCKS -
+                                              (WALLS == kAllWalls && std::is_same<Store, StoreF32>::value ? 1 : 0))
     k_coupled_step(const StepParams P, const void* __restrict__ src, const void* __restrict__ srcf,
                    void* __restrict__ dst, void* __restrict__ dstf, float* __restrict__ hist,
-                   const uint8_t* __restrict__ grain, float* __restrict__ fb, int xfix = 0)
+                   const uint8_t* __restrict__ grain, float* __restrict__ fb, int wfix = 0)
 {
     __shared__ float fs[5][TY + 2][TX + 2];
     __shared__ float ps[TY + 2][TX + 2];
-    coupled_tile<Store, GRAIN, WRITE_FB, TY, XWALL>(P, src, srcf, dst, dstf, hist, grain, fb, blockIdx.x * TX,
-                                                    blockIdx.y * TY, fs, ps, xfix);
+    coupled_tile<Store, GRAIN, WRITE_FB, TY, WALLS>(P, src, srcf, dst, dstf, hist, grain, fb, blockIdx.x * TX,
+                                                    blockIdx.y * TY, fs, ps, wfix);
 }
 
 // Descriptors of the batch being stepped, in constant memory: the domain
@@ -462,7 +544,7 @@ __constant__ DomainDesc c_batch_desc[kMaxBatchDomains];
 // the domain and their halos stay in L2.  A kernel boundary separates steps.
 template <class Store, int TYV>
 __global__ void __launch_bounds__(TX* TYV, (LBM_BATCH_WARPS / TYV > 0 ? LBM_BATCH_WARPS / TYV : 1))
-    k_batch_step(const int4* __restrict__ tiles, int ntiles, int chunk, int parity, int xfix)
+    k_batch_step(const int4* __restrict__ tiles, int ntiles, int chunk, int parity, int wfix)
 {
     __shared__ float fs[5][TYV + 2][TX + 2];
     __shared__ float ps[TYV + 2][TX + 2];
@@ -470,9 +552,9 @@ __global__ void __launch_bounds__(TX* TYV, (LBM_BATCH_WARPS / TYV > 0 ? LBM_BATC
     for (int t = blockIdx.x * chunk; t < t_end; ++t) {
         const int4 tl = tiles[t];
         const DomainDesc& d = c_batch_desc[tl.x];
-        coupled_tile<Store, true, false, TYV, true>(d.P, d.sc[parity], d.fl[parity], d.sc[1 - parity],
+        coupled_tile<Store, true, false, TYV, kColumns>(d.P, d.sc[parity], d.fl[parity], d.sc[1 - parity],
                                                     d.fl[1 - parity], d.hist, d.grain, nullptr, tl.y, tl.z, fs, ps,
-                                                    xfix);
+                                                    wfix);
         __syncthreads();  // the tile arrays are reused by the next tile
     }
 }
@@ -929,8 +1011,10 @@ cudaError_t flow_steps_t(const StepParams& P, int n, void* sc, void* const fl[2]
     return e;
 }
 
+constexpr long long kFoldNodes = 1 << 20;
+
 template <class Store>
-cudaError_t coupled_step(const StepParams& P, int n_sub, StepBuffers& B, cudaStream_t s, int repair, int skip_columns)
+cudaError_t coupled_step(const StepParams& P, int n_sub, StepBuffers& B, cudaStream_t s, int repair, int skip_walls)
 {
     const dim3 block(TX, TY), grid((P.nx + TX - 1) / TX, (P.ny + TY - 1) / TY);
     const void* src = B.sc[B.cs];
@@ -939,18 +1023,30 @@ cudaError_t coupled_step(const StepParams& P, int n_sub, StepBuffers& B, cudaStr
     void* dstf = B.fl[1 - B.cf];
     const bool grain = B.grain != nullptr, wfb = n_sub > 1;
     if (B.ev_begin && !B.ev_substeps) cudaEventRecord(B.ev_begin, s);
-    // left/right walls: with skip_columns their column pass is left out and
-    // the next step, launched with `repair`, updates them at its load
-    // (coupled_tile); only steps with one flow step per coupled step do
-    // that, with flow sub-steps the column pass stays
-    const bool xwall = !wfb && !P.periodic_x;
-    const int xfix = xwall ? repair : 0;
-    if (xwall && grain)
-        k_coupled_step<Store, true, false, true>
-            <<<grid, block, 0, s>>>(P, src, srcf, dst, dstf, B.hist, B.grain, B.fb, xfix);
-    else if (xwall)
-        k_coupled_step<Store, false, false, true>
-            <<<grid, block, 0, s>>>(P, src, srcf, dst, dstf, B.hist, B.grain, B.fb, xfix);
+    // walls: with skip_walls wall passes are left out and the next step,
+    // launched with `repair`, updates the walls as it loads them
+    // (coupled_tile); only steps with one flow step per coupled step do that:
+    // flow sub-steps start from updated walls.  Up to kFoldNodes every pass is
+    // left out: two launches of few threads cost more than the wall code in the
+    // step (100^2 forced flow 5.9 -> 4.4 us per step, 777 x 500 16.0 -> 14.7);
+    // on larger grids, where the row pass is under 4 us of a step and the step's
+    // own speed counts for more (1500^2 FP16 69.4 against 70.6 us), only the
+    // columns' strided pass.
+    const bool all = !wfb && !(P.periodic_x && P.periodic_y) && (long long)P.nx * P.ny <= kFoldNodes;
+    const bool columns = !wfb && !P.periodic_x && !all;
+    const int wfix = all || columns ? repair : 0;
+    if (all && grain)
+        k_coupled_step<Store, true, false, kAllWalls>
+            <<<grid, block, 0, s>>>(P, src, srcf, dst, dstf, B.hist, B.grain, B.fb, wfix);
+    else if (all)
+        k_coupled_step<Store, false, false, kAllWalls>
+            <<<grid, block, 0, s>>>(P, src, srcf, dst, dstf, B.hist, B.grain, B.fb, wfix);
+    else if (columns && grain)
+        k_coupled_step<Store, true, false, kColumns>
+            <<<grid, block, 0, s>>>(P, src, srcf, dst, dstf, B.hist, B.grain, B.fb, wfix);
+    else if (columns)
+        k_coupled_step<Store, false, false, kColumns>
+            <<<grid, block, 0, s>>>(P, src, srcf, dst, dstf, B.hist, B.grain, B.fb, wfix);
     else if (grain && wfb)
         k_coupled_step<Store, true, true><<<grid, block, 0, s>>>(P, src, srcf, dst, dstf, B.hist, B.grain, B.fb);
     else if (grain)
@@ -962,7 +1058,7 @@ cudaError_t coupled_step(const StepParams& P, int n_sub, StepBuffers& B, cudaStr
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if (B.ev_end && !B.ev_substeps) cudaEventRecord(B.ev_end, s);
-    if ((e = walls<Store>(P, dst, dstf, 0, s, !(xwall && skip_columns))) != cudaSuccess) return e;
+    if (!(all && skip_walls) && (e = walls<Store>(P, dst, dstf, 0, s, !(columns && skip_walls))) != cudaSuccess) return e;
     B.cs = 1 - B.cs;
     B.cf = 1 - B.cf;
     if (n_sub > 1) {
@@ -981,11 +1077,12 @@ cudaError_t coupled_step(const StepParams& P, int n_sub, StepBuffers& B, cudaStr
 
 // run: tiles per CTA; 0 makes the grid persistent (one contiguous run of
 // tiles per resident CTA).
-// repair / skip_columns: as for the single-domain step; the column list holds
-// the left/right walls of every domain that is not periodic in x.
+// repair / skip_walls: as for the single-domain step on a large grid (the
+// columns); the column list holds the left/right walls of every domain that is
+// not periodic in x.
 template <class Store, int TYV>
 cudaError_t batch_step_t(const BatchTables& T, int parity, int ctas, int run, cudaStream_t s, int repair,
-                         int skip_columns)
+                         int skip_walls)
 {
     const int k = TYV == 4 ? 0 : TYV == 8 ? 1 : 2;
     const int chunk = run > 0 ? run : (T.ntiles[k] + ctas - 1) / ctas;
@@ -998,22 +1095,22 @@ cudaError_t batch_step_t(const BatchTables& T, int parity, int ctas, int run, cu
     // the fused kernel wrote buffers 1 - parity; walls act on those (rows, then columns)
     if (T.nwall[0])
         k_batch_walls<Store><<<(T.nwall[0] + 127) / 128, 128, 0, s>>>(T.descs, T.walls[0], T.nwall[0], 1 - parity);
-    if (T.nwall[1] && !skip_columns)
+    if (T.nwall[1] && !skip_walls)
         k_batch_walls<Store><<<(T.nwall[1] + 127) / 128, 128, 0, s>>>(T.descs, T.walls[1], T.nwall[1], 1 - parity);
     return cudaGetLastError();
 }
 
 template <class Store>
 cudaError_t batch_step_store(const BatchTables& T, int ty, int parity, int ctas, int run, cudaStream_t s,
-                             int repair, int skip_columns)
+                             int repair, int skip_walls)
 {
     cudaError_t e = cudaMemcpyToSymbolAsync(c_batch_desc, T.descs, sizeof(DomainDesc) * T.ndomains, 0,
                                             cudaMemcpyDeviceToDevice, s);
     if (e != cudaSuccess) return e;
     switch (ty) {
-    case 4: return batch_step_t<Store, 4>(T, parity, ctas, run, s, repair, skip_columns);
-    case 16: return batch_step_t<Store, 16>(T, parity, ctas, run, s, repair, skip_columns);
-    default: return batch_step_t<Store, 8>(T, parity, ctas, run, s, repair, skip_columns);
+    case 4: return batch_step_t<Store, 4>(T, parity, ctas, run, s, repair, skip_walls);
+    case 16: return batch_step_t<Store, 16>(T, parity, ctas, run, s, repair, skip_walls);
+    default: return batch_step_t<Store, 8>(T, parity, ctas, run, s, repair, skip_walls);
     }
 }
 
@@ -1030,12 +1127,12 @@ int batch_ctas_t()
 }  // namespace
 
 cudaError_t launch_batch_step(const BatchTables& T, int storage, int ty, int run, int parity, int ctas,
-                              cudaStream_t s, int repair, int skip_columns)
+                              cudaStream_t s, int repair, int skip_walls)
 {
     switch (storage) {
-    case kStoreF16: return batch_step_store<StoreF16>(T, ty, parity, ctas, run, s, repair, skip_columns);
-    case kStoreBF16: return batch_step_store<StoreBF16>(T, ty, parity, ctas, run, s, repair, skip_columns);
-    default: return batch_step_store<StoreF32>(T, ty, parity, ctas, run, s, repair, skip_columns);
+    case kStoreF16: return batch_step_store<StoreF16>(T, ty, parity, ctas, run, s, repair, skip_walls);
+    case kStoreBF16: return batch_step_store<StoreBF16>(T, ty, parity, ctas, run, s, repair, skip_walls);
+    default: return batch_step_store<StoreF32>(T, ty, parity, ctas, run, s, repair, skip_walls);
     }
 }
 
@@ -1057,12 +1154,12 @@ cudaError_t flow_steps(const StepParams& P, int storage, int n, void* sc, void* 
 }
 
 cudaError_t launch_coupled_step(const StepParams& P, int storage, int n_sub, StepBuffers& B, cudaStream_t s,
-                                int repair, int skip_columns)
+                                int repair, int skip_walls)
 {
     switch (storage) {
-    case kStoreF16: return coupled_step<StoreF16>(P, n_sub, B, s, repair, skip_columns);
-    case kStoreBF16: return coupled_step<StoreBF16>(P, n_sub, B, s, repair, skip_columns);
-    default: return coupled_step<StoreF32>(P, n_sub, B, s, repair, skip_columns);
+    case kStoreF16: return coupled_step<StoreF16>(P, n_sub, B, s, repair, skip_walls);
+    case kStoreBF16: return coupled_step<StoreBF16>(P, n_sub, B, s, repair, skip_walls);
+    default: return coupled_step<StoreF32>(P, n_sub, B, s, repair, skip_walls);
     }
 }
 
