@@ -22,12 +22,42 @@
 #include <stddef.h>
 
 #include <type_traits>
+#include <utility>
 
 #include "lbm_kernels.h"
 
 namespace lbm {
 
 namespace {
+
+// Programmatic dependent launch of the flow steps: a kernel is launched before
+// its predecessor on the stream has drained, so that its launch and the start
+// of its CTAs overlap the predecessor's last wave.  pdl_begin releases the
+// successor likewise and then waits until every kernel before this one has
+// completed and its writes are visible; no buffer is touched before it.  (The
+// coupled steps do without: in a captured graph their launches cost little, and
+// early CTAs took SM slots from the last wave, 1024^2 0.7 % slower.)
+__device__ __forceinline__ void pdl_begin()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <class... Par, class... Arg>
+cudaError_t launch_pdl(void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Arg&&... arg)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Arg>(arg)...);
+}
 
 constexpr int kLocalGradIters = 2;  // fixed-point passes of the local grad(phi) scheme
 
@@ -756,6 +786,7 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
     const bool walls = (!P.periodic_x && (rx0 <= 0 || rx0 + kFmW >= P.nx)) ||
                        (!P.periodic_y && (ry0 <= 0 || ry0 + RH >= P.ny));
 
+    pdl_begin();
     float ph[NR], fy[NR];
     bool on[NR];
 #pragma unroll
@@ -867,8 +898,8 @@ cudaError_t launch_flow_multi(const StepParams& P, const void* src, void* dst, c
         if (e != cudaSuccess) return e;
     }
     const dim3 grid((P.nx + ow - 1) / ow, (P.ny + oh - 1) / oh);
-    k_flow_multi<Store, K><<<grid, dim3(kFmW, kFmY), smem, s>>>(P, src, dst, phi, phi_np, fb, sc, ks, repair);
-    return cudaGetLastError();
+    return launch_pdl(k_flow_multi<Store, K>, grid, dim3(kFmW, kFmY), smem, s, P, src, dst, phi, phi_np, fb, sc, ks,
+                      repair);
 }
 
 // Steps per launch for n >= 2 flow steps: a launch costs about its steps plus
@@ -964,6 +995,7 @@ template <class Store>
 __global__ void k_walls(const StepParams P, void* __restrict__ pop, void* __restrict__ popf, int axis, int lo,
                         int count, int flow_only)
 {
+    pdl_begin();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= 2 * count) return;
     const int which = t / count;           // 0: low side, 1: high side
@@ -988,15 +1020,16 @@ __global__ void k_batch_walls(const DomainDesc* __restrict__ descs, const int4* 
 template <class Store>
 cudaError_t walls(const StepParams& P, void* sc, void* fl, int flow_only, cudaStream_t s, bool columns = true)
 {
+    cudaError_t e = cudaSuccess;
     if (!P.periodic_y) {
         const int lo = P.periodic_x ? 0 : 1, hi = P.periodic_x ? P.nx - 1 : P.nx - 2;
         const int count = hi - lo + 1;
-        k_walls<Store><<<(2 * count + 127) / 128, 128, 0, s>>>(P, sc, fl, 1, lo, count, flow_only);
+        e = launch_pdl(k_walls<Store>, (2 * count + 127) / 128, 128, 0, s, P, sc, fl, 1, lo, count, flow_only);
     }
-    if (!P.periodic_x && columns) {
-        k_walls<Store><<<(2 * P.ny + 127) / 128, 128, 0, s>>>(P, sc, fl, 0, 0, P.ny, flow_only);
+    if (e == cudaSuccess && !P.periodic_x && columns) {
+        e = launch_pdl(k_walls<Store>, (2 * P.ny + 127) / 128, 128, 0, s, P, sc, fl, 0, 0, P.ny, flow_only);
     }
-    return cudaGetLastError();
+    return e;
 }
 
 template <class Store>
