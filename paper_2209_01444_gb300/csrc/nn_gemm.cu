@@ -564,28 +564,37 @@ __device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, uint32_t parity, 
     }
 }
 
-// The warp-specialised MMA issuer's wait for its operand tiles, bounded by
-// g_operand_wait_ns; on expiry it raises the error and abort flags as
-// mbar_wait_abort does.
-__device__ __forceinline__ bool mbar_wait_operands_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag)
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar)
 {
-    const unsigned long long lim = g_operand_wait_ns;
-    const uint32_t addr = smem_u32(bar);
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// The producer and MMA warps run their loops with all lanes, so that addresses,
+// coordinates and descriptors stay in uniform registers (a single lane's would
+// be moved there for every instruction: 120 cycles per MMA whatever its width,
+// where one of 32 columns takes 32), and one elected lane issues.
+__device__ __forceinline__ uint32_t elect_lane()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p;
+}
+
+// mbar_wait_abort for a whole warp, with the same answer in every lane.  lim:
+// the wait's bound in nanoseconds (0: gives up at once).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
+                                               unsigned long long lim = kWaitNs)
+{
     const unsigned long long t0 = global_ns();
     for (uint32_t it = 0;; ++it) {
-        uint32_t done = 0;
-        if (lim != 0)
-            asm volatile(
-                "{\n\t.reg .pred p;\n\t"
-                "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                "selp.u32 %0, 1, 0, p;\n\t}"
-                : "=r"(done)
-                : "r"(addr), "r"(parity)
-                : "memory");
-        if (done) return true;
+        if (lim != 0 && __all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
         if (lim == 0 || (it & 63) == 63) {
-            if (*abort_flag) return false;
-            if (lim == 0 || global_ns() - t0 > lim) {
+            if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+            if (__any_sync(0xffffffffu, lim == 0 || global_ns() - t0 > lim)) {
                 *abort_flag = 1;
                 atomicExch(&g_gemm_error, 1);
                 return false;
@@ -594,9 +603,32 @@ __device__ __forceinline__ bool mbar_wait_operands_abort(uint64_t* bar, uint32_t
     }
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar)
+// The same instructions issued by the elected lane of a convergent warp.
+__device__ __forceinline__ void umma_lead(uint32_t lead, uint32_t d_tmem, uint32_t alo, uint32_t ahi, uint32_t blo,
+                                          uint32_t bhi, uint32_t idesc, uint32_t acc)
 {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "setp.ne.b32 q, %7, 0;\n\t"
+        "mov.b64 a, {%1, %2};\n\t"
+        "mov.b64 b, {%3, %4};\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n\t}"
+        ::"r"(d_tmem), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc), "r"(lead)
+        : "memory");
+}
+
+// Low and high words of a tile's descriptor; a tile `bytes` further has
+// bytes / 16 added to the low word (shared addresses stay below 2^18).
+template <int BK>
+__device__ __forceinline__ uint32_t tile_desc_lo(uint32_t saddr)
+{
+    return (saddr >> 4) | (1u << 16);
+}
+template <int BK>
+__device__ __forceinline__ constexpr uint32_t tile_desc_hi()
+{
+    return ((BK == 64 ? 1024u : 512u) >> 4) | (1u << 14) | ((BK == 64 ? 2u : 4u) << 29);
 }
 
 template <int BN, bool OUT_BF16, int BK, bool CONV, int MT, bool ROW3 = false>
@@ -659,9 +691,12 @@ __global__ void __launch_bounds__(kWsThreads, 1)
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {  // ---------------------------------------- producer
-            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmA) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmB) : "memory");
+        const uint32_t lead = elect_lane();
+        {  // ------------------------------------------------------ producer
+            if (lead) {
+                asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmA) : "memory");
+                asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmB) : "memory");
+            }
             int it = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
@@ -679,8 +714,9 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 }
                 for (int kb = 0; kb < nk; ++kb, ++it) {
                     const int st = it % S;
-                    if (it >= S && !(ok = mbar_wait_abort(&empty[st], (uint32_t)((it / S - 1) & 1), abort_flag)))
+                    if (it >= S && !(ok = mbar_wait_warp(&empty[st], (uint32_t)((it / S - 1) & 1), abort_flag)))
                         break;
+                    if (!lead) continue;
                     uint8_t* a = smem + st * STAGE;
                     mbar_expect_tx(&full[st], TX);
                     if constexpr (ROW3) {
@@ -711,47 +747,44 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {  // --------------------------------------------- MMA
-            int it = 0, lt = 0;
-            bool ok = true;
-            for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++lt) {
-                const int acc = lt & 1;
-                if (lt >= 2 && !(ok = mbar_wait_abort(&acc_empty[acc], (uint32_t)((lt / 2 - 1) & 1), abort_flag)))
-                    break;
+        // ------------------------------------------------------------- MMA
+        const uint32_t lead = elect_lane();
+        const unsigned long long lim = g_operand_wait_ns;
+        constexpr uint32_t HI = tile_desc_hi<BK>();
+        int it = 0, lt = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++lt) {
+            const int acc = lt & 1;
+            if (lt >= 2 && !(ok = mbar_wait_warp(&acc_empty[acc], (uint32_t)((lt / 2 - 1) & 1), abort_flag))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t d = tmem + (uint32_t)(acc * ACC_COLS);
+            for (int kb = 0; kb < nk; ++kb, ++it) {
+                const int st = it % S;
+                if (!(ok = mbar_wait_warp(&full[st], (uint32_t)((it / S) & 1), abort_flag, lim))) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint32_t d = tmem + (uint32_t)(acc * ACC_COLS);
-                for (int kb = 0; kb < nk; ++kb, ++it) {
-                    const int st = it % S;
-                    if (!(ok = mbar_wait_operands_abort(&full[st], (uint32_t)((it / S) & 1), abort_flag))) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t a0 = smem_u32(smem + st * STAGE), b0s = a0 + MT * A_BYTES;
-                    if constexpr (ROW3) {
-                        // tap kx reads the row box from pixel kx on: its A tile starts kx rows in
+                const uint32_t a0 = tile_desc_lo<BK>(smem_u32(smem + st * STAGE)), b0s = a0 + (MT * A_BYTES >> 4);
+                // tap kx of ROW3 reads the row box from pixel kx on: its A tile starts kx rows in
 #pragma unroll
-                        for (int kx = 0; kx < 3; ++kx)
+                for (int kx = 0; kx < NB; ++kx)
 #pragma unroll
-                            for (int k = 0; k < BK / 16; ++k)
+                    for (int k = 0; k < BK / 16; ++k)
 #pragma unroll
-                                for (int i = 0; i < MT; ++i)
-                                    umma(d + (uint32_t)(i * SUB_COLS),
-                                         tile_desc<BK>(a0 + i * A_BYTES + kx * BK * 2 + k * 32),
-                                         tile_desc<BK>(b0s + kx * B_BYTES + k * 32), IDESC,
-                                         (kb > 0 || kx > 0 || k > 0) ? 1u : 0u);
-                    } else {
-#pragma unroll
-                        for (int k = 0; k < BK / 16; ++k)
-#pragma unroll
-                            for (int i = 0; i < MT; ++i)
-                                umma(d + (uint32_t)(i * SUB_COLS), tile_desc<BK>(a0 + i * A_BYTES + k * 32),
-                                     tile_desc<BK>(b0s + k * 32), IDESC, (kb > 0 || k > 0) ? 1u : 0u);
-                    }
+                        for (int i = 0; i < MT; ++i)
+                            umma_lead(lead, d + (uint32_t)(i * SUB_COLS),
+                                      a0 + ((i * A_BYTES + kx * BK * 2 + k * 32) >> 4), HI,
+                                      b0s + ((kx * B_BYTES + k * 32) >> 4), HI, IDESC,
+                                      (kb > 0 || kx > 0 || k > 0) ? 1u : 0u);
+                if (lead) {
                     umma_commit(&empty[st]);
                     counts[1] = it + 1;
                 }
-                if (ok) umma_commit(&acc_full[acc]);
+                __syncwarp();
             }
-            umma_commit(done);  // completes once every MMA issued has finished
+            if (ok && lead) umma_commit(&acc_full[acc]);
+            __syncwarp();
         }
+        if (lead) umma_commit(done);  // completes once every MMA issued has finished
+        __syncwarp();
     } else {  // --------------------------------------------------- epilogue
         const int q = warp & 3;  // TMEM lane quarter this warp may access
         const int et = threadIdx.x - 64;
@@ -848,6 +881,8 @@ __global__ void __launch_bounds__(kWsThreads, 1)
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
+
+#include "nn_wgrad.cuh"
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 
@@ -1089,7 +1124,63 @@ cudaError_t launch_split_reduce_t(const float* part, int splits, int M, int N, f
     return cudaGetLastError();
 }
 
+template <int CB, int BN, int KYS>
+cudaError_t launch_wgrad(const void* X, int B, int W, int C, int cpitch, const void* dY, const WgradGeo& g, int splits,
+                         float* part, cudaStream_t s)
+{
+    constexpr int smem = wg_stages<CB, BN, KYS>() * wg_stage<CB, BN, KYS>() + 1024 + 256;
+    cudaError_t e = cudaFuncSetAttribute(k_wgrad<CB, BN, KYS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    CUtensorMap tx, ty;
+    if ((e = make_map_4d(&tx, X, B, g.H, W, C, cpitch, g.bk + 2, KYS, 1, CB)) != cudaSuccess) return e;
+    if ((e = make_map_4d(&ty, dY, B, g.H, W, g.N, g.N, g.bk, 1, 1, BN)) != cudaSuccess) return e;
+    k_wgrad<CB, BN, KYS><<<dim3(g.ncb * g.nnb * (3 / KYS), splits), kWsThreads, smem, s>>>(tx, ty, part, g);
+    return cudaGetLastError();
+}
+
 }  // namespace
+
+bool wgrad_direct_supported(int W, int C, int cpitch, int N)
+{
+    return W >= 32 && W % 32 == 0 && C >= 32 && C % 32 == 0 && cpitch % 8 == 0 && C <= cpitch && N >= 8 && N % 8 == 0;
+}
+
+cudaError_t wgrad_direct(const void* X, int B, int H, int W, int C, int cpitch, int cin, const void* dY, int N,
+                         float* dW, int ldd, cudaStream_t s, int splits, float* workspace)
+{
+    const long long P = (long long)B * H * W;
+    if (!wgrad_direct_supported(W, C, cpitch, N) || cin < 1 || cin > C || 9 * cin > ldd || !workspace || P > 0x7fffffffLL)
+        return cudaErrorInvalidValue;
+    if (((uintptr_t)X | (uintptr_t)dY | (uintptr_t)workspace) & 15) return cudaErrorInvalidValue;
+    WgradGeo g;
+    g.cin = cin;
+    g.N = N;
+    g.H = H;
+    g.bk = W % 64 == 0 ? 64 : 32;
+    g.nx = W / g.bk;
+    g.blocks = (int)(P / g.bk);
+    // slices in K blocks of 64 pixels where the rows, or a gathered copy of them
+    // (cin < C: the padded first layer), are cut so; of 32 otherwise
+    const int unit = cin < C ? 64 / g.bk : 1;
+    const int units = (g.blocks + unit - 1) / unit;
+    if (splits < 1) splits = 1;
+    if (splits > units) splits = units;
+    g.per_split = (units + splits - 1) / splits * unit;
+    splits = (g.blocks + g.per_split - 1) / g.per_split;
+    const bool wc = C % 64 == 0, wn = N % 64 == 0;
+    g.ncb = C / (wc ? 64 : 32);
+    g.nnb = (N + (wn ? 64 : 32) - 1) / (wn ? 64 : 32);
+    // one CTA for the three vertical taps where that fills three SMs of four,
+    // else one each, two CTAs to an SM
+    const bool three = 4LL * g.ncb * g.nnb * splits >= 3LL * sm_count();
+    const auto launch = wc ? (wn ? (three ? launch_wgrad<64, 64, 3> : launch_wgrad<64, 64, 1>)
+                                 : (three ? launch_wgrad<64, 32, 3> : launch_wgrad<64, 32, 1>))
+                           : (wn ? (three ? launch_wgrad<32, 64, 3> : launch_wgrad<32, 64, 1>)
+                                 : (three ? launch_wgrad<32, 32, 3> : launch_wgrad<32, 32, 1>));
+    const cudaError_t e = launch(X, B, W, C, cpitch, dY, g, splits, workspace, s);
+    if (e != cudaSuccess) return e;
+    return launch_split_reduce_t(workspace, splits, 9 * cin, N, dW, ldd, s);
+}
 
 cudaError_t gemm_bf16_tout(const void* A, int lda, const void* B, int ldb, float* D, int ldd, int M, int N, int K,
                            cudaStream_t s, int splits, float* workspace)

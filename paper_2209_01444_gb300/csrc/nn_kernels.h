@@ -51,6 +51,16 @@ bool wgrad3_supported(int B, int H, int W, int C, int cout);
 cudaError_t wgrad3_bf16(const void* XT3, const void* dYT, int B, int H, int W, int C, int cout, float* D, int ldd,
                         cudaStream_t s, int splits, float* workspace);
 
+// Weight gradient dW[N][9 cin] (pitch ldd) of a 3 x 3 zero-padded convolution
+// from its NHWC BF16 input X (C channels, pitch cpitch, of which the first cin
+// are the layer's: the others carry zeros) and output gradient dY [B H W][N];
+// W and C multiples of 32, N of 8.  The pixels are summed in `splits` slices
+// (workspace: splits x 9 cin x N floats), as wgrad3_bf16 and, for cin < C, the
+// GEMM over nine gathered taps sum them.
+bool wgrad_direct_supported(int W, int C, int cpitch, int N);
+cudaError_t wgrad_direct(const void* X, int B, int H, int W, int C, int cpitch, int cin, const void* dY, int N,
+                         float* dW, int ldd, cudaStream_t s, int splits, float* workspace);
+
 // Read (and optionally clear) the flag a GEMM raises when a bounded wait ran out.
 cudaError_t gemm_error(int* flag, bool clear);
 // Bound of the GEMMs' waits for their operand tiles on the current device.

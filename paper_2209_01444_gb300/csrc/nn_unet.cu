@@ -48,6 +48,7 @@ struct Conv {
     bf16* wf = nullptr;      // [cin][9 cout] rotated kernel for the input gradient
     bf16* wpad = nullptr;    // [cout][9 cin_pad] kernel with zero channels (first convolution only)
     int cin_pad = 0;
+    bool first = false;  // reads the network's input, stored up to kX0Pitch channels
 };
 
 struct Up {
@@ -96,6 +97,7 @@ struct lbm_unet {
     float *loss = nullptr, *part = nullptr;
     bf16 *col = nullptr, *colT = nullptr, *tA = nullptr, *tB = nullptr;
     bf16 *gA = nullptr, *gB = nullptr, *dU = nullptr;
+    long long col_n = 0;
     float* g32 = nullptr;
     float* ws = nullptr;
     long long ws_n = 0;
@@ -196,6 +198,7 @@ void plan(lbm_unet* u)
         L.W = W;
         L.P = P;
         L.ea.cin = cprev;
+        L.ea.first = l == 0;
         L.ea.cout = L.c;
         L.ea.w = add(9LL * cprev * L.c);
         L.ea.b = add(L.c);
@@ -285,6 +288,7 @@ cudaError_t allocate(lbm_unet* u)
         for (const Conv* cv : {&v.ea, &v.eb, &v.da, &v.db})
             if (cv->cout && !nn::conv3x3_supported(u->B, v.H, v.W, cv->cin)) col_n = std::max(col_n, 9 * v.P * cv->cin);
     UN_ALLOC(u->col, col_n);
+    u->col_n = col_n;
     // the table of kernel flips derive() runs in one launch (the weight and
     // flipped-weight buffers stay where they are for the network's life)
     std::vector<nn::FlipJob> jobs;
@@ -305,6 +309,10 @@ cudaError_t allocate(lbm_unet* u)
     return e;
 }
 
+// Channels of the convolution's input as the weight gradient reads them: the
+// first layer's are stored up to kX0Pitch, zero past its cin.
+int wgrad_channels(const Conv& cv) { return cv.first ? kX0Pitch : cv.cin; }
+
 // Buffers only training needs, allocated at the first backward pass.
 cudaError_t allocate_backward(lbm_unet* u)
 {
@@ -314,7 +322,10 @@ cudaError_t allocate_backward(lbm_unet* u)
     do {                                         \
         if ((e = alloc(u, &(p), (n)))) return e; \
     } while (0)
-    long long col_n = 9LL * u->P0 * kInPitch, ws_n = 0, t_n = 0, g_n = u->P0 * u->base;
+    // col: gathered copy of an output gradient whose input gradient the implicit
+    // convolution lacks; colT, tA: transposed copies where the weight gradient
+    // needs them (tA, tB: the up-convolutions')
+    long long col_n = 1, colT_n = 1, ws_n = 0, t_n = 1, g_n = u->P0 * u->base;
     const int L = u->L;
     for (int l = 0; l < L; ++l) {
         Level& v = u->lv[l];
@@ -323,9 +334,12 @@ cudaError_t allocate_backward(lbm_unet* u)
         if (l < L - 1) UN_ALLOC(v.dcat, P * 2 * c);
         for (Conv* cv : {&v.ea, &v.eb, &v.da, &v.db}) {
             if (!cv->cout) continue;
-            col_n = std::max(col_n, 9 * P * std::max(cv->cin, cv->cout));
+            if (!nn::conv3x3_supported(u->B, v.H, v.W, cv->cout)) col_n = std::max(col_n, 9 * P * cv->cout);
             ws_n = std::max(ws_n, split_ws(9 * cv->cin, cv->cout, P));
-            t_n = std::max(t_n, P * std::max(cv->cout, cv->cin));
+            if (!nn::wgrad_direct_supported(v.W, wgrad_channels(*cv), wgrad_channels(*cv), cv->cout)) {
+                colT_n = std::max(colT_n, 9 * P * cv->cin);
+                t_n = std::max(t_n, P * cv->cout);
+            }
             g_n = std::max(g_n, P * std::max(cv->cout, cv->cin));
         }
         if (v.up.cout) {
@@ -335,10 +349,13 @@ cudaError_t allocate_backward(lbm_unet* u)
             g_n = std::max(g_n, Pl * 4 * c);
         }
     }
-    bf16* col = nullptr;
-    UN_ALLOC(col, col_n);
-    u->col = col;  // the forward's smaller buffer stays allocated until destroy
-    UN_ALLOC(u->colT, col_n);
+    if (col_n > u->col_n) {
+        bf16* col = nullptr;
+        UN_ALLOC(col, col_n);
+        u->col = col;  // the forward's smaller buffer stays allocated until destroy
+        u->col_n = col_n;
+    }
+    UN_ALLOC(u->colT, colT_n);
     UN_ALLOC(u->tA, t_n);
     UN_ALLOC(u->tB, t_n);
     UN_ALLOC(u->gA, g_n);
@@ -408,19 +425,20 @@ cudaError_t conv_bwd(lbm_unet* u, const Level& v, const Conv& cv, const bf16* in
     const int K9 = 9 * cv.cin;
     cudaError_t e;
     // dW [cout][9 cin] = dY^T X_taps, computed as its transpose so that the
-    // 9 cin taps fill the MMA's 128 rows and cout (as small as 32) is the N
+    // taps and channels fill the MMA's 128 rows and cout (as small as 32) is the N
     // width; the split-K reduction writes it back as [cout][9 cin].  Where the
-    // shapes allow, only the three horizontal shifts of X are written out and
-    // the GEMM takes the vertical ones by TMA coordinates (a third of the
-    // gathered bytes); otherwise all nine taps are gathered.
-    const bool three = nn::wgrad3_supported(u->B, v.H, v.W, cv.cin, cv.cout);
-    if ((e = nn::gatherT(in, u->B, v.H, v.W, cv.cin, inpitch, three ? 3 : 9, u->colT, P, u->s))) return e;
-    if ((e = nn::gatherT(dY, u->B, v.H, v.W, cv.cout, cv.cout, 1, u->tA, P, u->s))) return e;
+    // shapes allow, straight from X and dY as they are (the first layer's input
+    // carries zero channels up to its pitch); otherwise nine transposed taps of
+    // X and the transpose of dY are written out for a plain GEMM.
     const int sp = splits_for(K9, cv.cout, P);
-    if (three)
-        e = nn::wgrad3_bf16(u->colT, u->tA, u->B, v.H, v.W, cv.cin, cv.cout, u->g + cv.w, K9, u->s, sp, u->ws);
-    else
+    const int C = wgrad_channels(cv);
+    if (nn::wgrad_direct_supported(v.W, C, inpitch, cv.cout)) {
+        e = nn::wgrad_direct(in, u->B, v.H, v.W, C, inpitch, cv.cin, dY, cv.cout, u->g + cv.w, K9, u->s, sp, u->ws);
+    } else {
+        if ((e = nn::gatherT(in, u->B, v.H, v.W, cv.cin, inpitch, 9, u->colT, P, u->s))) return e;
+        if ((e = nn::gatherT(dY, u->B, v.H, v.W, cv.cout, cv.cout, 1, u->tA, P, u->s))) return e;
         e = nn::gemm_bf16_tout(u->colT, (int)P, u->tA, (int)P, u->g + cv.w, K9, K9, cv.cout, (int)P, u->s, sp, u->ws);
+    }
     if (e) return e;
     if ((e = nn::colsum(dY, false, P, cv.cout, cv.cout, u->g + cv.b, u->part, kPartBlocks, u->s))) return e;
     if (!dx) return cudaSuccess;
