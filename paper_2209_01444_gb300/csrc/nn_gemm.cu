@@ -276,8 +276,9 @@ __device__ __forceinline__ void apply_relu_mask(float (&v)[16], const Mask16& k,
             if (!(__uint_as_float(w[j] & 0xffff0000u) > 0.0f)) v[2 * j + 1] = 0.0f;
         }
     } else {
-        for (int j = 0; j < n && j < 16; ++j)
-            if (!(__bfloat162float(m[j]) > 0.0f)) v[j] = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            if (j < n && !(__bfloat162float(m[j]) > 0.0f)) v[j] = 0.0f;
     }
 }
 
@@ -497,7 +498,9 @@ __global__ void __launch_bounds__(kThreads, 2)
                     off = q * ldd + sh.c0 + co;
                 }
                 if (col + 16 > N) {  // ragged last tile: element stores
-                    for (int j = 0; col + j < N; ++j) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        if (col + j >= N) break;
                         if (OUT_BF16)
                             ((__nv_bfloat16*)D)[off + j] = __float2bfloat16_rn(v[j]);
                         else
@@ -530,7 +533,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 // neighbouring CTAs share weight tiles and, for convolutions, input halos in
 // L2).  Warp 0 (one lane) issues the TMA loads into an S-deep ring, warp 1
 // (one lane) issues the MMAs into one of two TMEM accumulators, and warps
-// 2-5 drain the other accumulator (tcgen05.ld, bias, activation, stores), so
+// 2-9 drain the other accumulator (tcgen05.ld, bias, activation, stores), so
 // the epilogue of one tile overlaps the main loop of the next.  Every wait is
 // bounded; a wait that runs out raises the error flag and a shared abort flag
 // that makes the other roles stop, then the CTA drains its copies and MMAs
@@ -538,6 +541,9 @@ __global__ void __launch_bounds__(kThreads, 2)
 // one (tap, channel block) pair, or, in the row-reuse form (ROW3), one (input
 // row, channel block) pair whose box serves the row's three taps.
 constexpr int kWsThreads = 192;
+// Epilogue warps of k_gemm_ws: two per TMEM lane quarter.
+constexpr int kWsEpi = 8;
+constexpr int kWsGemmThreads = 64 + 32 * kWsEpi;
 
 __device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag)
 {
@@ -618,6 +624,32 @@ __device__ __forceinline__ void umma_lead(uint32_t lead, uint32_t d_tmem, uint32
         : "memory");
 }
 
+// 32 accumulator columns of this warp's 32 lanes; complete after tcgen05.wait::ld.
+__device__ __forceinline__ void tmem_ld32(uint32_t (&r)[32], uint32_t addr)
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+          "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+          "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(addr));
+}
+
+// Waits for it; the values pass through, so that no use moves before the wait.
+__device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                   "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+                   "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+                 :
+                 : "memory");
+}
+
 // Low and high words of a tile's descriptor; a tile `bytes` further has
 // bytes / 16 added to the low word (shared addresses stay below 2^18).
 template <int BK>
@@ -632,7 +664,7 @@ __device__ __forceinline__ constexpr uint32_t tile_desc_hi()
 }
 
 template <int BN, bool OUT_BF16, int BK, bool CONV, int MT, bool ROW3 = false>
-__global__ void __launch_bounds__(kWsThreads, 1)
+__global__ void __launch_bounds__(kWsGemmThreads, 1)
     k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, void* __restrict__ D,
               const float* __restrict__ bias, int M, int N, int K, int ldd, int relu, ConvGeo geo, ShuffleGeo sh,
               int tiles_m, int tiles)
@@ -672,7 +704,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(&acc_full[a], 1);
-            mbar_init(&acc_empty[a], 128);
+            mbar_init(&acc_empty[a], 32 * kWsEpi);
         }
         mbar_init(done, 1);
         *abort_flag = 0;
@@ -786,9 +818,14 @@ __global__ void __launch_bounds__(kWsThreads, 1)
         if (lead) umma_commit(done);  // completes once every MMA issued has finished
         __syncwarp();
     } else {  // --------------------------------------------------- epilogue
+        // Units of 128 rows x 32 columns, taken in turn by the two warps of each
+        // lane quarter: with one warp per quarter and 16 columns at a time the
+        // drain of an accumulator, not the MMAs, set the pace of narrow tiles
+        // (32 -> 32 channels at 4 x 512^2: 64 us, 31 us with no drain at all).
         const int q = warp & 3;  // TMEM lane quarter this warp may access
-        const int et = threadIdx.x - 64;
-        (void)et;
+        const int grp = (warp - 2) >> 2;
+        constexpr int UN = BN / 32;  // units per sub-tile
+        const bool bias4 = bias && ((uintptr_t)bias & 15) == 0;
         int lt = 0;
         for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++lt) {
             const int acc = lt & 1;
@@ -796,69 +833,82 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int n0 = (t / tiles_m) * BN;
 #pragma unroll 1
-            for (int sub = 0; sub < MT; ++sub) {
-            const int row = (t % tiles_m) * (kBM * MT) + sub * kBM + q * 32 + lane;
-            const uint32_t lane_base =
-                tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * ACC_COLS + sub * SUB_COLS);
-            long long rbase = (long long)row * ldd;
-            int sy = 0, sx = 0, sb = 0;
-            if (sh.Wl) {
-                sx = row % sh.Wl;
-                sy = (row / sh.Wl) % sh.Hl;
-                sb = row / (sh.Wl * sh.Hl);
-            }
-#pragma unroll 1
-            for (int c = 0; c < BN; c += 16) {
-                const bool mrow = sh.mask && row < M && n0 + c < N;
-                const __nv_bfloat16* mp = mrow ? sh.mask + (long long)row * sh.mpitch + n0 + c : nullptr;
-                const Mask16 mk = mrow ? load_relu_mask(mp, n0 + c + 16 <= N) : Mask16{};
-                uint32_t r[16];
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                    "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                    : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                      "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-                      "=r"(r[14]), "=r"(r[15])
-                    : "r"(lane_base + (uint32_t)c));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            for (int un = grp; un < MT * UN; un += 2) {
+                const int sub = un / UN, c = (un % UN) * 32;
+                const int row = (t % tiles_m) * (kBM * MT) + sub * kBM + q * 32 + lane;
                 const int col = n0 + c;
-                if (row < M && col < N) {
-                    float v[16];
+                uint32_t r[32];
+                tmem_ld32(r, tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * ACC_COLS + sub * SUB_COLS + c));
+                const bool all = col + 32 <= N, live = row < M && col < N;
+                float v[32];
+                if (bias4 && all) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        float x = __uint_as_float(r[j]) + ((bias && col + j < N) ? bias[col + j] : 0.0f);
-                        v[j] = relu ? fmaxf(x, 0.0f) : x;
+                    for (int j = 0; j < 8; ++j) {
+                        const float4 b = ((const float4*)(bias + col))[j];
+                        v[4 * j] = b.x;
+                        v[4 * j + 1] = b.y;
+                        v[4 * j + 2] = b.z;
+                        v[4 * j + 3] = b.w;
                     }
-                    if (mrow) apply_relu_mask(v, mk, mp, col + 16 <= N, N - col);
-                    long long off = rbase + col;
-                    if (sh.Wl) {
-                        const int sub = col / sh.c, co = col - sub * sh.c;
-                        const long long qq = ((long long)sb * 2 * sh.Hl + 2 * sy + (sub >> 1)) * (2LL * sh.Wl) +
-                                             2 * sx + (sub & 1);
-                        off = qq * ldd + sh.c0 + co;
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) v[j] = (bias && col + j < N) ? bias[col + j] : 0.0f;
+                }
+                const bool mrow = sh.mask && live;
+                const __nv_bfloat16* mp = mrow ? sh.mask + (long long)row * sh.mpitch + col : nullptr;
+                Mask16 mk[2] = {};
+                if (mrow && all) {
+                    mk[0] = load_relu_mask(mp, true);
+                    mk[1] = load_relu_mask(mp + 16, true);
+                }
+                tmem_wait32(r);
+                if (!live) continue;
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const float x = __uint_as_float(r[j]) + v[j];
+                    v[j] = relu ? fmaxf(x, 0.0f) : x;
+                }
+                long long off[2];  // of each half's first value
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    off[k] = (long long)row * ldd + col + 16 * k;
+                    if (sh.Wl) {  // the 2 x 2 pixel shuffle: 16 columns lie in one sub-pixel
+                        const int sx = row % sh.Wl, sy = (row / sh.Wl) % sh.Hl, sb = row / (sh.Wl * sh.Hl);
+                        const int sp = (col + 16 * k) / sh.c, co = col + 16 * k - sp * sh.c;
+                        const long long qq = ((long long)sb * 2 * sh.Hl + 2 * sy + (sp >> 1)) * (2LL * sh.Wl) +
+                                             2 * sx + (sp & 1);
+                        off[k] = qq * ldd + sh.c0 + co;
                     }
-                    if (col + 16 > N) {
-                        for (int j = 0; col + j < N; ++j) {
+                }
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    float(&w)[16] = *(float(*)[16])(v + 16 * k);
+                    const int left = N - col - 16 * k;
+                    if (left <= 0) break;
+                    if (mrow) apply_relu_mask(w, mk[k], mp + 16 * k, all, left);
+                    if (left < 16) {
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) {
+                            if (j >= left) break;
                             if (OUT_BF16)
-                                ((__nv_bfloat16*)D)[off + j] = __float2bfloat16_rn(v[j]);
+                                ((__nv_bfloat16*)D)[off[k] + j] = __float2bfloat16_rn(w[j]);
                             else
-                                ((float*)D)[off + j] = v[j];
+                                ((float*)D)[off[k] + j] = w[j];
                         }
                     } else if (OUT_BF16) {
                         __nv_bfloat162 h[8];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-                        uint4* dst = (uint4*)((__nv_bfloat16*)D + off);
+                        for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(w[2 * j], w[2 * j + 1]);
+                        uint4* dst = (uint4*)((__nv_bfloat16*)D + off[k]);
                         dst[0] = *(uint4*)&h[0];
                         dst[1] = *(uint4*)&h[4];
                     } else {
-                        float4* dst = (float4*)((float*)D + off);
+                        float4* dst = (float4*)((float*)D + off[k]);
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
-                            dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                            dst[j] = make_float4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
                     }
                 }
-            }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             mbar_arrive(&acc_empty[acc]);
@@ -967,14 +1017,14 @@ cudaError_t launch_ws_mt(const CUtensorMap& a, const CUtensorMap& b, void* D, co
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
         int occ = 0;
         if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_gemm_ws<BN, OUT_BF16, BK, CONV, MT, ROW3>,
-                                                               kWsThreads, smem)))
+                                                               kWsGemmThreads, smem)))
             return e;
         per_sm = occ < 1 ? 1 : occ;
     }
     const int tiles_m = (M + kBM * MT - 1) / (kBM * MT);
     const int tiles = tiles_m * ((N + BN - 1) / BN);
     const int grid = tiles < sms * per_sm ? tiles : sms * per_sm;
-    k_gemm_ws<BN, OUT_BF16, BK, CONV, MT, ROW3><<<grid, kWsThreads, smem, s>>>(a, b, D, bias, M, N, K, ldd, relu, geo,
+    k_gemm_ws<BN, OUT_BF16, BK, CONV, MT, ROW3><<<grid, kWsGemmThreads, smem, s>>>(a, b, D, bias, M, N, K, ldd, relu, geo,
                                                                                sh, tiles_m, tiles);
     return cudaGetLastError();
 }
