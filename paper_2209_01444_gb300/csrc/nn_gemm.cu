@@ -624,6 +624,19 @@ __device__ __forceinline__ void umma_lead(uint32_t lead, uint32_t d_tmem, uint32
         : "memory");
 }
 
+// 32 bytes to dst, 16-byte aligned: one store of a whole sector where dst allows.
+__device__ __forceinline__ void store32(void* dst, const uint32_t* w)
+{
+    if (((uintptr_t)dst & 31) == 0) {
+        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]), "r"(w[1]),
+                     "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                     : "memory");
+    } else {
+        ((uint4*)dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        ((uint4*)dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    }
+}
+
 // 32 accumulator columns of this warp's 32 lanes; complete after tcgen05.wait::ld.
 __device__ __forceinline__ void tmem_ld32(uint32_t (&r)[32], uint32_t addr)
 {
@@ -899,14 +912,10 @@ __global__ void __launch_bounds__(kWsGemmThreads, 1)
                         __nv_bfloat162 h[8];
 #pragma unroll
                         for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(w[2 * j], w[2 * j + 1]);
-                        uint4* dst = (uint4*)((__nv_bfloat16*)D + off[k]);
-                        dst[0] = *(uint4*)&h[0];
-                        dst[1] = *(uint4*)&h[4];
+                        store32((__nv_bfloat16*)D + off[k], (const uint32_t*)h);
                     } else {
-                        float4* dst = (float4*)((float*)D + off[k]);
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            dst[j] = make_float4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+                        store32((float*)D + off[k], (const uint32_t*)w);
+                        store32((float*)D + off[k] + 8, (const uint32_t*)(w + 8));
                     }
                 }
             }
