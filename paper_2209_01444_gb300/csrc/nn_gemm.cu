@@ -247,6 +247,10 @@ struct ShuffleGeo {
     // output was mask; null: no mask
     const __nv_bfloat16* mask = nullptr;
     int mpitch = 0;
+    // FP32 output whose columns from c on are rounded to BF16 into dU, gathered
+    // by 2 x 2 sub-pixels of the Wf x Hf image of the rows (conv3x3_split)
+    __nv_bfloat16* dU = nullptr;
+    int Wf = 0, Hf = 0;
 };
 
 // The ReLU mask of 16 output columns: m[row][col .. col + 15] loaded before
@@ -899,7 +903,14 @@ __global__ void __launch_bounds__(kWsGemmThreads, 1)
                     const int left = N - col - 16 * k;
                     if (left <= 0) break;
                     if (mrow) apply_relu_mask(w, mk[k], mp + 16 * k, all, left);
-                    if (left < 16) {
+                    if (!OUT_BF16 && sh.dU && col + 16 * k >= sh.c) {
+                        const int x = row % sh.Wf, y = (row / sh.Wf) % sh.Hf, b = row / (sh.Wf * sh.Hf);
+                        const long long q = ((long long)b * (sh.Hf / 2) + y / 2) * (sh.Wf / 2) + x / 2;
+                        __nv_bfloat162 h[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(w[2 * j], w[2 * j + 1]);
+                        store32(sh.dU + (q * 4 + (y & 1) * 2 + (x & 1)) * sh.c + col + 16 * k - sh.c, (const uint32_t*)h);
+                    } else if (left < 16) {
 #pragma unroll
                         for (int j = 0; j < 16; ++j) {
                             if (j >= left) break;
@@ -1405,15 +1416,49 @@ bool conv3x3_supported(int B, int H, int W, int C)
     return C % 32 == 0 && conv_tile(B, H, W, &bw, &bh, &bb);
 }
 
+static cudaError_t conv3x3(const void* X, int B, int H, int W, int C, int cpitch, const void* Wm, int ldw, void* D,
+                           int ldd, const float* bias, int N, bool out_bf16, bool relu, const ShuffleGeo& sh,
+                           cudaStream_t s);
+
 cudaError_t conv3x3_bf16(const void* X, int B, int H, int W, int C, int cpitch, const void* Wm, int ldw, void* D,
                          int ldd, const float* bias, int N, bool out_bf16, bool relu, cudaStream_t s,
                          const void* mask, int mpitch)
 {
+    int bw, bh, bb;
+    if (C % 32 || !conv_tile(B, H, W, &bw, &bh, &bb)) return cudaErrorNotSupported;
+    if (mask && !mask_ok(mask, mpitch, out_bf16, N)) return cudaErrorInvalidValue;
+    if (N > ldd) return cudaErrorInvalidValue;
+    ShuffleGeo sh;
+    sh.mask = (const __nv_bfloat16*)mask;
+    sh.mpitch = mpitch;
+    return conv3x3(X, B, H, W, C, cpitch, Wm, ldw, D, ldd, bias, N, out_bf16, relu, sh, s);
+}
+
+bool conv3x3_split_supported(int B, int H, int W, int c)
+{
+    return H % 2 == 0 && W % 2 == 0 && conv3x3_supported(B, H, W, c);
+}
+
+cudaError_t conv3x3_split(const void* X, int B, int H, int W, int c, const void* Wm, float* D, void* dU,
+                          cudaStream_t s)
+{
+    if (!conv3x3_split_supported(B, H, W, c) || ((uintptr_t)dU & 15)) return cudaErrorInvalidValue;
+    ShuffleGeo sh;
+    sh.c = c;
+    sh.dU = (__nv_bfloat16*)dU;
+    sh.Wf = W;
+    sh.Hf = H;
+    return conv3x3(X, B, H, W, c, c, Wm, 9 * c, D, c, nullptr, 2 * c, false, false, sh, s);
+}
+
+static cudaError_t conv3x3(const void* X, int B, int H, int W, int C, int cpitch, const void* Wm, int ldw, void* D,
+                           int ldd, const float* bias, int N, bool out_bf16, bool relu, const ShuffleGeo& sh,
+                           cudaStream_t s)
+{
     const int bk = C % 64 == 0 ? 64 : C % 32 == 0 ? 32 : 0;
     int bw, bh, bb;
     if (!bk || !conv_tile(B, H, W, &bw, &bh, &bb)) return cudaErrorNotSupported;
-    if (mask && !mask_ok(mask, mpitch, out_bf16, N)) return cudaErrorInvalidValue;
-    if (N < 8 || N % 8 || cpitch % 8 || C > cpitch || ldw % 8 || ldw < 9 * C || ldd % 8 || N > ldd)
+    if (N < 8 || N % 8 || cpitch % 8 || C > cpitch || ldw % 8 || ldw < 9 * C || ldd % 8)
         return cudaErrorInvalidValue;
     if (((uintptr_t)X | (uintptr_t)Wm | (uintptr_t)D) & 15) return cudaErrorInvalidValue;
     const int bn = bn_for(N);
@@ -1431,9 +1476,6 @@ cudaError_t conv3x3_bf16(const void* X, int B, int H, int W, int C, int cpitch, 
     geo.cblocks = C / bk;
     geo.row3 = row3 ? 1 : 0;
     const int M = B * H * W, K = 9 * C;
-    ShuffleGeo sh;
-    sh.mask = (const __nv_bfloat16*)mask;
-    sh.mpitch = mpitch;
     return bk == 64 ? dispatch<64, true>(bn, out_bf16, ta, tb, D, bias, M, N, K, ldd, relu ? 1 : 0, 1, 1 << 30, geo,
                                          sh, s)
                     : dispatch<32, true>(bn, out_bf16, ta, tb, D, bias, M, N, K, ldd, relu ? 1 : 0, 1, 1 << 30, geo,

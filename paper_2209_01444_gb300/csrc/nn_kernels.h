@@ -35,6 +35,15 @@ cudaError_t conv3x3_bf16(const void* X, int B, int H, int W, int C, int cpitch, 
 
 bool conv3x3_supported(int B, int H, int W, int C);
 
+// The input gradient of a decoder's first convolution, whose input is the
+// concatenation [skip, up] of c channels each: the implicit convolution of X
+// [P][c] with Wm [2c][9c], its first c columns stored to D (FP32 [P][c]), the
+// others rounded to BF16 into dU[(b, y/2, x/2)][((y&1) 2 + (x&1)) c + co], the
+// layout of the up-convolution's output.  c a multiple of 32.
+bool conv3x3_split_supported(int B, int H, int W, int c);
+cudaError_t conv3x3_split(const void* X, int B, int H, int W, int c, const void* Wm, float* D, void* dU,
+                          cudaStream_t s);
+
 // 2 x 2 stride-2 up-convolution: the GEMM of X [B*Hl*Wl][cin] with Wm [4c][cin]
 // plus bias[4c], stored BF16 straight into Y[b][2y+dy][2x+dx][c0 + co] (pitch
 // ypitch) from column (dy * 2 + dx) * c + co; c a multiple of 16.

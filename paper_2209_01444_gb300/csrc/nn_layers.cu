@@ -378,6 +378,63 @@ __global__ void k_maxpool_bwd8(const bf16* __restrict__ X, int B, int H, int W, 
     }
 }
 
+// out = BF16((skip + the pooled path's gradient) masked by X > 0): the max-pool
+// backward, its sum with the skip connection's gradient, the ReLU mask of the
+// pooled layer and the rounding for the next GEMM in one pass (as k_maxpool_bwd8
+// and k_mask_cast8, which write and read the FP32 sum in between: 86 + 46 us at
+// 1 M pixels of 32 channels against 48).  Thread layout of k_maxpool_bwd8.
+__global__ void k_pool_mask_bwd8(const bf16* __restrict__ X, int B, int H, int W, int C, int xpitch,
+                                 const float* __restrict__ dY, const float* __restrict__ skip, int spitch,
+                                 bf16* __restrict__ out)
+{
+    const int Ho = H / 2, Wo = W / 2;
+    const int c = 8 * threadIdx.x;
+    const long long p = (long long)blockIdx.x * blockDim.y + threadIdx.y;
+    if (p >= (long long)B * Ho * Wo) return;
+    const int x = (int)(p % Wo);
+    const long long r = p / Wo;
+    const int y = (int)(r % Ho), b = (int)(r / Ho);
+    float v[4][8];
+    long long off[4];
+    float4 sk[4][2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        off[k] = ((long long)b * H + 2 * y + k / 2) * W + 2 * x + k % 2;
+        const uint4 q = *(const uint4*)(X + off[k] * xpitch + c);
+        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            v[k][2 * j] = __uint_as_float(w[j] << 16);
+            v[k][2 * j + 1] = __uint_as_float(w[j] & 0xffff0000u);
+        }
+        sk[k][0] = *(const float4*)(skip + off[k] * spitch + c);
+        sk[k][1] = *(const float4*)(skip + off[k] * spitch + c + 4);
+    }
+    const float4 g0 = *(const float4*)(dY + p * C + c), g1 = *(const float4*)(dY + p * C + c + 4);
+    const float g[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+    int arg[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        arg[j] = 0;
+        float best = v[0][j];
+#pragma unroll
+        for (int k = 1; k < 4; ++k)
+            if (v[k][j] > best) {
+                arg[j] = k;
+                best = v[k][j];
+            }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float a[8] = {sk[k][0].x, sk[k][0].y, sk[k][0].z, sk[k][0].w, sk[k][1].x, sk[k][1].y, sk[k][1].z, sk[k][1].w};
+        __align__(16) bf16 o[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            o[j] = __float2bfloat16(v[k][j] > 0.0f ? a[j] + (arg[j] == k ? g[j] : 0.0f) : 0.0f);
+        *(uint4*)(out + off[k] * C + c) = *(const uint4*)o;
+    }
+}
+
 // U[(b, y, x)][(dy, dx, c)] (2 x 2 up-convolution output) -> Y[b, 2y + dy, 2x + dx, c0 + c].
 __global__ void k_shuffle_fwd(const bf16* __restrict__ U, int B, int H, int W, int C, bf16* __restrict__ Y,
                               int ypitch, int c0)
@@ -585,11 +642,19 @@ __global__ void k_proj_bwd_x4(const float* __restrict__ dY, int P, int O, const 
 // 8 (t % G) .. + 7 of every (256 / G)-th pixel of the block's chunk from one
 // 16-byte load; the threads of one channel group are added by shuffles within
 // each warp and then over the warps through shared memory, in a fixed order.
+// dXb (or null): also the input gradient, masked by X > 0 (X the output of a
+// ReLU) and rounded to BF16 [P][C], from the same loads.
 template <int O>
 __global__ void __launch_bounds__(256) k_proj_bwd_w8(const float* __restrict__ dY, const bf16* __restrict__ X, int P,
-                                                     int C, int xpitch, int chunk, float* __restrict__ part)
+                                                     int C, int xpitch, int chunk, float* __restrict__ part,
+                                                     const float* __restrict__ Wt, bf16* __restrict__ dXb)
 {
     __shared__ float sm[8][8][O * 9];  // [warp][group][o * 9 + k], k = 8: the bias
+    __shared__ float wsh[O * 64];      // the weights (C <= 64)
+    if (dXb) {
+        for (int i = threadIdx.x; i < O * C; i += 256) wsh[i] = Wt[i];
+        __syncthreads();
+    }
     const int G = C >> 3, lanes = 256 / G;
     const int cg = threadIdx.x % G, pl = threadIdx.x / G;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -608,12 +673,22 @@ __global__ void __launch_bounds__(256) k_proj_bwd_w8(const float* __restrict__ d
             x[2 * k] = __uint_as_float(w[k] << 16);
             x[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
         }
+        float dx[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int o = 0; o < O; ++o) {
             const float d = dY[(long long)p * O + o];
 #pragma unroll
             for (int k = 0; k < 8; ++k) acc[o][k] += d * x[k];
             acc[o][8] += d;
+            if (dXb)
+#pragma unroll
+                for (int k = 0; k < 8; ++k) dx[k] += d * wsh[o * C + 8 * cg + k];
+        }
+        if (dXb) {
+            __align__(16) bf16 b[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) b[k] = __float2bfloat16(x[k] > 0.0f ? dx[k] : 0.0f);
+            *(uint4*)(dXb + (long long)p * C + 8 * cg) = *(const uint4*)b;
         }
     }
     // lanes with the same group differ in the bits above log2(G)
@@ -654,20 +729,34 @@ __global__ void k_flip3x3(const bf16* __restrict__ W, int cout, int cin, bf16* _
     Wf[i] = W[((long long)co * 9 + (8 - tf)) * cin + ci];
 }
 
-// Every kernel of a network in one launch: element i belongs to the last job
-// whose start is <= i (at most a few tens of jobs, scanned in order).
-__global__ void k_flip3x3_many(const FlipJob* __restrict__ jobs, int njobs, long long total)
+// Every kernel of a network in one launch, by 32 x 32 tiles of (co, ci) of one
+// tap through shared memory, so that reads and writes are contiguous (by
+// elements, reading scattered: 67 us for the five-level network's 7.8 M weights).
+// Block i belongs to the last job whose start is <= i (at most a few tens of
+// jobs, scanned in order).
+__global__ void k_flip3x3_many(const FlipJob* __restrict__ jobs, int njobs)
 {
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= total) return;
+    __shared__ bf16 t[32][33];
+    const long long i = blockIdx.x;
     int j = 0;
     while (j + 1 < njobs && jobs[j + 1].start <= i) ++j;
     const FlipJob jb = jobs[j];
-    const long long k = i - jb.start;
-    const int co = (int)(k % jb.cout);
-    const long long r = k / jb.cout;
-    const int tf = (int)(r % 9), ci = (int)(r / 9);
-    ((bf16*)jb.Wf)[k] = ((const bf16*)jb.W)[((long long)co * 9 + (8 - tf)) * jb.cin + ci];
+    const int tc = (jb.cout + 31) / 32, ti = (jb.cin + 31) / 32;
+    int k = (int)(i - jb.start);
+    const int co0 = (k % tc) * 32;
+    k /= tc;
+    const int ci0 = (k % ti) * 32, tap = k / ti;
+    for (int r = threadIdx.y; r < 32; r += 8) {
+        const int co = co0 + r, ci = ci0 + threadIdx.x;
+        if (co < jb.cout && ci < jb.cin)
+            t[r][threadIdx.x] = ((const bf16*)jb.W)[((long long)co * 9 + (8 - tap)) * jb.cin + ci];
+    }
+    __syncthreads();
+    for (int r = threadIdx.y; r < 32; r += 8) {
+        const int ci = ci0 + r, co = co0 + threadIdx.x;
+        if (co < jb.cout && ci < jb.cin)
+            ((bf16*)jb.Wf)[((long long)ci * 9 + tap) * jb.cout + co] = t[threadIdx.x][r];
+    }
 }
 
 // Wp[co][t * cin_pad + ci] = W[co][t * cin + ci] for ci < cin, else 0: the
@@ -846,6 +935,33 @@ __global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float
     if (wb) wb[i] = __float2bfloat16(wi);
 }
 
+// The same, four weights per thread (16-byte aligned arrays, n a multiple of 4).
+__global__ void k_adam4(float4* __restrict__ w, const float4* __restrict__ g, float4* __restrict__ m,
+                        float4* __restrict__ v, long long n4, float lr, float b1, float b2, float eps, float c1,
+                        float c2, uint2* __restrict__ wb)
+{
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (i >= n4) return;
+    const float4 g4 = g[i];
+    float4 m4 = m[i], v4 = v[i], w4 = w[i];
+    auto step = [&](float gi, float& mi, float& vi, float& wi) {
+        mi = b1 * mi + (1.0f - b1) * gi;
+        vi = b2 * vi + (1.0f - b2) * gi * gi;
+        wi = wi - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    };
+    step(g4.x, m4.x, v4.x, w4.x);
+    step(g4.y, m4.y, v4.y, w4.y);
+    step(g4.z, m4.z, v4.z, w4.z);
+    step(g4.w, m4.w, v4.w, w4.w);
+    m[i] = m4;
+    v[i] = v4;
+    w[i] = w4;
+    if (wb) {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(w4.x, w4.y), hi = __floats2bfloat162_rn(w4.z, w4.w);
+        wb[i] = make_uint2(*(const uint32_t*)&lo, *(const uint32_t*)&hi);
+    }
+}
+
 // FP32 [P][F] fields -> BF16 NHWC [P][cpitch] with (x - mean) / std per field
 // and zero extra channels.
 // One thread per pixel: F <= 8 fields in, cpitch BF16 channels out as
@@ -986,6 +1102,22 @@ cudaError_t maxpool_bwd(const void* X, int B, int H, int W, int C, int xpitch, c
     return cudaGetLastError();
 }
 
+cudaError_t pool_mask_bwd(const void* X, int B, int H, int W, int C, int xpitch, const float* dY, float* skip,
+                          int spitch, void* out, cudaStream_t s)
+{
+    const long long Po = (long long)B * (H / 2) * (W / 2);
+    const bool vec = C % 8 == 0 && C / 8 <= 256 && xpitch % 8 == 0 && spitch % 4 == 0 &&
+                     (((uintptr_t)X | (uintptr_t)dY | (uintptr_t)skip | (uintptr_t)out) & 15) == 0;
+    if (!vec) {
+        const cudaError_t e = maxpool_bwd(X, B, H, W, C, xpitch, dY, skip, spitch, s);
+        return e != cudaSuccess ? e : mask_cast(skip, spitch, X, xpitch, (long long)B * H * W, C, out, C, s);
+    }
+    const dim3 b(C / 8, 256 / (C / 8));
+    k_pool_mask_bwd8<<<(unsigned)((Po + b.y - 1) / b.y), b, 0, s>>>((const bf16*)X, B, H, W, C, xpitch, dY, skip, spitch,
+                                                                    (bf16*)out);
+    return cudaGetLastError();
+}
+
 cudaError_t shuffle_fwd(const void* U, int B, int H, int W, int C, void* Y, int ypitch, int c0, cudaStream_t s)
 {
     k_shuffle_fwd<<<blocks((long long)B * H * W * 4 * C), 256, 0, s>>>((const bf16*)U, B, H, W, C, (bf16*)Y, ypitch,
@@ -1028,8 +1160,11 @@ cudaError_t proj_fwd(const void* X, int P, int C, int xpitch, const float* Wt, c
 }
 
 cudaError_t proj_bwd(const float* dY, const void* X, int P, int C, int xpitch, const float* Wt, int O, float* dX,
-                     int dpitch, float* dW, float* db, float* part, int part_blocks, cudaStream_t s)
+                     int dpitch, float* dW, float* db, float* part, int part_blocks, cudaStream_t s, void* dXb)
 {
+    const bool vec = (C == 8 || C == 16 || C == 32 || C == 64) && O >= 1 && O <= 8 && xpitch % 8 == 0 &&
+                     (((uintptr_t)X | (uintptr_t)dXb) & 15) == 0;
+    if (dXb && vec) dX = nullptr;  // formed, masked and rounded with the weight partials
     if (dX) {
         const bool vec = C % 4 == 0 && C / 4 <= 256 && dpitch % 4 == 0 &&
                          (((uintptr_t)dX | (uintptr_t)Wt) & 15) == 0;
@@ -1042,12 +1177,10 @@ cudaError_t proj_bwd(const float* dY, const void* X, int P, int C, int xpitch, c
     }
     const int chunk = (P + part_blocks - 1) / part_blocks;
     const int nb = (P + chunk - 1) / chunk;
-    const bool vec = (C == 8 || C == 16 || C == 32 || C == 64) && O >= 1 && O <= 8 && xpitch % 8 == 0 &&
-                     ((uintptr_t)X & 15) == 0;
     if (vec) {
         switch (O) {
 #define NN_PROJ_W8(OV) \
-    case OV: k_proj_bwd_w8<OV><<<nb, 256, 0, s>>>(dY, (const bf16*)X, P, C, xpitch, chunk, part); break;
+    case OV: k_proj_bwd_w8<OV><<<nb, 256, 0, s>>>(dY, (const bf16*)X, P, C, xpitch, chunk, part, Wt, (bf16*)dXb); break;
             NN_PROJ_W8(1)
             NN_PROJ_W8(2)
             NN_PROJ_W8(3)
@@ -1065,6 +1198,7 @@ cudaError_t proj_bwd(const float* dY, const void* X, int P, int C, int xpitch, c
     }
     const int slots = O * (C + 1);
     k_proj_sum<<<(unsigned)((slots + 7) / 8), 256, 0, s>>>(part, nb, O, C, dW, db);
+    if (dXb && !vec) return mask_cast(dX, dpitch, X, xpitch, P, C, dXb, C, s);
     return cudaGetLastError();
 }
 
@@ -1118,7 +1252,7 @@ cudaError_t pad_conv3x3(const void* W, int cout, int cin, int cin_pad, void* Wp,
 cudaError_t flip3x3_many(const FlipJob* jobs, int njobs, long long total, cudaStream_t s)
 {
     if (njobs < 1 || total < 1) return cudaSuccess;
-    k_flip3x3_many<<<blocks(total), 256, 0, s>>>(jobs, njobs, total);
+    k_flip3x3_many<<<(unsigned)total, dim3(32, 8), 0, s>>>(jobs, njobs);
     return cudaGetLastError();
 }
 
@@ -1164,7 +1298,11 @@ cudaError_t adam(float* w, const float* g, float* m, float* v, long long n, floa
                  int t, void* wb, cudaStream_t s)
 {
     const float c1 = 1.0f - powf(b1, (float)t), c2 = 1.0f - powf(b2, (float)t);
-    k_adam<<<blocks(n), 256, 0, s>>>(w, g, m, v, n, lr, b1, b2, eps, c1, c2, (bf16*)wb);
+    if (n % 4 == 0 && (((uintptr_t)w | (uintptr_t)g | (uintptr_t)m | (uintptr_t)v | (uintptr_t)wb) & 15) == 0)
+        k_adam4<<<blocks(n / 4), 256, 0, s>>>((float4*)w, (const float4*)g, (float4*)m, (float4*)v, n / 4, lr, b1, b2,
+                                              eps, c1, c2, (uint2*)wb);
+    else
+        k_adam<<<blocks(n), 256, 0, s>>>(w, g, m, v, n, lr, b1, b2, eps, c1, c2, (bf16*)wb);
     return cudaGetLastError();
 }
 

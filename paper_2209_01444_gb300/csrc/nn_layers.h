@@ -13,16 +13,22 @@ cudaError_t transpose(const void* in, int rows, int cols, int ipitch, void* out,
 cudaError_t maxpool_fwd(const void* X, int B, int H, int W, int C, int xpitch, void* Y, cudaStream_t s);
 cudaError_t maxpool_bwd(const void* X, int B, int H, int W, int C, int xpitch, const float* dY, float* dX, int dpitch,
                         cudaStream_t s);
+// out (BF16 [P][C]) = the sum of skip (FP32, pitch spitch; clobbered where a
+// shape needs two passes) and the max-pool gradient dY, masked by X > 0.
+cudaError_t pool_mask_bwd(const void* X, int B, int H, int W, int C, int xpitch, const float* dY, float* skip,
+                          int spitch, void* out, cudaStream_t s);
 cudaError_t shuffle_fwd(const void* U, int B, int H, int W, int C, void* Y, int ypitch, int c0, cudaStream_t s);
 cudaError_t shuffle_bwd(const void* dY, bool dy_fp32, int ypitch, int c0, int B, int H, int W, int C, void* dU,
                         cudaStream_t s);
 cudaError_t proj_fwd(const void* X, int P, int C, int xpitch, const float* Wt, const float* bias, int O,
                      const float* R, float* Y, cudaStream_t s);
 cudaError_t proj_bwd(const float* dY, const void* X, int P, int C, int xpitch, const float* Wt, int O, float* dX,
-                     int dpitch, float* dW, float* db, float* part, int part_blocks, cudaStream_t s);
+                     int dpitch, float* dW, float* db, float* part, int part_blocks, cudaStream_t s,
+                     void* dXb = nullptr);  // dXb: BF16 [P][C], dX masked by X > 0 (dX is then scratch)
 cudaError_t flip3x3(const void* W, int cout, int cin, void* Wf, cudaStream_t s);
 // Several flips in one launch: job j flips the kernel at W (cout x 9 cin) into
-// Wf, its elements numbered from start (jobs in order of start; device table).
+// Wf, its 9 ceil(cout / 32) ceil(cin / 32) tiles numbered from start (jobs in
+// order of start; device table); total: the number of tiles.
 struct FlipJob {
     const void* W;
     void* Wf;

@@ -68,7 +68,8 @@ struct Level {
     bf16* pool = nullptr;  // [P/4][c]
     bf16* dA = nullptr;    // decoder activations [P][c]
     bf16* dD = nullptr;
-    float* dcat = nullptr;  // gradient of cat_l, FP32 [P][2c]
+    float* dcat = nullptr;  // gradient of cat_l, FP32 [P][dpitch]
+    int dpitch = 0;         // 2c, or c where only its first half is kept (conv3x3_split)
 };
 
 struct Tensor {
@@ -297,7 +298,7 @@ cudaError_t allocate(lbm_unet* u)
         for (Conv* cv : {&v.ea, &v.eb, &v.da, &v.db})
             if (cv->cout) {
                 jobs.push_back({u->wb + cv->w, cv->wf, cv->cout, cv->cin, total});
-                total += 9LL * cv->cout * cv->cin;
+                total += 9LL * ((cv->cout + 31) / 32) * ((cv->cin + 31) / 32);
             }
     nn::FlipJob* table = nullptr;
     UN_ALLOC(table, (long long)jobs.size());
@@ -331,7 +332,10 @@ cudaError_t allocate_backward(lbm_unet* u)
         Level& v = u->lv[l];
         const long long P = v.P;
         const int c = v.c;
-        if (l < L - 1) UN_ALLOC(v.dcat, P * 2 * c);
+        if (l < L - 1) {
+            v.dpitch = nn::conv3x3_split_supported(u->B, v.H, v.W, c) ? c : 2 * c;
+            UN_ALLOC(v.dcat, P * v.dpitch);
+        }
         for (Conv* cv : {&v.ea, &v.eb, &v.da, &v.db}) {
             if (!cv->cout) continue;
             if (!nn::conv3x3_supported(u->B, v.H, v.W, cv->cout)) col_n = std::max(col_n, 9 * P * cv->cout);
@@ -505,18 +509,24 @@ cudaError_t backward(lbm_unet* u, const float* x, const float* t)
         return e;
     const bf16* top = L > 1 ? u->lv[0].dD : u->lv[0].s;
     if ((e = nn::proj_bwd(u->G, top, (int)P0, w0, w0, u->w + u->out_w, F, u->g32, w0, u->g + u->out_w, u->g + u->out_b,
-                          u->part, kPartBlocks, u->s)))
+                          u->part, kPartBlocks, u->s, u->gA)))
         return e;
-    if ((e = mask_cast(u, u->g32, w0, top, L > 1 ? w0 : u->lv[0].spitch, P0, w0, u->gA))) return e;
     // decoder, top level first; gA holds the masked gradient of the level's output
     for (int l = 0; l < L - 1; ++l) {
         Level& v = u->lv[l];
         const Level& lo = u->lv[l + 1];
         const int c = v.c;
         if ((e = conv_bwd(u, v, v.db, v.dA, c, u->gA, u->g32, c, u->gB))) return e;
-        if ((e = conv_bwd(u, v, v.da, v.s, 2 * c, u->gB, v.dcat, 2 * c))) return e;
-        // up-convolution: gradient of u_l is the second half of dcat
-        if ((e = nn::shuffle_bwd(v.dcat, true, 2 * c, c, u->B, lo.H, lo.W, c, u->dU, u->s))) return e;
+        // input gradient of the first decoder convolution: the skip connection's
+        // half stays FP32 (dcat), the up-convolution's goes, rounded, to the
+        // layout of that convolution's output (dU)
+        if (v.dpitch == c) {
+            if ((e = conv_bwd(u, v, v.da, v.s, 2 * c, u->gB, nullptr, 0))) return e;
+            if ((e = nn::conv3x3_split(u->gB, u->B, v.H, v.W, c, v.da.wf, v.dcat, u->dU, u->s))) return e;
+        } else {
+            if ((e = conv_bwd(u, v, v.da, v.s, 2 * c, u->gB, v.dcat, 2 * c))) return e;
+            if ((e = nn::shuffle_bwd(v.dcat, true, 2 * c, c, u->B, lo.H, lo.W, c, u->dU, u->s))) return e;
+        }
         if ((e = nn::colsum(u->dU, false, lo.P, 4 * c, 4 * c, u->g + v.up.b, u->part, kPartBlocks, u->s))) return e;
         const bf16* hlow = (l + 1 < L - 1) ? lo.dD : lo.s;
         if ((e = nn::gatherT(u->dU, u->B, lo.H, lo.W, 4 * c, 4 * c, 1, u->tA, lo.P, u->s))) return e;
@@ -536,9 +546,8 @@ cudaError_t backward(lbm_unet* u, const float* x, const float* t)
         Level& v = u->lv[l];
         const int c = v.c;
         if (l < L - 1) {
-            // skip gradient (first half of dcat) plus the pooled path's gradient in g32
-            if ((e = nn::maxpool_bwd(v.s, u->B, v.H, v.W, c, 2 * c, u->g32, v.dcat, 2 * c, u->s))) return e;
-            if ((e = mask_cast(u, v.dcat, 2 * c, v.s, 2 * c, v.P, c, u->gA))) return e;
+            // skip gradient (first c columns of dcat) plus the pooled path's gradient in g32
+            if ((e = nn::pool_mask_bwd(v.s, u->B, v.H, v.W, c, 2 * c, u->g32, v.dcat, v.dpitch, u->gA, u->s))) return e;
         }
         if ((e = conv_bwd(u, v, v.eb, v.a, c, u->gA, u->g32, c, u->gB))) return e;
         const bf16* in = l == 0 ? u->x0 : u->lv[l - 1].pool;
