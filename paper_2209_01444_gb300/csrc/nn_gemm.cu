@@ -1181,6 +1181,89 @@ __global__ void k_split_reduce_t_tile(const float* __restrict__ part, int splits
     }
 }
 
+// Every deferred sum of a backward pass in one launch (ReduceJob; a block of 32
+// x 8 threads per start .. next start): one kernel after the other they were 44
+// launches of 4 to 15 us, most of a few blocks.  Each job adds its terms in the
+// order of the kernel named, so the results are the same bits.
+__global__ void __launch_bounds__(256) k_reduce_jobs(const ReduceJob* __restrict__ jobs, int njobs)
+{
+    __shared__ float t[32][33];
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    int lo = 0, hi = njobs - 1;  // the last job whose start is <= blockIdx.x
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (jobs[mid].start <= (int)blockIdx.x)
+            lo = mid;
+        else
+            hi = mid - 1;
+    }
+    const ReduceJob jb = jobs[lo];
+    const int blk = (int)blockIdx.x - jb.start;
+    const float* __restrict__ part = jb.part;
+    const size_t MN = (size_t)jb.M * jb.N;
+    if (jb.kind == kReduceTransposed && jb.splits >= 16 && jb.M <= 65535) {  // k_split_reduce_t_many
+        const int nb = (jb.N + 31) / 32, row = blk / nb, col = blk % nb * 32 + tx;
+        float acc = 0.0f;
+        if (col < jb.N) {
+            const float* p = part + (size_t)row * jb.N + col;
+            for (int z = ty; z < jb.splits; z += 64) {
+                float v[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) v[k] = z + 8 * k < jb.splits ? p[(size_t)(z + 8 * k) * MN] : 0.0f;
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (z + 8 * k < jb.splits) acc += v[k];
+            }
+        }
+        t[ty][tx] = acc;
+        __syncthreads();
+        if (ty == 0 && col < jb.N) {
+            float v = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v += t[k][tx];
+            jb.D[(size_t)col * jb.ldd + row] = v;
+        }
+    } else if (jb.kind == kReduceTransposed) {  // k_split_reduce_t_tile
+        const int nb = (jb.N + 31) / 32, r0 = blk / nb * 32, c0 = blk % nb * 32;
+        float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        for (int z = 0; z < jb.splits; ++z)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int row = r0 + ty + 8 * k, col = c0 + tx;
+                if (row < jb.M && col < jb.N) acc[k] += part[z * MN + (size_t)row * jb.N + col];
+            }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) t[ty + 8 * k][tx] = acc[k];
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int col = c0 + ty + 8 * k, row = r0 + tx;
+            if (row < jb.M && col < jb.N) jb.D[(size_t)col * jb.ldd + row] = t[tx][ty + 8 * k];
+        }
+    } else if (jb.kind == kReducePlain) {  // k_split_reduce
+        const size_t i = (size_t)blk * 256 + ty * 32 + tx;
+        if (i >= MN) return;
+        float acc = 0.0f;
+        for (int z = 0; z < jb.splits; z += 8) {
+            float v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = z + k < jb.splits ? part[(size_t)(z + k) * MN + i] : 0.0f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (z + k < jb.splits) acc += v[k];
+        }
+        jb.D[i / jb.N * jb.ldd + i % jb.N] = acc;
+    } else {  // kReduceColumns: k_sum_parts, a warp per column
+        const int c = blk * 8 + ty;
+        if (c >= jb.N) return;
+        float acc = 0.0f;
+        for (int b = tx; b < jb.splits; b += 32) acc += part[(size_t)b * jb.N + c];
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d);
+        if (tx == 0) jb.D[c] = acc;
+    }
+}
+
 // D[col][row] (pitch ldd) = the sum of the slices' partial tiles.
 cudaError_t launch_split_reduce_t(const float* part, int splits, int M, int N, float* D, int ldd, cudaStream_t s)
 {
@@ -1210,18 +1293,40 @@ cudaError_t launch_wgrad(const void* X, int B, int W, int C, int cpitch, const v
 
 }  // namespace
 
+int reduce_job_blocks(const ReduceJob& j)
+{
+    const int nb = (j.N + 31) / 32;
+    if (j.kind == kReduceTransposed) return nb * (j.splits >= 16 && j.M <= 65535 ? j.M : (j.M + 31) / 32);
+    if (j.kind == kReducePlain) return (int)(((long long)j.M * j.N + 255) / 256);
+    return (j.N + 7) / 8;
+}
+
+cudaError_t reduce_jobs(const ReduceJob* jobs, int njobs, int blocks, cudaStream_t s)
+{
+    if (njobs < 1) return cudaSuccess;
+    k_reduce_jobs<<<blocks, dim3(32, 8), 0, s>>>(jobs, njobs);
+    return cudaGetLastError();
+}
+
 bool wgrad_direct_supported(int W, int C, int cpitch, int N)
 {
     return W >= 32 && W % 32 == 0 && C >= 32 && C % 32 == 0 && cpitch % 8 == 0 && C <= cpitch && N >= 8 && N % 8 == 0;
 }
 
+// Slices of `units` K blocks: at most `splits`, of equal length but the last.
+static int even_slices(int units, int splits, int* per)
+{
+    if (splits < 1) splits = 1;
+    if (splits > units) splits = units;
+    *per = (units + splits - 1) / splits;
+    return (units + *per - 1) / *per;
+}
+
 cudaError_t wgrad_direct(const void* X, int B, int H, int W, int C, int cpitch, int cin, const void* dY, int N,
-                         float* dW, int ldd, cudaStream_t s, int splits, float* workspace)
+                         cudaStream_t s, int splits, float* part, int* slices)
 {
     const long long P = (long long)B * H * W;
-    if (!wgrad_direct_supported(W, C, cpitch, N) || cin < 1 || cin > C || 9 * cin > ldd || !workspace || P > 0x7fffffffLL)
-        return cudaErrorInvalidValue;
-    if (((uintptr_t)X | (uintptr_t)dY | (uintptr_t)workspace) & 15) return cudaErrorInvalidValue;
+    if (!wgrad_direct_supported(W, C, cpitch, N) || cin < 1 || cin > C || P > 0x7fffffffLL) return cudaErrorInvalidValue;
     WgradGeo g;
     g.cin = cin;
     g.N = N;
@@ -1232,11 +1337,11 @@ cudaError_t wgrad_direct(const void* X, int B, int H, int W, int C, int cpitch, 
     // slices in K blocks of 64 pixels where the rows, or a gathered copy of them
     // (cin < C: the padded first layer), are cut so; of 32 otherwise
     const int unit = cin < C ? 64 / g.bk : 1;
-    const int units = (g.blocks + unit - 1) / unit;
-    if (splits < 1) splits = 1;
-    if (splits > units) splits = units;
-    g.per_split = (units + splits - 1) / splits * unit;
-    splits = (g.blocks + g.per_split - 1) / g.per_split;
+    splits = even_slices((g.blocks + unit - 1) / unit, splits, &g.per_split);
+    g.per_split *= unit;
+    *slices = splits;
+    if (!part) return cudaSuccess;
+    if (((uintptr_t)X | (uintptr_t)dY | (uintptr_t)part) & 15) return cudaErrorInvalidValue;
     const bool wc = C % 64 == 0, wn = N % 64 == 0;
     g.ncb = C / (wc ? 64 : 32);
     g.nnb = (N + (wn ? 64 : 32) - 1) / (wn ? 64 : 32);
@@ -1247,9 +1352,38 @@ cudaError_t wgrad_direct(const void* X, int B, int H, int W, int C, int cpitch, 
                                  : (three ? launch_wgrad<64, 32, 3> : launch_wgrad<64, 32, 1>))
                            : (wn ? (three ? launch_wgrad<32, 64, 3> : launch_wgrad<32, 64, 1>)
                                  : (three ? launch_wgrad<32, 32, 3> : launch_wgrad<32, 32, 1>));
-    const cudaError_t e = launch(X, B, W, C, cpitch, dY, g, splits, workspace, s);
+    return launch(X, B, W, C, cpitch, dY, g, splits, part, s);
+}
+
+template <int BN>
+static cudaError_t launch_tn(const void* A, const void* B, int M, int N, int P, int splits, int per, float* part,
+                             cudaStream_t s)
+{
+    constexpr int smem = tn_stages<BN>() * tn_stage<BN>() + 1024 + 256;
+    cudaError_t e = cudaFuncSetAttribute(k_gemm_tn<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    return launch_split_reduce_t(workspace, splits, 9 * cin, N, dW, ldd, s);
+    CUtensorMap ta, tb;
+    if ((e = make_map(&ta, A, P, M, M, 64, 64)) != cudaSuccess) return e;
+    if ((e = make_map(&tb, B, P, N, N, 64, BN > 32 ? 64 : 32)) != cudaSuccess) return e;
+    k_gemm_tn<BN><<<dim3((M + kBM - 1) / kBM, (N + BN - 1) / BN, splits), kWsThreads, smem, s>>>(
+        ta, tb, part, M, N, (P + 63) / 64, per);
+    return cudaGetLastError();
+}
+
+cudaError_t gemm_tn(const void* A, const void* B, int M, int N, int P, cudaStream_t s, int splits, float* part,
+                    int* slices)
+{
+    if (M < 8 || M % 8 || N < 8 || N % 8 || P < 1) return cudaErrorInvalidValue;
+    int per = 0;
+    *slices = even_slices((P + 63) / 64, splits, &per);
+    if (!part) return cudaSuccess;
+    if (((uintptr_t)A | (uintptr_t)B | (uintptr_t)part) & 15) return cudaErrorInvalidValue;
+    switch (bn_for(N)) {
+    case 256: return launch_tn<256>(A, B, M, N, P, *slices, per, part, s);
+    case 128: return launch_tn<128>(A, B, M, N, P, *slices, per, part, s);
+    case 64: return launch_tn<64>(A, B, M, N, P, *slices, per, part, s);
+    default: return launch_tn<32>(A, B, M, N, P, *slices, per, part, s);
+    }
 }
 
 cudaError_t gemm_bf16_tout(const void* A, int lda, const void* B, int ldb, float* D, int ldd, int M, int N, int K,

@@ -60,15 +60,32 @@ bool wgrad3_supported(int B, int H, int W, int C, int cout);
 cudaError_t wgrad3_bf16(const void* XT3, const void* dYT, int B, int H, int W, int C, int cout, float* D, int ldd,
                         cudaStream_t s, int splits, float* workspace);
 
-// Weight gradient dW[N][9 cin] (pitch ldd) of a 3 x 3 zero-padded convolution
-// from its NHWC BF16 input X (C channels, pitch cpitch, of which the first cin
-// are the layer's: the others carry zeros) and output gradient dY [B H W][N];
-// W and C multiples of 32, N of 8.  The pixels are summed in `splits` slices
-// (workspace: splits x 9 cin x N floats), as wgrad3_bf16 and, for cin < C, the
-// GEMM over nine gathered taps sum them.
+// A sum left for reduce_jobs: D from the `splits` partial arrays at part.
+// kReduceTransposed: M x N tiles, D[n][m] (pitch ldd); kReducePlain: D[m][n];
+// kReduceColumns: rows of N column sums, D[n].  start: the job's first block
+// (jobs in order; reduce_job_blocks of each).
+enum ReduceKind { kReduceTransposed, kReducePlain, kReduceColumns };
+struct ReduceJob {
+    const float* part;
+    float* D;
+    int kind, splits, M, N, ldd, start;
+};
+int reduce_job_blocks(const ReduceJob& j);
+cudaError_t reduce_jobs(const ReduceJob* device_jobs, int njobs, int blocks, cudaStream_t s);
+
+// Partial weight gradients, part[slice][9 cin][N] FP32, of a 3 x 3 zero-padded
+// convolution from its NHWC BF16 input X (C channels, pitch cpitch, of which the
+// first cin are the layer's: the others carry zeros) and output gradient dY
+// [B H W][N]; W and C multiples of 32, N of 8.  The pixels are cut into at most
+// `splits` slices, as wgrad3_bf16 and, for cin < C, the GEMM over nine gathered
+// taps cut them; *slices receives their number.  part null: only that.
 bool wgrad_direct_supported(int W, int C, int cpitch, int N);
 cudaError_t wgrad_direct(const void* X, int B, int H, int W, int C, int cpitch, int cin, const void* dY, int N,
-                         float* dW, int ldd, cudaStream_t s, int splits, float* workspace);
+                         cudaStream_t s, int splits, float* part, int* slices);
+// part[slice][M][N] = A^T B over the slice's pixels, A [P][M] and B [P][N] BF16;
+// slices as gemm_bf16 over their transposes.
+cudaError_t gemm_tn(const void* A, const void* B, int M, int N, int P, cudaStream_t s, int splits, float* part,
+                    int* slices);
 
 // Read (and optionally clear) the flag a GEMM raises when a bounded wait ran out.
 cudaError_t gemm_error(int* flag, bool clear);

@@ -276,11 +276,10 @@ __global__ void k_maxpool_fwd8(const bf16* __restrict__ X, int B, int H, int W, 
                                bf16* __restrict__ Y)
 {
     const int Ho = H / 2, Wo = W / 2, G = C / 8;
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= (long long)B * Ho * Wo * G) return;
-    const int g = (int)(i % G);
-    const long long p = i / G;
-    const int x = (int)(p % Wo), y = (int)((p / Wo) % Ho), b = (int)(p / ((long long)Wo * Ho));
+    const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;  // fewer than 2^31 groups
+    if (i >= (unsigned)B * Ho * Wo * G) return;
+    const unsigned p = i / G;
+    const int g = i - p * G, row = p / Wo, x = p - row * Wo, b = row / Ho, y = row - b * Ho;
     const bf16* base = X + (((long long)b * H + 2 * y) * W + 2 * x) * xpitch + g * 8;
     const uint4 q[4] = {*(const uint4*)base, *(const uint4*)(base + xpitch), *(const uint4*)(base + (long long)W * xpitch),
                         *(const uint4*)(base + (long long)W * xpitch + xpitch)};
@@ -296,7 +295,7 @@ __global__ void k_maxpool_fwd8(const bf16* __restrict__ X, int B, int H, int W, 
         }
         r[j] = __floats2bfloat162_rn(m.x, m.y);
     }
-    *(uint4*)(Y + p * C + g * 8) = *(const uint4*)r;
+    *(uint4*)(Y + (size_t)p * C + g * 8) = *(const uint4*)r;
 }
 
 // The gradient goes to the first maximum of each 2 x 2 window (row-major order).
@@ -389,11 +388,9 @@ __global__ void k_pool_mask_bwd8(const bf16* __restrict__ X, int B, int H, int W
 {
     const int Ho = H / 2, Wo = W / 2;
     const int c = 8 * threadIdx.x;
-    const long long p = (long long)blockIdx.x * blockDim.y + threadIdx.y;
-    if (p >= (long long)B * Ho * Wo) return;
-    const int x = (int)(p % Wo);
-    const long long r = p / Wo;
-    const int y = (int)(r % Ho), b = (int)(r / Ho);
+    const unsigned p = blockIdx.x * blockDim.y + threadIdx.y;  // fewer than 2^31 pixels
+    if (p >= (unsigned)B * Ho * Wo) return;
+    const int r = p / Wo, x = p - r * Wo, b = r / Ho, y = r - b * Ho;
     float v[4][8];
     long long off[4];
     float4 sk[4][2];
@@ -410,7 +407,7 @@ __global__ void k_pool_mask_bwd8(const bf16* __restrict__ X, int B, int H, int W
         sk[k][0] = *(const float4*)(skip + off[k] * spitch + c);
         sk[k][1] = *(const float4*)(skip + off[k] * spitch + c + 4);
     }
-    const float4 g0 = *(const float4*)(dY + p * C + c), g1 = *(const float4*)(dY + p * C + c + 4);
+    const float4 g0 = *(const float4*)(dY + (size_t)p * C + c), g1 = *(const float4*)(dY + (size_t)p * C + c + 4);
     const float g[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
     int arg[8];
 #pragma unroll
@@ -664,31 +661,45 @@ __global__ void __launch_bounds__(256) k_proj_bwd_w8(const float* __restrict__ d
     for (int o = 0; o < O; ++o)
 #pragma unroll
         for (int k = 0; k < 9; ++k) acc[o][k] = 0.0f;
-    for (int p = p0 + pl; p < p1; p += lanes) {
-        const uint4 v = *(const uint4*)(X + (long long)p * xpitch + 8 * cg);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-        float x[8];
+    // four pixels' loads in flight; their products are added in pixel order
+    for (int pb = p0 + pl; pb < p1; pb += 4 * lanes) {
+        uint4 v4[4];
+        float d4[4][O];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            x[2 * k] = __uint_as_float(w[k] << 16);
-            x[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
+        for (int j = 0; j < 4; ++j) {
+            const int p = min(pb + j * lanes, p1 - 1);
+            v4[j] = *(const uint4*)(X + (long long)p * xpitch + 8 * cg);
+#pragma unroll
+            for (int o = 0; o < O; ++o) d4[j][o] = dY[(long long)p * O + o];
         }
-        float dx[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int o = 0; o < O; ++o) {
-            const float d = dY[(long long)p * O + o];
+        for (int j = 0; j < 4; ++j) {
+            const int p = pb + j * lanes;
+            if (p >= p1) break;
+            const uint32_t w[4] = {v4[j].x, v4[j].y, v4[j].z, v4[j].w};
+            float x[8];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) acc[o][k] += d * x[k];
-            acc[o][8] += d;
-            if (dXb)
+            for (int k = 0; k < 4; ++k) {
+                x[2 * k] = __uint_as_float(w[k] << 16);
+                x[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
+            }
+            float dx[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int k = 0; k < 8; ++k) dx[k] += d * wsh[o * C + 8 * cg + k];
-        }
-        if (dXb) {
-            __align__(16) bf16 b[8];
+            for (int o = 0; o < O; ++o) {
+                const float d = d4[j][o];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) b[k] = __float2bfloat16(x[k] > 0.0f ? dx[k] : 0.0f);
-            *(uint4*)(dXb + (long long)p * C + 8 * cg) = *(const uint4*)b;
+                for (int k = 0; k < 8; ++k) acc[o][k] += d * x[k];
+                acc[o][8] += d;
+                if (dXb)
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) dx[k] += d * wsh[o * C + 8 * cg + k];
+            }
+            if (dXb) {
+                __align__(16) bf16 b[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) b[k] = __float2bfloat16(x[k] > 0.0f ? dx[k] : 0.0f);
+                *(uint4*)(dXb + (long long)p * C + 8 * cg) = *(const uint4*)b;
+            }
         }
     }
     // lanes with the same group differ in the bits above log2(G)
@@ -814,14 +825,22 @@ __global__ void k_colsum_part8(const bf16* __restrict__ g, long long rows, int C
     const long long r0 = (long long)blockIdx.x * chunk;
     const long long r1 = r0 + chunk < rows ? r0 + chunk : rows;
     float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    // eight rows' loads in flight; their values are added in row order
     if (rl < lanes)
-        for (long long r = r0 + rl; r < r1; r += lanes) {
-            const uint4 v = *(const uint4*)(g + r * pitch + 8 * cg);
-            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        for (long long r = r0 + rl; r < r1; r += 8 * lanes) {
+            uint4 v[8];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                acc[2 * k] += __uint_as_float(w[k] << 16);
-                acc[2 * k + 1] += __uint_as_float(w[k] & 0xffff0000u);
+            for (int j = 0; j < 8; ++j)
+                v[j] = r + j * lanes < r1 ? *(const uint4*)(g + (r + j * lanes) * pitch + 8 * cg) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (r + j * lanes >= r1) break;
+                const uint32_t w[4] = {v[j].x, v[j].y, v[j].z, v[j].w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    acc[2 * k] += __uint_as_float(w[k] << 16);
+                    acc[2 * k + 1] += __uint_as_float(w[k] & 0xffff0000u);
+                }
             }
         }
 #pragma unroll
@@ -1077,7 +1096,8 @@ cudaError_t transpose(const void* in, int rows, int cols, int ipitch, void* out,
 cudaError_t maxpool_fwd(const void* X, int B, int H, int W, int C, int xpitch, void* Y, cudaStream_t s)
 {
     if (H % 2 || W % 2) return cudaErrorInvalidValue;
-    if (C % 8 == 0 && xpitch % 8 == 0 && (((uintptr_t)X | (uintptr_t)Y) & 15) == 0)
+    if (C % 8 == 0 && xpitch % 8 == 0 && (((uintptr_t)X | (uintptr_t)Y) & 15) == 0 &&
+        (long long)B * (H / 2) * (W / 2) * (C / 8) < 0x7fffffffLL - 256)
         k_maxpool_fwd8<<<blocks((long long)B * (H / 2) * (W / 2) * (C / 8)), 256, 0, s>>>((const bf16*)X, B, H, W, C,
                                                                                         xpitch, (bf16*)Y);
     else
@@ -1106,7 +1126,7 @@ cudaError_t pool_mask_bwd(const void* X, int B, int H, int W, int C, int xpitch,
                           int spitch, void* out, cudaStream_t s)
 {
     const long long Po = (long long)B * (H / 2) * (W / 2);
-    const bool vec = C % 8 == 0 && C / 8 <= 256 && xpitch % 8 == 0 && spitch % 4 == 0 &&
+    const bool vec = C % 8 == 0 && C / 8 <= 256 && xpitch % 8 == 0 && spitch % 4 == 0 && Po < 0x7fffffffLL - 256 &&
                      (((uintptr_t)X | (uintptr_t)dY | (uintptr_t)skip | (uintptr_t)out) & 15) == 0;
     if (!vec) {
         const cudaError_t e = maxpool_bwd(X, B, H, W, C, xpitch, dY, skip, spitch, s);
@@ -1265,6 +1285,16 @@ cudaError_t flip3x3(const void* W, int cout, int cin, void* Wf, cudaStream_t s)
 cudaError_t colsum(const void* g, bool g_fp32, long long rows, int C, int pitch, float* out, float* part,
                    int part_blocks, cudaStream_t s)
 {
+    int nb = 0;
+    const cudaError_t e = colsum_part(g, g_fp32, rows, C, pitch, part, part_blocks, &nb, s);
+    if (e != cudaSuccess) return e;
+    k_sum_parts<<<(unsigned)((C + 7) / 8), 256, 0, s>>>(part, nb, C, out);
+    return cudaGetLastError();
+}
+
+cudaError_t colsum_part(const void* g, bool g_fp32, long long rows, int C, int pitch, float* part, int part_blocks,
+                        int* nblocks, cudaStream_t s)
+{
     if (rows < 1 || C < 1 || part_blocks < 1) return cudaErrorInvalidValue;
     // at most part_blocks partial rows; a block's rows are split among its
     // row lanes, and a block takes about 32 rows per lane (fewer, longer blocks
@@ -1275,13 +1305,14 @@ cudaError_t colsum(const void* g, bool g_fp32, long long rows, int C, int pitch,
     long long chunk = (rows + part_blocks - 1) / part_blocks;
     if (chunk < 32 * lanes) chunk = 32 * lanes;
     const int nb = (int)((rows + chunk - 1) / chunk);
+    *nblocks = nb;
+    if (!part) return cudaSuccess;
     if (g_fp32)
         k_colsum_part<float><<<nb, 128, 0, s>>>((const float*)g, rows, C, pitch, (int)chunk, part);
     else if (vec)
         k_colsum_part8<<<nb, 128, 0, s>>>((const bf16*)g, rows, C, pitch, (int)chunk, part);
     else
         k_colsum_part<bf16><<<nb, 128, 0, s>>>((const bf16*)g, rows, C, pitch, (int)chunk, part);
-    k_sum_parts<<<(unsigned)((C + 7) / 8), 256, 0, s>>>(part, nb, C, out);
     return cudaGetLastError();
 }
 

@@ -43,6 +43,10 @@ cudaError_t mask_cast(const float* g, int gpitch, const void* y, int ypitch, lon
 cudaError_t pad_conv3x3(const void* W, int cout, int cin, int cin_pad, void* Wp, cudaStream_t s);
 cudaError_t colsum(const void* g, bool g_fp32, long long rows, int C, int pitch, float* out, float* part,
                    int part_blocks, cudaStream_t s);
+// Its partial sums alone, [*nblocks][C] at part (null: only their number); the
+// columns are then added over the blocks in k_sum_parts' order.
+cudaError_t colsum_part(const void* g, bool g_fp32, long long rows, int C, int pitch, float* part, int part_blocks,
+                        int* nblocks, cudaStream_t s);
 // Mean of w (pred - target)^2 over n elements and its gradient; with x (the
 // network input, F fields per pixel, phase field first) each pixel's
 // elements are weighted by w = 1 + alpha max(0, 1 - phi^2), else w = 1.

@@ -49,12 +49,15 @@ struct Conv {
     bf16* wpad = nullptr;    // [cout][9 cin_pad] kernel with zero channels (first convolution only)
     int cin_pad = 0;
     bool first = false;  // reads the network's input, stored up to kX0Pitch channels
+    float* wpart = nullptr;  // partial weight gradients, summed at the end of a backward pass (null: at once)
+    float* bpart = nullptr;  // partial bias gradients
 };
 
 struct Up {
     int cin = 0, cout = 0;  // cin = 2 cout
     long long w = 0, b = 0;
     bf16* wt = nullptr;  // [cin][4 cout] transpose for the input gradient
+    float *wpart = nullptr, *bpart = nullptr;  // as in Conv
 };
 
 struct Level {
@@ -96,7 +99,7 @@ struct lbm_unet {
     bf16* x0 = nullptr;
     float *Y = nullptr, *T = nullptr, *G = nullptr;
     float *loss = nullptr, *part = nullptr;
-    bf16 *col = nullptr, *colT = nullptr, *tA = nullptr, *tB = nullptr;
+    bf16 *col = nullptr, *colT = nullptr, *tA = nullptr;
     bf16 *gA = nullptr, *gB = nullptr, *dU = nullptr;
     long long col_n = 0;
     float* g32 = nullptr;
@@ -105,6 +108,8 @@ struct lbm_unet {
     nn::FlipJob* flip_jobs = nullptr;  // device table of the kernel flips (derive)
     int n_flip = 0;
     long long flip_total = 0;
+    nn::ReduceJob* red_jobs = nullptr;  // device table of the sums that end a backward pass
+    int n_red = 0, red_blocks = 0;
     cudaStream_t s = nullptr;
     std::vector<void*> allocs;
     long long bytes = 0;
@@ -324,10 +329,17 @@ cudaError_t allocate_backward(lbm_unet* u)
         if ((e = alloc(u, &(p), (n)))) return e; \
     } while (0)
     // col: gathered copy of an output gradient whose input gradient the implicit
-    // convolution lacks; colT, tA: transposed copies where the weight gradient
-    // needs them (tA, tB: the up-convolutions')
-    long long col_n = 1, colT_n = 1, ws_n = 0, t_n = 1, g_n = u->P0 * u->base;
+    // convolution lacks; colT, tA, ws: transposed copies and partial sums where
+    // the weight gradient needs them
+    long long col_n = 1, colT_n = 1, ws_n = 1, t_n = 1, g_n = u->P0 * u->base;
     const int L = u->L;
+    std::vector<nn::ReduceJob> jobs;
+    auto defer = [&](nn::ReduceJob j) {
+        j.start = u->red_blocks;
+        jobs.push_back(j);
+        u->red_blocks += nn::reduce_job_blocks(j);
+    };
+    u->red_blocks = 0;
     for (int l = 0; l < L; ++l) {
         Level& v = u->lv[l];
         const long long P = v.P;
@@ -336,20 +348,36 @@ cudaError_t allocate_backward(lbm_unet* u)
             v.dpitch = nn::conv3x3_split_supported(u->B, v.H, v.W, c) ? c : 2 * c;
             UN_ALLOC(v.dcat, P * v.dpitch);
         }
+        int n = 0;
         for (Conv* cv : {&v.ea, &v.eb, &v.da, &v.db}) {
             if (!cv->cout) continue;
-            if (!nn::conv3x3_supported(u->B, v.H, v.W, cv->cout)) col_n = std::max(col_n, 9 * P * cv->cout);
-            ws_n = std::max(ws_n, split_ws(9 * cv->cin, cv->cout, P));
-            if (!nn::wgrad_direct_supported(v.W, wgrad_channels(*cv), wgrad_channels(*cv), cv->cout)) {
-                colT_n = std::max(colT_n, 9 * P * cv->cin);
-                t_n = std::max(t_n, P * cv->cout);
+            const int K9 = 9 * cv->cin, N = cv->cout, C = wgrad_channels(*cv);
+            if (!nn::conv3x3_supported(u->B, v.H, v.W, N)) col_n = std::max(col_n, 9 * P * N);
+            if (nn::wgrad_direct_supported(v.W, C, cv->first ? kX0Pitch : cv->cin, N)) {
+                if ((e = nn::wgrad_direct(nullptr, u->B, v.H, v.W, C, C, cv->cin, nullptr, N, u->s,
+                                          splits_for(K9, N, P), nullptr, &n)))
+                    return e;
+                UN_ALLOC(cv->wpart, (long long)n * K9 * N);
+                defer({cv->wpart, u->g + cv->w, nn::kReduceTransposed, n, K9, N, K9, 0});
+            } else {
+                colT_n = std::max(colT_n, P * K9);
+                t_n = std::max(t_n, P * N);
+                ws_n = std::max(ws_n, split_ws(K9, N, P));
             }
+            if ((e = nn::colsum_part(nullptr, false, P, N, N, nullptr, kPartBlocks, &n, u->s))) return e;
+            UN_ALLOC(cv->bpart, (long long)n * N);
+            defer({cv->bpart, u->g + cv->b, nn::kReduceColumns, n, 1, N, N, 0});
             g_n = std::max(g_n, P * std::max(cv->cout, cv->cin));
         }
         if (v.up.cout) {
             const long long Pl = P / 4;
-            ws_n = std::max(ws_n, split_ws(4 * c, 2 * c, Pl));
-            t_n = std::max(t_n, Pl * 4 * c);
+            if ((e = nn::gemm_tn(nullptr, nullptr, 4 * c, 2 * c, (int)Pl, u->s, splits_for(4 * c, 2 * c, Pl), nullptr, &n)))
+                return e;
+            UN_ALLOC(v.up.wpart, (long long)n * 4 * c * 2 * c);
+            defer({v.up.wpart, u->g + v.up.w, nn::kReducePlain, n, 4 * c, 2 * c, 2 * c, 0});
+            if ((e = nn::colsum_part(nullptr, false, Pl, 4 * c, 4 * c, nullptr, kPartBlocks, &n, u->s))) return e;
+            UN_ALLOC(v.up.bpart, (long long)n * 4 * c);
+            defer({v.up.bpart, u->g + v.up.b, nn::kReduceColumns, n, 1, 4 * c, 4 * c, 0});
             g_n = std::max(g_n, Pl * 4 * c);
         }
     }
@@ -361,12 +389,16 @@ cudaError_t allocate_backward(lbm_unet* u)
     }
     UN_ALLOC(u->colT, colT_n);
     UN_ALLOC(u->tA, t_n);
-    UN_ALLOC(u->tB, t_n);
     UN_ALLOC(u->gA, g_n);
     UN_ALLOC(u->gB, g_n);
     UN_ALLOC(u->dU, g_n);
     UN_ALLOC(u->g32, g_n);
-    UN_ALLOC(u->ws, ws_n);
+    nn::ReduceJob* table = nullptr;
+    UN_ALLOC(table, (long long)jobs.size());
+    if ((e = cudaMemcpy(table, jobs.data(), jobs.size() * sizeof(nn::ReduceJob), cudaMemcpyHostToDevice))) return e;
+    u->red_jobs = table;
+    u->n_red = (int)jobs.size();
+    UN_ALLOC(u->ws, ws_n);  // last: marks the buffers complete
     u->ws_n = ws_n;
 #undef UN_ALLOC
     return e;
@@ -430,21 +462,22 @@ cudaError_t conv_bwd(lbm_unet* u, const Level& v, const Conv& cv, const bf16* in
     cudaError_t e;
     // dW [cout][9 cin] = dY^T X_taps, computed as its transpose so that the
     // taps and channels fill the MMA's 128 rows and cout (as small as 32) is the N
-    // width; the split-K reduction writes it back as [cout][9 cin].  Where the
+    // width; the sum of the slices writes it back as [cout][9 cin].  Where the
     // shapes allow, straight from X and dY as they are (the first layer's input
     // carries zero channels up to its pitch); otherwise nine transposed taps of
     // X and the transpose of dY are written out for a plain GEMM.
     const int sp = splits_for(K9, cv.cout, P);
     const int C = wgrad_channels(cv);
-    if (nn::wgrad_direct_supported(v.W, C, inpitch, cv.cout)) {
-        e = nn::wgrad_direct(in, u->B, v.H, v.W, C, inpitch, cv.cin, dY, cv.cout, u->g + cv.w, K9, u->s, sp, u->ws);
+    int n = 0;
+    if (cv.wpart) {
+        e = nn::wgrad_direct(in, u->B, v.H, v.W, C, inpitch, cv.cin, dY, cv.cout, u->s, sp, cv.wpart, &n);
     } else {
         if ((e = nn::gatherT(in, u->B, v.H, v.W, cv.cin, inpitch, 9, u->colT, P, u->s))) return e;
         if ((e = nn::gatherT(dY, u->B, v.H, v.W, cv.cout, cv.cout, 1, u->tA, P, u->s))) return e;
         e = nn::gemm_bf16_tout(u->colT, (int)P, u->tA, (int)P, u->g + cv.w, K9, K9, cv.cout, (int)P, u->s, sp, u->ws);
     }
     if (e) return e;
-    if ((e = nn::colsum(dY, false, P, cv.cout, cv.cout, u->g + cv.b, u->part, kPartBlocks, u->s))) return e;
+    if ((e = nn::colsum_part(dY, false, P, cv.cout, cv.cout, cv.bpart, kPartBlocks, &n, u->s))) return e;
     if (!dx) return cudaSuccess;
     if (dxb) {
         e = nn::conv3x3_bf16(dY, u->B, v.H, v.W, cv.cout, cv.cout, cv.wf, 9 * cv.cout, dxb, cv.cin, nullptr, cv.cin,
@@ -527,13 +560,10 @@ cudaError_t backward(lbm_unet* u, const float* x, const float* t)
             if ((e = conv_bwd(u, v, v.da, v.s, 2 * c, u->gB, v.dcat, 2 * c))) return e;
             if ((e = nn::shuffle_bwd(v.dcat, true, 2 * c, c, u->B, lo.H, lo.W, c, u->dU, u->s))) return e;
         }
-        if ((e = nn::colsum(u->dU, false, lo.P, 4 * c, 4 * c, u->g + v.up.b, u->part, kPartBlocks, u->s))) return e;
         const bf16* hlow = (l + 1 < L - 1) ? lo.dD : lo.s;
-        if ((e = nn::gatherT(u->dU, u->B, lo.H, lo.W, 4 * c, 4 * c, 1, u->tA, lo.P, u->s))) return e;
-        if ((e = nn::gatherT(hlow, u->B, lo.H, lo.W, 2 * c, 2 * c, 1, u->tB, lo.P, u->s))) return e;
-        const int sp = splits_for(4 * c, 2 * c, lo.P);
-        if ((e = nn::gemm_bf16(u->tA, (int)lo.P, u->tB, (int)lo.P, u->g + v.up.w, 2 * c, nullptr, 4 * c, 2 * c,
-                               (int)lo.P, false, false, u->s, sp, u->ws)))
+        int n = 0;
+        if ((e = nn::colsum_part(u->dU, false, lo.P, 4 * c, 4 * c, v.up.bpart, kPartBlocks, &n, u->s))) return e;
+        if ((e = nn::gemm_tn(u->dU, hlow, 4 * c, 2 * c, (int)lo.P, u->s, splits_for(4 * c, 2 * c, lo.P), v.up.wpart, &n)))
             return e;
         // gradient of the up-convolution's input, masked by that input (a ReLU
         // output) and rounded to BF16 in the GEMM's epilogue
@@ -554,7 +584,7 @@ cudaError_t backward(lbm_unet* u, const float* x, const float* t)
         const int inpitch = l == 0 ? kX0Pitch : u->lv[l - 1].c;
         if ((e = conv_bwd(u, v, v.ea, in, inpitch, u->gB, l == 0 ? nullptr : u->g32, v.ea.cin))) return e;
     }
-    return cudaSuccess;
+    return nn::reduce_jobs(u->red_jobs, u->n_red, u->red_blocks, u->s);
 }
 
 }  // namespace

@@ -183,26 +183,14 @@ __global__ void __launch_bounds__(kWsThreads, KYS == 1 ? 2 : 1)
             const bool keep = kx < 3 && ci < geo.cin;
             float* row = out + ((size_t)(3 * ky + kx) * geo.cin + ci) * geo.N + nb * BN;
 #pragma unroll 1
-            for (int c = 0; c < BN; c += 16) {
-                uint32_t r[16];
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                    "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                    : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                      "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-                      "=r"(r[15])
-                    : "r"(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * BN + c)));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            for (int c = 0; c < BN; c += 32) {
+                uint32_t r[32];
+                tmem_ld32(r, tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * BN + c));
+                tmem_wait32(r);
                 if (!keep) continue;
 #pragma unroll
-                for (int j = 0; j < 16; j += 8) {
-                    if (nb * BN + c + j >= geo.N) break;  // N is a multiple of 8
-                    float4* d = (float4*)(row + c + j);
-                    d[0] = make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]), __uint_as_float(r[j + 2]),
-                                       __uint_as_float(r[j + 3]));
-                    d[1] = make_float4(__uint_as_float(r[j + 4]), __uint_as_float(r[j + 5]),
-                                       __uint_as_float(r[j + 6]), __uint_as_float(r[j + 7]));
-                }
+                for (int j = 0; j < 32; j += 8)
+                    if (nb * BN + c + j < geo.N) store32(row + c + j, r + j);  // N is a multiple of 8
             }
         }
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -223,4 +211,131 @@ __global__ void __launch_bounds__(kWsThreads, KYS == 1 ? 2 : 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+}
+
+// Split-K GEMM over pixels from operands as they lie in memory: part[z][m][n] =
+// sum over the slice's pixels p of A[p][m] B[p][n] (FP32, M x N), A [P][M] and
+// B [P][N] BF16 contiguous: the up-convolutions' weight gradient without
+// transposed copies.  128 x BN tiles, K blocks of 64 pixels; the slices and their
+// order are those of k_gemm over the transposes, whose partial sums these are
+// bit for bit.
+template <int BN>
+constexpr int tn_stage() { return 64 * (128 + BN) * 2; }
+template <int BN>
+constexpr int tn_stages()
+{
+    constexpr int n = (BN <= 64 ? 100 : 200) * 1024 / tn_stage<BN>();
+    return n > 8 ? 8 : n;
+}
+
+template <int BN>
+__global__ void __launch_bounds__(kWsThreads, BN <= 64 ? 2 : 1)
+    k_gemm_tn(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+              float* __restrict__ part, int M, int N, int blocks, int per_split)
+{
+    constexpr int S = tn_stages<BN>(), STAGE = tn_stage<BN>();
+    constexpr int NB = BN > 64 ? BN / 64 : 1, YB = BN > 32 ? 128 : 64;  // B boxes and bytes of their rows
+    constexpr int ABOX = 64 * 128, BBOX = 64 * YB;
+    constexpr uint32_t IDESC = idesc_bf16(kBM, BN) | (1u << 15) | (1u << 16);
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint64_t* full = (uint64_t*)(smem + S * STAGE);
+    uint64_t* empty = full + S;
+    uint64_t* done = empty + S;
+    uint32_t* tmem_slot = (uint32_t*)(done + 1);
+    volatile int* abort_flag = (volatile int*)(tmem_slot + 1);
+    int* counts = (int*)(tmem_slot + 2);  // [0] loads issued, [1] stages consumed
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int m0 = blockIdx.x * kBM, n0 = blockIdx.y * BN;
+    const int b0 = blockIdx.z * per_split, nk = min(blocks - b0, per_split);
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(done, 1);
+        *abort_flag = 0;
+        counts[0] = counts[1] = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
+                     "r"((uint32_t)BN)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = *tmem_slot;
+
+    if (warp == 0) {
+        const uint32_t lead = elect_lane();
+        for (int it = 0; it < nk; ++it) {
+            const int st = it % S, p0 = (b0 + it) * 64;
+            if (it >= S && !mbar_wait_warp(&empty[st], (uint32_t)((it / S - 1) & 1), abort_flag)) break;
+            uint8_t* a = smem + st * STAGE;
+            if (lead) {
+                mbar_expect_tx(&full[st], STAGE);
+#pragma unroll
+                for (int j = 0; j < 2; ++j) tma_load_2d(a + j * ABOX, &tmA, m0 + 64 * j, p0, &full[st]);
+#pragma unroll
+                for (int j = 0; j < NB; ++j) tma_load_2d(a + 2 * ABOX + j * BBOX, &tmB, n0 + 64 * j, p0, &full[st]);
+                counts[0] = it + 1;
+            }
+            __syncwarp();
+        }
+    } else if (warp == 1) {
+        const uint32_t lead = elect_lane();
+        const unsigned long long lim = g_operand_wait_ns;
+        constexpr uint32_t AHI = mn_desc_hi<128>(), BHI = mn_desc_hi<YB>();
+        for (int it = 0; it < nk; ++it) {
+            const int st = it % S;
+            if (!mbar_wait_warp(&full[st], (uint32_t)((it / S) & 1), abort_flag, lim)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            const uint32_t a0 = smem_u32(smem + st * STAGE);
+            const uint32_t alo = mn_desc_lo(a0, ABOX), blo = mn_desc_lo(a0 + 2 * ABOX, BBOX);
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                umma_lead(lead, tmem, alo + (16 * 128 * s >> 4), AHI, blo + (16 * YB * s >> 4), BHI, IDESC,
+                          (it > 0 || s > 0) ? 1u : 0u);
+            if (lead) {
+                umma_commit(&empty[st]);
+                counts[1] = it + 1;
+            }
+            __syncwarp();
+        }
+        if (lead) umma_commit(done);
+        __syncwarp();
+    } else if (mbar_wait_abort(done, 0, abort_flag) && !*abort_flag) {
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const int q = warp & 3, row = m0 + q * 32 + lane;
+        float* out = part + ((size_t)blockIdx.z * M + row) * N + n0;
+#pragma unroll 1
+        for (int c = 0; c < BN; c += 32) {
+            uint32_t r[32];
+            tmem_ld32(r, tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c);
+            tmem_wait32(r);
+            if (row >= M) continue;
+#pragma unroll
+            for (int j = 0; j < 32; j += 8)
+                if (n0 + c + j < N) store32(out + c + j, r + j);  // N is a multiple of 8
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned long long t0 = global_ns();
+        bool fin = false;
+        while (!(fin = (bool)mbar_try(done, 0)) && global_ns() - t0 < kWaitNs) {
+        }
+        if (!fin) atomicExch(&g_gemm_error, 1);
+        if (*abort_flag)
+            for (int it = counts[1]; it < counts[0]; ++it) mbar_wait(&full[it % S], (uint32_t)((it / S) & 1));
+    }
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)BN) : "memory");
 }
