@@ -238,6 +238,10 @@ struct ConvGeo {
     int C = 0;             // input channels (a multiple of BK)
     int cblocks = 0;       // C / BK
     int row3 = 0;          // the A map's box is kBM + 2 pixels of one row (row-reuse form)
+    // tw > 0: a tile is tw x 128 / tw pixels (tw a power of two) of one image, tx
+    // x ty tiles cover it and nsub all images; pixels outside are not stored.
+    // tw == 0: 128 consecutive pixels, whole rows of whole images.
+    int tw = 0, tx = 0, ty = 0, nsub = 0;
 };
 struct ShuffleGeo {
     int Wl = 0, Hl = 0;    // low-resolution image; Wl == 0: plain row-major store
@@ -755,7 +759,12 @@ __global__ void __launch_bounds__(kWsGemmThreads, 1)
                 for (int i = 0; i < MT; ++i) {
                     const int mi = m0 + i * kBM;
                     x0[i] = y0[i] = b0[i] = 0;
-                    if (CONV) {
+                    if (CONV && geo.tw) {
+                        const int si = mi / kBM, r = si / geo.tx;
+                        x0[i] = (si - r * geo.tx) * geo.tw;
+                        b0[i] = r / geo.ty;
+                        y0[i] = (r - b0[i] * geo.ty) * (kBM / geo.tw);
+                    } else if (CONV) {
                         x0[i] = mi % geo.W;
                         y0[i] = (mi / geo.W) % geo.H;
                         b0[i] = mi / (geo.W * geo.H);
@@ -852,7 +861,13 @@ __global__ void __launch_bounds__(kWsGemmThreads, 1)
 #pragma unroll 1
             for (int un = grp; un < MT * UN; un += 2) {
                 const int sub = un / UN, c = (un % UN) * 32;
-                const int row = (t % tiles_m) * (kBM * MT) + sub * kBM + q * 32 + lane;
+                int row = (t % tiles_m) * (kBM * MT) + sub * kBM + q * 32 + lane;
+                if (CONV && geo.tw) {  // pixel of a two-dimensional tile
+                    const int si = row / kBM, rt = si / geo.tx, b = rt / geo.ty, m = row % kBM;
+                    const int x = (si - rt * geo.tx) * geo.tw + m % geo.tw;
+                    const int y = (rt - b * geo.ty) * (kBM / geo.tw) + m / geo.tw;
+                    row = x < geo.W && y < geo.H ? (b * geo.H + y) * geo.W + x : M;
+                }
                 const int col = n0 + c;
                 uint32_t r[32];
                 tmem_ld32(r, tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * ACC_COLS + sub * SUB_COLS + c));
@@ -1041,7 +1056,8 @@ cudaError_t launch_ws_mt(const CUtensorMap& a, const CUtensorMap& b, void* D, co
             return e;
         per_sm = occ < 1 ? 1 : occ;
     }
-    const int tiles_m = (M + kBM * MT - 1) / (kBM * MT);
+    const int Mt = geo.tw ? geo.nsub * kBM : M;  // rows of whole sub-tiles
+    const int tiles_m = (Mt + kBM * MT - 1) / (kBM * MT);
     const int tiles = tiles_m * ((N + BN - 1) / BN);
     const int grid = tiles < sms * per_sm ? tiles : sms * per_sm;
     k_gemm_ws<BN, OUT_BF16, BK, CONV, MT, ROW3><<<grid, kWsGemmThreads, smem, s>>>(a, b, D, bias, M, N, K, ldd, relu, geo,
@@ -1072,7 +1088,8 @@ cudaError_t launch_ws_rows(const CUtensorMap& a, const CUtensorMap& b, void* D, 
     sm_count();
     constexpr int MTMAX = (BN <= 32 && BK == 32) ? 4 : BN <= 128 ? 2 : 1;
     const long long ntiles_n = (N + BN - 1) / BN;
-    auto fills = [&](int mt) { return (M + 128LL * mt - 1) / (128LL * mt) * ntiles_n >= g_sms; };
+    const long long Mt = geo.tw ? 128LL * geo.nsub : M;
+    auto fills = [&](int mt) { return (Mt + 128LL * mt - 1) / (128LL * mt) * ntiles_n >= g_sms; };
     if constexpr (MTMAX == 4)
         if (fills(4))
             return launch_ws_mt<BN, OUT_BF16, BK, CONV, 4, ROW3>(a, b, D, bias, M, N, K, ldd, relu, geo, sh, s);
@@ -1093,9 +1110,22 @@ cudaError_t launch_ws(const CUtensorMap& a, const CUtensorMap& b, void* D, const
     return launch_ws_rows<BN, OUT_BF16, BK, CONV, false>(a, b, D, bias, M, N, K, ldd, relu, geo, sh, s);
 }
 
+#ifndef LBM_BN_FILL
+#define LBM_BN_FILL 0.5
+#endif
 // Widest tile that N allows: narrower tiles with more CTAs re-read A and
 // measured slower even where the wide tiles leave SMs idle.
 int bn_for(int N) { return N >= 256 ? 256 : N > 64 ? 128 : N > 32 ? 64 : 32; }
+
+// The same for a persistent GEMM of `tiles_m` row tiles: narrowed to 64 columns at
+// least while that leaves SMs without a tile.  A CTA's loads per K block, not the
+// MMAs, set its pace, and fewer columns are fewer weights to load.
+int bn_fill(int N, long long tiles_m)
+{
+    int bn = bn_for(N);
+    while (bn > 64 && tiles_m * ((N + bn - 1) / bn) < LBM_BN_FILL * sm_count()) bn /= 2;
+    return bn;
+}
 
 template <int BK, bool CONV>
 cudaError_t dispatch(int bn, bool ob, const CUtensorMap& ta, const CUtensorMap& tb, void* out, const float* bias, int M,
@@ -1486,7 +1516,7 @@ cudaError_t gemm_bf16(const void* A, int lda, const void* B, int ldb, void* D, i
                       int N, int K, bool out_bf16, bool relu, cudaStream_t s, int splits, float* workspace,
                       const void* mask, int mpitch)
 {
-    const int bn = bn_for(N);
+    const int bn = splits > 1 ? bn_for(N) : bn_fill(N, (M + kBM - 1) / kBM);
     if (N < 8 || N % 8) return cudaErrorInvalidValue;
     if (mask && (!mask_ok(mask, mpitch, out_bf16, N) || splits > 1)) return cudaErrorInvalidValue;
     if (lda % 8 || ldb % 8 || ldd % 8 || K > lda || K > ldb || N > ldd || M < 1 || K < 1) return cudaErrorInvalidValue;
@@ -1544,10 +1574,34 @@ bool conv_tile(int B, int H, int W, int* bw, int* bh, int* bb)
     return true;
 }
 
-bool conv3x3_supported(int B, int H, int W, int C)
+bool conv3x3_whole_rows(int B, int H, int W)
 {
     int bw, bh, bb;
-    return C % 32 == 0 && conv_tile(B, H, W, &bw, &bh, &bb);
+    return conv_tile(B, H, W, &bw, &bh, &bb);
+}
+
+bool conv3x3_supported(int C) { return C % 32 == 0; }
+
+// Two-dimensional tiles for images that no run of 128 consecutive pixels fits:
+// the width that pads least, row reuse (128 wide, at most 64 columns) counting
+// for a third of the loads it saves.
+static void conv_tile_2d(int B, int H, int W, int bn, ConvGeo* g, bool* row3)
+{
+    double best = 0.0;
+    for (int tw = 128; tw >= 8; tw /= 2) {
+        const int th = kBM / tw;
+        const long long tx = (W + tw - 1) / tw, ty = (H + th - 1) / th;
+        const bool r3 = tw == kBM && W >= 2 * kBM && bn <= 64;
+        const double cost = (double)(tx * ty) * (r3 ? 1.0 : 1.3);
+        if (best == 0.0 || cost < best) {
+            best = cost;
+            g->tw = tw;
+            g->tx = (int)tx;
+            g->ty = (int)ty;
+            g->nsub = (int)(B * tx * ty);
+            *row3 = r3;
+        }
+    }
 }
 
 static cudaError_t conv3x3(const void* X, int B, int H, int W, int C, int cpitch, const void* Wm, int ldw, void* D,
@@ -1558,8 +1612,7 @@ cudaError_t conv3x3_bf16(const void* X, int B, int H, int W, int C, int cpitch, 
                          int ldd, const float* bias, int N, bool out_bf16, bool relu, cudaStream_t s,
                          const void* mask, int mpitch)
 {
-    int bw, bh, bb;
-    if (C % 32 || !conv_tile(B, H, W, &bw, &bh, &bb)) return cudaErrorNotSupported;
+    if (C % 32) return cudaErrorNotSupported;
     if (mask && !mask_ok(mask, mpitch, out_bf16, N)) return cudaErrorInvalidValue;
     if (N > ldd) return cudaErrorInvalidValue;
     ShuffleGeo sh;
@@ -1568,15 +1621,15 @@ cudaError_t conv3x3_bf16(const void* X, int B, int H, int W, int C, int cpitch, 
     return conv3x3(X, B, H, W, C, cpitch, Wm, ldw, D, ldd, bias, N, out_bf16, relu, sh, s);
 }
 
-bool conv3x3_split_supported(int B, int H, int W, int c)
+bool conv3x3_split_supported(int H, int W, int c)
 {
-    return H % 2 == 0 && W % 2 == 0 && conv3x3_supported(B, H, W, c);
+    return H % 2 == 0 && W % 2 == 0 && conv3x3_supported(c);
 }
 
 cudaError_t conv3x3_split(const void* X, int B, int H, int W, int c, const void* Wm, float* D, void* dU,
                           cudaStream_t s)
 {
-    if (!conv3x3_split_supported(B, H, W, c) || ((uintptr_t)dU & 15)) return cudaErrorInvalidValue;
+    if (!conv3x3_split_supported(H, W, c) || ((uintptr_t)dU & 15)) return cudaErrorInvalidValue;
     ShuffleGeo sh;
     sh.c = c;
     sh.dU = (__nv_bfloat16*)dU;
@@ -1590,20 +1643,28 @@ static cudaError_t conv3x3(const void* X, int B, int H, int W, int C, int cpitch
                            cudaStream_t s)
 {
     const int bk = C % 64 == 0 ? 64 : C % 32 == 0 ? 32 : 0;
-    int bw, bh, bb;
-    if (!bk || !conv_tile(B, H, W, &bw, &bh, &bb)) return cudaErrorNotSupported;
+    if (!bk) return cudaErrorNotSupported;
     if (N < 8 || N % 8 || cpitch % 8 || C > cpitch || ldw % 8 || ldw < 9 * C || ldd % 8)
         return cudaErrorInvalidValue;
     if (((uintptr_t)X | (uintptr_t)Wm | (uintptr_t)D) & 15) return cudaErrorInvalidValue;
-    const int bn = bn_for(N);
-    // rows of at least 256 pixels: each stage loads one box of 130 pixels of
-    // an input row and serves its three taps from it
-    const bool row3 = bw == kBM && W >= 2 * kBM && bn <= 64;
+    const int bn = bn_fill(N, ((long long)B * H * W + kBM - 1) / kBM);
+    ConvGeo geo;
+    int bw, bh, bb;
+    bool row3 = false;
+    if (conv_tile(B, H, W, &bw, &bh, &bb)) {
+        // rows of at least 256 pixels: each stage loads one box of 130 pixels of
+        // an input row and serves its three taps from it
+        row3 = bw == kBM && W >= 2 * kBM && bn <= 64;
+    } else {
+        conv_tile_2d(B, H, W, bn, &geo, &row3);
+        bw = geo.tw;
+        bh = kBM / geo.tw;
+        bb = 1;
+    }
     CUtensorMap ta, tb;
     cudaError_t e = make_map_4d(&ta, X, B, H, W, C, cpitch, row3 ? kBM + 2 : bw, bh, bb, bk);
     if (e == cudaSuccess) e = make_map(&tb, Wm, N, 9 * C, ldw, bn, bk);
     if (e != cudaSuccess) return e;
-    ConvGeo geo;
     geo.W = W;
     geo.H = H;
     geo.C = C;
@@ -1622,7 +1683,7 @@ cudaError_t upconv2x2_bf16(const void* X, int lda, const void* Wm, int ldw, void
     const int N = 4 * c, M = B * Hl * Wl, K = cin;
     if (c % 16 || lda % 8 || ldw % 8 || ypitch % 8 || K > lda || K > ldw || c0 + c > ypitch) return cudaErrorInvalidValue;
     if (((uintptr_t)X | (uintptr_t)Wm | (uintptr_t)Y) & 15) return cudaErrorInvalidValue;
-    const int bn = bn_for(N);
+    const int bn = bn_fill(N, (M + kBM - 1) / kBM);
     CUtensorMap ta, tb;
     cudaError_t e = make_map(&ta, X, M, K, lda, kBM, kBK);
     if (e == cudaSuccess) e = make_map(&tb, Wm, N, K, ldw, bn, kBK);

@@ -25,22 +25,24 @@ cudaError_t gemm_bf16_tout(const void* A, int lda, const void* B, int ldb, float
 // Implicit 3 x 3 convolution (zero padding) on tensor cores:
 // D[p][n] = act(sum over taps t and channels c < C of X[pixel p shifted by t][c]
 // * Wm[n][t * C + c] + bias[n]) with X NHWC BF16 [B][H][W][cpitch] and the
-// weight matrix Wm [N][ldw] (ldw >= 9C).  C must be a multiple of 32 and a
-// 128-pixel tile whole rows of whole images (W a multiple of 128, or a divisor
-// of 128 with matching H); cudaErrorNotSupported otherwise.
+// weight matrix Wm [N][ldw] (ldw >= 9C).  C a multiple of 32, else
+// cudaErrorNotSupported.  Tiles are 128 consecutive pixels where those are whole
+// rows of whole images (conv3x3_whole_rows: W a multiple of 128, or a divisor of
+// 128 with matching H), two-dimensional ones with a ragged edge otherwise.
 // mask: as for gemm_bf16 (BF16 output).
 cudaError_t conv3x3_bf16(const void* X, int B, int H, int W, int C, int cpitch, const void* Wm, int ldw, void* D,
                          int ldd, const float* bias, int N, bool out_bf16, bool relu, cudaStream_t s,
                          const void* mask = nullptr, int mpitch = 0);
 
-bool conv3x3_supported(int B, int H, int W, int C);
+bool conv3x3_supported(int C);
+bool conv3x3_whole_rows(int B, int H, int W);
 
 // The input gradient of a decoder's first convolution, whose input is the
 // concatenation [skip, up] of c channels each: the implicit convolution of X
 // [P][c] with Wm [2c][9c], its first c columns stored to D (FP32 [P][c]), the
 // others rounded to BF16 into dU[(b, y/2, x/2)][((y&1) 2 + (x&1)) c + co], the
 // layout of the up-convolution's output.  c a multiple of 32.
-bool conv3x3_split_supported(int B, int H, int W, int c);
+bool conv3x3_split_supported(int H, int W, int c);
 cudaError_t conv3x3_split(const void* X, int B, int H, int W, int c, const void* Wm, float* D, void* dU,
                           cudaStream_t s);
 

@@ -281,18 +281,18 @@ cudaError_t allocate(lbm_unet* u)
         }
         for (Conv* cv : {&v.ea, &v.eb, &v.da, &v.db})
             if (cv->cout) UN_ALLOC(cv->wf, 9LL * cv->cin * cv->cout);
-        if (l == 0 && nn::conv3x3_supported(u->B, v.H, v.W, kX0Pitch)) {
+        if (l == 0 && nn::conv3x3_whole_rows(u->B, v.H, v.W)) {
             v.ea.cin_pad = kX0Pitch;
             UN_ALLOC(v.ea.wpad, 9LL * kX0Pitch * v.ea.cout);
         }
         if (v.up.cout) UN_ALLOC(v.up.wt, 8LL * c * c);
     }
     // gathered-copy buffer for the convolutions the implicit kernel does not
-    // take (the first one, 8 input channels; any level of an odd image size)
+    // take (the first one, 8 input channels; channels no multiple of 32)
     long long col_n = 9LL * P0 * kInPitch;
     for (const Level& v : u->lv)
         for (const Conv* cv : {&v.ea, &v.eb, &v.da, &v.db})
-            if (cv->cout && !nn::conv3x3_supported(u->B, v.H, v.W, cv->cin)) col_n = std::max(col_n, 9 * v.P * cv->cin);
+            if (cv->cout && !nn::conv3x3_supported(cv->cin)) col_n = std::max(col_n, 9 * v.P * cv->cin);
     UN_ALLOC(u->col, col_n);
     u->col_n = col_n;
     // the table of kernel flips derive() runs in one launch (the weight and
@@ -345,14 +345,14 @@ cudaError_t allocate_backward(lbm_unet* u)
         const long long P = v.P;
         const int c = v.c;
         if (l < L - 1) {
-            v.dpitch = nn::conv3x3_split_supported(u->B, v.H, v.W, c) ? c : 2 * c;
+            v.dpitch = nn::conv3x3_split_supported(v.H, v.W, c) ? c : 2 * c;
             UN_ALLOC(v.dcat, P * v.dpitch);
         }
         int n = 0;
         for (Conv* cv : {&v.ea, &v.eb, &v.da, &v.db}) {
             if (!cv->cout) continue;
             const int K9 = 9 * cv->cin, N = cv->cout, C = wgrad_channels(*cv);
-            if (!nn::conv3x3_supported(u->B, v.H, v.W, N)) col_n = std::max(col_n, 9 * P * N);
+            if (!nn::conv3x3_supported(N)) col_n = std::max(col_n, 9 * P * N);
             if (nn::wgrad_direct_supported(v.W, C, cv->first ? kX0Pitch : cv->cin, N)) {
                 if ((e = nn::wgrad_direct(nullptr, u->B, v.H, v.W, C, C, cv->cin, nullptr, N, u->s,
                                           splits_for(K9, N, P), nullptr, &n)))
