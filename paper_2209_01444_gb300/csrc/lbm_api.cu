@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "lbm.h"
+#include "host_staging.h"
 #include "lbm_kernels.h"
 #include "trace.h"
 
@@ -404,49 +405,25 @@ int graph_for(lbm_handle* h, cudaGraphExec_t* out)
     return LBM_OK;
 }
 
-// Pinned host staging buffer of lbm_get_fields (and of lbm_get_fields_f32 into
-// pageable memory), shared by every handle of the process (at most 2 x
-// kPinHalf bytes, allocated on first use, kept until exit); a call holds the
-// mutex while it uses it.
-constexpr size_t kPinHalf = (size_t)32 << 20;
-struct PinnedStaging {
-    std::mutex mu;
-    float* p = nullptr;
-    size_t bytes = 0;
-} g_pinned;
+using lbm::g_pinned;
+using lbm::kPinHalf;
 
 // The shared staging buffer, grown to at least `bytes`; the caller holds
 // g_pinned.mu for as long as it uses the buffer.  Null (with h's error set)
 // when page-locked memory cannot be had.
 float* staging_buffer(lbm_handle* h, size_t bytes)
 {
-    if (g_pinned.bytes < bytes) {
-        if (g_pinned.p) cudaFreeHost(g_pinned.p);
-        g_pinned.p = nullptr;
-        g_pinned.bytes = 0;
-        cudaError_t e = cudaHostAlloc((void**)&g_pinned.p, bytes, cudaHostAllocPortable);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            fail(h, LBM_ENOMEM, std::string("pinned band buffer: ") + cudaGetErrorString(e));
-            return nullptr;
-        }
-        g_pinned.bytes = bytes;
-    }
-    return g_pinned.p;
+    cudaError_t e = cudaSuccess;
+    float* p = lbm::pinned_staging(bytes, &e);
+    if (!p) fail(h, LBM_ENOMEM, std::string("pinned band buffer: ") + cudaGetErrorString(e));
+    return p;
 }
 
 // Runs fn(r0, r1) over the row range [0, rows) on up to 16 host threads.
 template <class Fn>
 void parallel_rows(int rows, Fn fn)
 {
-    const int nt = std::max(1, std::min({(int)std::thread::hardware_concurrency(), 16, rows / 8}));
-    if (nt == 1) {
-        fn(0, rows);
-        return;
-    }
-    std::vector<std::thread> pool;
-    for (int t = 0; t < nt; ++t) pool.emplace_back(fn, rows * t / nt, rows * (t + 1) / nt);
-    for (std::thread& th : pool) th.join();
+    lbm::parallel_range(rows, 8, [&](long long r0, long long r1) { fn((int)r0, (int)r1); });
 }
 
 }  // namespace
@@ -1309,6 +1286,26 @@ int params_to_step(const lbm_params* p, StepParams* out, const char** why)
 
 // Message returned by lbm_last_error(NULL) for calls that take no handle.
 void set_last_error(const char* msg) { g_create_error = msg; }
+
+PinnedStaging g_pinned;
+
+float* pinned_staging(size_t bytes, cudaError_t* e)
+{
+    *e = cudaSuccess;
+    if (g_pinned.bytes < bytes) {
+        if (g_pinned.p) cudaFreeHost(g_pinned.p);
+        g_pinned.p = nullptr;
+        g_pinned.bytes = 0;
+        *e = cudaHostAlloc((void**)&g_pinned.p, bytes, cudaHostAllocPortable);
+        if (*e != cudaSuccess) {
+            cudaGetLastError();
+            g_pinned.p = nullptr;
+            return nullptr;
+        }
+        g_pinned.bytes = bytes;
+    }
+    return g_pinned.p;
+}
 
 }  // namespace lbm
 

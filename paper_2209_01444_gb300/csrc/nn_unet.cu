@@ -29,6 +29,7 @@
 #include <string>
 #include <vector>
 
+#include "host_staging.h"
 #include "lbm.h"
 #include "nn_kernels.h"
 #include "nn_layers.h"
@@ -670,13 +671,37 @@ int lbm_unet_set_params(lbm_unet* u, const float* host)
     return LBM_OK;
 }
 
+// The packed tensors of a padded device vector to host memory: through the
+// page-locked staging buffer at the host link's rate, then on up to 16 threads
+// into the caller's (pageable, often untouched) memory.  A zeroed vector as the
+// way-station of a pageable copy took 2.4 ms for the five-level network's 31 MB.
 static int get_vec(lbm_unet* u, const float* dev, float* host)
 {
     if (!u || !host) return LBM_EINVAL;
-    std::vector<float> pad((size_t)u->n_padded);
-    UN_CHECK(u, cudaStreamSynchronize(u->s));
-    UN_CHECK(u, cudaMemcpy(pad.data(), dev, pad.size() * sizeof(float), cudaMemcpyDeviceToHost));
-    for (const Tensor& t : u->tensors) std::memcpy(host + t.packed, &pad[t.padded], (size_t)t.n * sizeof(float));
+    const long long chunk = 2 * (long long)lbm::kPinHalf / (long long)sizeof(float);
+    std::lock_guard<std::mutex> hold(lbm::g_pinned.mu);
+    cudaError_t e = cudaSuccess;
+    float* pin = lbm::pinned_staging((size_t)std::min(u->n_padded, chunk) * sizeof(float), &e);
+    if (!pin) {  // no page-locked memory: tensor by tensor
+        UN_CHECK(u, cudaStreamSynchronize(u->s));
+        for (const Tensor& t : u->tensors)
+            UN_CHECK(u, cudaMemcpy(host + t.packed, dev + t.padded, (size_t)t.n * sizeof(float), cudaMemcpyDeviceToHost));
+        return LBM_OK;
+    }
+    for (long long c0 = 0; c0 < u->n_padded; c0 += chunk) {
+        const long long c1 = std::min(u->n_padded, c0 + chunk);
+        UN_CHECK(u, cudaMemcpyAsync(pin, dev + c0, (size_t)(c1 - c0) * sizeof(float), cudaMemcpyDeviceToHost, u->s));
+        UN_CHECK(u, cudaStreamSynchronize(u->s));
+        lbm::parallel_range(u->n_packed, 1 << 18, [&](long long p0, long long p1) {
+            for (const Tensor& t : u->tensors) {
+                // values [a, b) of this tensor: in this thread's share and in the chunk
+                const long long a = std::max({0LL, p0 - t.packed, c0 - t.padded});
+                const long long b = std::min({t.n, p1 - t.packed, c1 - t.padded});
+                if (a < b)
+                    std::memcpy(host + t.packed + a, pin + (t.padded + a - c0), (size_t)(b - a) * sizeof(float));
+            }
+        });
+    }
     return LBM_OK;
 }
 
