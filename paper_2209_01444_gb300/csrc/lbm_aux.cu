@@ -6,6 +6,7 @@
 
 #include "lbm_kernels.h"
 #include "lbm_reduce.cuh"
+#include "pdl.cuh"
 
 namespace lbm {
 
@@ -347,19 +348,27 @@ __global__ void __launch_bounds__(kRedThreadsPerBlock) k_reduce_nodes(const Step
                                                                       const void* __restrict__ fl,
                                                                       double* __restrict__ partials)
 {
+    pdl_release();
     reduce_chunk<Store>(P, sc, fl, partials);
+    pdl_wait();  // launched beside k_tips: completes after it
 }
 
 // Pass 2: one warp per value folds the partials: lane l takes blocks
 // l, l + 32, ..., then a shuffle tree adds the lanes (a fixed order).
 __global__ void k_reduce_final(const double* __restrict__ partials, int nblocks, double* __restrict__ out)
 {
+    pdl_begin();
     const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (k >= kRedVals) return;
     double v = 0.0;
-    for (int b = lane; b < nblocks; b += 32) {
-        const double p = partials[(long long)b * kRedVals + k];
-        v = (k == 4) ? fmax(v, p) : v + p;
+    for (int b = lane; b < nblocks; b += 32 * 8) {
+        // eight partials in flight, added in block order
+        double p[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) p[j] = b + 32 * j < nblocks ? partials[(long long)(b + 32 * j) * kRedVals + k] : 0.0;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (b + 32 * j < nblocks) v = (k == 4) ? fmax(v, p[j]) : v + p[j];
     }
     v = (k == 4) ? warp_max(v) : warp_sum(v);
     if (lane == 0) out[k] = v;
@@ -473,6 +482,7 @@ __global__ void __cluster_dims__(kTipCluster, 1, 1) __launch_bounds__(kTipThread
            double* __restrict__ out)
 {
     namespace cg = cooperative_groups;
+    pdl_release();
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int r = blockIdx.x / kTipCluster;
@@ -607,11 +617,15 @@ template <class Store>
 cudaError_t reduce_t(const StepParams& P, const void* sc, const void* fl, double cx, double cy, double c, double s,
                      double* partials, double* out, cudaStream_t st)
 {
+    // The tips' few CTAs (10 us) run beside the node pass: k_tips starts once the
+    // state is complete and releases k_reduce_nodes, which reads the same state,
+    // at once; that one's completion waits for the tips'.
     const int nb = reduce_blocks(P);
-    k_reduce_nodes<Store><<<nb, kRedThreadsPerBlock, 0, st>>>(P, sc, fl, partials);
-    k_reduce_final<<<1, 32 * kRedVals, 0, st>>>(partials, nb, out);
     k_tips<Store><<<3 * kTipCluster, kTipThreads, 0, st>>>(P, sc, cx, cy, c, s, out);
-    return cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = launch_pdl(k_reduce_nodes<Store>, nb, kRedThreadsPerBlock, 0, st, P, sc, fl, partials);
+    if (e == cudaSuccess) e = launch_pdl(k_reduce_final, 1, 32 * kRedVals, 0, st, (const double*)partials, nb, out);
+    return e;
 }
 
 }  // namespace

@@ -47,23 +47,31 @@ template <class Store>
 __device__ __forceinline__ void reduce_chunk(const StepParams& P, const void* __restrict__ sc,
                                              const void* __restrict__ fl, double* __restrict__ partials)
 {
-    const long long N = (long long)P.nx * P.ny;
-    const long long first = (long long)blockIdx.x * kRedNodesPerBlock;
-    const long long last = min(first + kRedNodesPerBlock, N);
+    // (grids hold at most 2^31 nodes: 32-bit division, once per thread)
+    const unsigned N = (unsigned)P.nx * (unsigned)P.ny;
+    const unsigned first = blockIdx.x * (unsigned)kRedNodesPerBlock;
+    const unsigned nodes = min((unsigned)kRedNodesPerBlock, N - first);
+    unsigned y = (first + threadIdx.x) / (unsigned)P.nx, x = (first + threadIdx.x) - y * (unsigned)P.nx;
     float sp1 = 0.0f, sdC = 0.0f, sdH = 0.0f, sh = 0.0f, umax = 0.0f;
     int bad = 0, count = 0;
-    for (long long t = first + threadIdx.x; t < last; t += kRedThreadsPerBlock) {
-        const int y = (int)(t / P.nx), x = (int)(t - (long long)y * P.nx);
+    // the next node's 24 loads are in flight while a node is added
+    float v[24], w[24];
+    auto load = [&](float (&d)[24]) {
         const long long o = (long long)y * P.pitch + x;
-        float f[5], n[5], g[5], h[9];
 #pragma unroll
-        for (int i = 0; i < 5; ++i) f[i] = Store::load(sc, fl, kF + i, o, P);
+        for (int i = 0; i < 24; ++i) d[i] = Store::load(sc, fl, i, o, P);
+        x += kRedThreadsPerBlock;
+        while (x >= (unsigned)P.nx) {
+            x -= (unsigned)P.nx;
+            ++y;
+        }
+    };
+    if (threadIdx.x < nodes) load(w);
+    for (unsigned t = threadIdx.x; t < nodes; t += kRedThreadsPerBlock) {
 #pragma unroll
-        for (int i = 0; i < 5; ++i) n[i] = Store::load(sc, fl, kN + i, o, P);
-#pragma unroll
-        for (int i = 0; i < 5; ++i) g[i] = Store::load(sc, fl, kG + i, o, P);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) h[i] = Store::load(sc, fl, kH + i, o, P);
+        for (int i = 0; i < 24; ++i) v[i] = w[i];
+        if (t + kRedThreadsPerBlock < nodes) load(w);
+        const float *f = v + kF, *n = v + kN, *g = v + kG, *h = v + kH;
         const Macro m = node_macros(f, n, g, h, P);
         float s9 = 0.0f;
 #pragma unroll

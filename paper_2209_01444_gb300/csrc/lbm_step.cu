@@ -22,42 +22,17 @@
 #include <stddef.h>
 
 #include <type_traits>
-#include <utility>
 
 #include "lbm_kernels.h"
+#include "pdl.cuh"
 
 namespace lbm {
 
 namespace {
 
-// Programmatic dependent launch of the flow steps: a kernel is launched before
-// its predecessor on the stream has drained, so that its launch and the start
-// of its CTAs overlap the predecessor's last wave.  pdl_begin releases the
-// successor likewise and then waits until every kernel before this one has
-// completed and its writes are visible; no buffer is touched before it.  (The
-// coupled steps do without: in a captured graph their launches cost little, and
-// early CTAs took SM slots from the last wave, 1024^2 0.7 % slower.)
-__device__ __forceinline__ void pdl_begin()
-{
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-
-template <class... Par, class... Arg>
-cudaError_t launch_pdl(void (*kernel)(Par...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Arg&&... arg)
-{
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, std::forward<Arg>(arg)...);
-}
+// The flow steps are launched as programmatic dependents (pdl.cuh).  The coupled
+// steps are not: in a captured graph their launches cost little, and early CTAs
+// took SM slots from the last wave (1024^2 0.7 % slower).
 
 constexpr int kLocalGradIters = 2;  // fixed-point passes of the local grad(phi) scheme
 
