@@ -18,6 +18,7 @@
 // sides the wrapped values land on wall nodes, which the wall scheme then
 // overwrites completely: the wall kernels after the step, or the next step of
 // the same call as it loads them (coupled_tile).
+#include <cuda_pipeline_primitives.h>
 #include <cuda_runtime.h>
 #include <stddef.h>
 
@@ -612,8 +613,10 @@ __device__ __forceinline__ void flow_collide(const StepParams& P, float phi, flo
     collide_flow<1, Store::kSF>(h, m, P.s2u, ho);
 }
 
-// The same for two nodes at once, in packed FP32 (one instruction for both):
-// the operations and their order are those of flow_macros and collide_flow.
+// The same for two nodes at once, in packed FP32 (one instruction for both), with
+// the sums that directions share taken once: of flow_macros and collide_flow
+// 68 operations are left of 94 (their packed form runs at half rate, so the FMA
+// pipe, not the issue slots, sets the pace of a collision).
 struct F2 {
     float2 v;
 };
@@ -623,40 +626,41 @@ __device__ __forceinline__ F2 operator+(F2 a, F2 b) { return {__fadd2_rn(a.v, b.
 __device__ __forceinline__ F2 operator-(F2 a, F2 b) { return fma2(b, f2(-1.0f), a); }
 __device__ __forceinline__ F2 operator*(F2 a, F2 b) { return {__fmul2_rn(a.v, b.v)}; }
 
+// nw: q~ - 1 = -(1 + phi)/2; hFy: half the body force along y.
 template <class Store>
-__device__ __forceinline__ void flow_collide2(const StepParams& P, F2 phi, F2 Fy, const F2 (&h)[9], F2 (&out)[9])
+__device__ __forceinline__ void flow_collide2(const StepParams& P, F2 nw, F2 hFy, const F2 (&h)[9], F2 (&out)[9])
 {
-    const F2 half = f2(0.5f), third = f2(1.0f / 3.0f), Fx = f2(P.Fx);
-    const F2 ns2 = f2(-P.s2u);
-    const F2 jx = h[1] - h[3] + h[5] - h[6] - h[7] + h[8];
-    const F2 jy = h[2] - h[4] + h[5] + h[6] - h[7] - h[8];
-    const F2 rest = h[1] + h[2] + h[3] + h[4] + h[5] + h[6] + h[7] + h[8];
-    const F2 usx = fma2(half, Fx, jx), usy = fma2(half, Fy, jy);
-    const F2 nw = fma2(f2(-0.5f), phi + f2(1.0f), f2(1.0f)) + f2(-1.0f);  // q~ - 1
+    constexpr float SO = (float)Store::kSF;
+    const F2 half = f2(0.5f), ns2 = f2(-P.s2u), hFx = f2(0.5f * P.Fx);
+    const F2 a = h[5] - h[7], b = h[6] - h[8], e = h[5] + h[7], f = h[6] + h[8];
+    const F2 s13 = h[1] + h[3], s24 = h[2] + h[4], d = e + f;
+    const F2 usx = (h[1] - h[3]) + (a - b) + hFx, usy = (h[2] - h[4]) + (a + b) + hFy;  // u*
+    const F2 mxx = s13 + d, myy = s24 + d, mxy = e - f, rest = mxx + s24;
     const F2 nt = nw * half;
     const F2 u = fma2(nt, usx, usx), v = fma2(nt, usy, usy);
     const F2 p = f2(0.6f) * fma2(f2(-(2.0f / 3.0f)), fma2(u, u, v * v), rest);
-    const F2 Fpx = fma2(nw, usx, Fx), Fpy = fma2(nw, usy, Fy);
-    const F2 mxx = h[1] + h[3] + h[5] + h[6] + h[7] + h[8];
-    const F2 myy = h[2] + h[4] + h[5] + h[6] + h[7] + h[8];
-    const F2 mxy = h[5] - h[6] + h[7] - h[8];
-    const F2 r1 = fma2(half, Fpx, u), r2 = fma2(half, Fpy, v);
+    // r1 = u + F'_x / 2 with F' = F + (1 - q~) f, f = -u*, and likewise r2
+    const F2 r1 = u + fma2(nt, usx, hFx), r2 = v + fma2(nt, usy, hFy);
     const F2 pu = fma2(u, u, p);
     const F2 r3 = fma2(ns2, mxx - pu, mxx);
     const F2 r4 = fma2(ns2, myy - fma2(v, v, p), myy);
     const F2 r5 = fma2(ns2, fma2(u * f2(-1.0f), v, mxy), mxy);
-    const F2 r6 = r2 * third, r7 = r1 * third, r8 = fma2(v, v, pu) * third;
-    const F2 hO = f2(0.5f * Store::kSF), qO = f2(0.25f * Store::kSF);
-    out[0] = r8 - (r3 + r4);
-    if (Store::kSF != 1) out[0] = out[0] * f2((float)Store::kSF);
-    out[1] = hO * (r1 + r3 - r7 - r8);
-    out[3] = hO * (r3 - r1 + r7 - r8);
-    out[2] = hO * (r2 + r4 - r6 - r8);
-    out[4] = hO * (r4 - r2 + r6 - r8);
-    out[5] = qO * (r5 + r6 + r7 + r8);
-    out[6] = qO * (r6 - r5 - r7 + r8);
-    out[7] = qO * (r5 - r6 - r7 + r8);
-    out[8] = qO * (r7 - (r5 + r6) + r8);
+    const F2 r8 = fma2(v, v, pu) * f2(1.0f / 3.0f);
+    // (r1 - r7 along the axes, not its equal 2 r7: momentum is kept whatever the
+    // rounding of 1/3)
+    const F2 r6 = r2 * f2(1.0f / 3.0f), r7 = r1 * f2(1.0f / 3.0f);
+    out[0] = f2(SO) * (r8 - (r3 + r4));
+    const F2 hO = f2(0.5f * SO), ax = hO * (r3 - r8), ay = hO * (r4 - r8), bx = hO * (r1 - r7), by = hO * (r2 - r6);
+    out[1] = ax + bx;
+    out[3] = ax - bx;
+    out[2] = ay + by;
+    out[4] = ay - by;
+    const F2 q = f2(0.25f * SO), s = q * (r6 + r7), t = q * (r6 - r7);
+    const F2 c = q * (r8 + r5), g = q * (r8 - r5);
+    out[5] = c + s;
+    out[7] = c - s;
+    out[6] = g + t;
+    out[8] = g - t;
 }
 
 // One flow sub-step (two-time-scaling of Sec. 4): collide and stream h with phi
@@ -690,7 +694,12 @@ __global__ void __launch_bounds__(256, 8) k_flow_substep(const StepParams P, con
 // here a CTA takes a region of kFmW x kFmH nodes and keeps its flow populations
 // in shared memory for `ks` <= K steps.  The outermost nodes lose one ring per
 // step (their neighbours are not in the region), so the CTA writes the inner
-// (kFmW - 2 K) x (kFmH - 2 K) nodes, which are exact.
+// (kFmW - 2 KX) x (kFmH - 2 K) nodes, which are exact (KX: K rounded up, so that
+// regions start on a multiple of VW nodes).  Loads and stores of the populations
+// move VW = 4 (K = 5: 2) nodes of a plane at a time, the loads straight into
+// shared memory (cp.async): loading and storing took two thirds of a launch with
+// a register and an instruction per value (1.12 M nodes, four steps: 46.5
+// against 44 us; FP16 2.4 M nodes, 32 steps: 778 against 643 us).
 // Per step and node, each thread reads its own populations, collides (its rows
 // in pairs, packed FP32), and after a barrier pushes them to the neighbours'
 // places, in the storage type (16-bit storage rounds at every step as a store
@@ -702,6 +711,17 @@ constexpr int kFmW = 64;   // region width: two warps
 constexpr int kFmY = 8;    // rows of threads
 constexpr int kFmR = 4;    // rows per thread
 constexpr int kFmH = kFmY * kFmR;
+constexpr int kFmB = 4;    // border columns left and right (groups of four stay aligned)
+constexpr int kFmPW = kFmW + 2 * kFmB;
+constexpr int fm_kx(int K) { return K == 5 ? 6 : (K + 3) / 4 * 4; }
+template <int BYTES>
+struct VecOf;
+template <>
+struct VecOf<4> { using V = uint32_t; };
+template <>
+struct VecOf<8> { using V = uint2; };
+template <>
+struct VecOf<16> { using V = uint4; };
 
 // A flow population in shared memory: the storage type, in units of 1/kSF.
 template <class Store>
@@ -725,7 +745,7 @@ __device__ __forceinline__ float flow_dec(typename Store::T v)
 template <class Store>
 constexpr int flow_multi_smem()
 {
-    return 9 * (kFmW + 2) * (kFmH + 2) * (int)sizeof(typename Store::T) + 2 * (kFmW + kFmH) * (int)sizeof(float2);
+    return 9 * kFmPW * (kFmH + 2) * (int)sizeof(typename Store::T) + 2 * (kFmW + kFmH) * (int)sizeof(float2);
 }
 
 template <class Store, int K>
@@ -735,20 +755,21 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
                  int ks, int repair)
 {
     static_assert(kFmR % 2 == 0, "rows in pairs");
-    static_assert(kFmH > 2 * K && kFmW > 2 * K, "region size");
+    constexpr int KX = fm_kx(K);
+    static_assert(kFmH > 2 * K && kFmW > 2 * KX, "region size");
     using T = typename Store::T;
     constexpr int NR = kFmR, RH = kFmH;
-    // a border of one node around the region takes what leaves it (never read),
-    // so that every push is one store at a constant offset from the node
-    constexpr int PW = kFmW + 2, PP = PW * (RH + 2), PJ = kFmY * PW;
+    // a border around the region takes what leaves it (never read), so that
+    // every push is one store at a constant offset from the node
+    constexpr int PW = kFmPW, PP = PW * (RH + 2), PJ = kFmY * PW;
     constexpr int kPush[9] = {0, 1, PW, -1, -PW, PW + 1, PW - 1, -PW - 1, -PW + 1};
     extern __shared__ float2 fm_smem[];
     float2* rowS = fm_smem;              // [2][kFmW] scalars of the row walls' interior nodes
     float2* colS = rowS + 2 * kFmW;      // [2][RH] and of the column walls'
-    T* s = (T*)(colS + 2 * RH);          // [9][RH + 2][PW]
+    T* s = (T*)(colS + 2 * RH);          // [9][RH + 2][PW], node (lx, ly) at [ly + 1][lx + kFmB]
 
     const int lx = threadIdx.x, ty = threadIdx.y, t = ty * kFmW + lx;
-    const int rx0 = blockIdx.x * (kFmW - 2 * K) - K, ry0 = blockIdx.y * (RH - 2 * K) - K;
+    const int rx0 = blockIdx.x * (kFmW - 2 * KX) - KX, ry0 = blockIdx.y * (RH - 2 * K) - K;
     // node of this thread's column and rows; outside a wall there is none
     int gx = rx0 + lx;
     bool colx = true;
@@ -757,12 +778,12 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
     else
         colx = gx >= 0 && gx < P.nx;
     const int margin = K - ks;  // rings the region has in excess
-    T* const own = s + (ty + 1) * PW + lx + 1;  // row ty + kFmY j is PJ j further
+    T* const own = s + (ty + 1) * PW + lx + kFmB;  // row ty + kFmY j is PJ j further
     const bool walls = (!P.periodic_x && (rx0 <= 0 || rx0 + kFmW >= P.nx)) ||
                        (!P.periodic_y && (ry0 <= 0 || ry0 + RH >= P.ny));
 
     pdl_begin();
-    float ph[NR], fy[NR];
+    float nw[NR], hfy[NR];
     bool on[NR];
 #pragma unroll
     for (int j = 0; j < NR; ++j) {
@@ -775,12 +796,34 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
             rowy = gy >= 0 && gy < P.ny;
         on[j] = colx && rowy && ly >= margin && ly < RH - margin;
         const long long o = on[j] ? (long long)gy * P.pitch + gx : 0;
-        const T* e = (const T*)src + block_index(o, 9);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) own[i * PP + PJ * j] = e[32 * i];
-        ph[j] = phi[block_index(o, phi_np)];
-        fy[j] = fb[o];
+        nw[j] = -0.5f * (phi[block_index(o, phi_np)] + 1.0f);
+        hfy[j] = 0.5f * fb[o];
     }
+    // the region's populations, groups of VW nodes of a row and plane; rx0 is a
+    // multiple of VW, so a group inside the row lies in one node block
+    constexpr int VW = KX % 4 == 0 ? 4 : 2, G = kFmW / VW, GB = VW * (int)sizeof(T);
+    for (int q = t; q < G * RH; q += kFmW * kFmY) {
+        const int ly = q / G, c = VW * (q % G);
+        int y = ry0 + ly, x = rx0 + c;
+        if (P.periodic_y)
+            y = (y < 0 || y >= P.ny) ? wrap(y, P.ny) : y;
+        else
+            y = min(max(y, 0), P.ny - 1);  // (rows outside a wall are not used)
+        T* d = s + (ly + 1) * PW + c + kFmB;
+        if (!P.periodic_x) x = min(max(x, 0), P.pitch - VW);  // (nor are columns)
+        if (!P.periodic_x || (x >= 0 && x + VW <= P.nx)) {
+            const T* e = (const T*)src + block_index((long long)y * P.pitch + x, 9);
+#pragma unroll
+            for (int i = 0; i < 9; ++i) __pipeline_memcpy_async(d + i * PP, e + 32 * i, GB);
+        } else {
+            for (int k = 0; k < VW; ++k) {
+                const T* e = (const T*)src + block_index((long long)y * P.pitch + wrap(x + k, P.nx), 9);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) d[i * PP + k] = e[32 * i];
+            }
+        }
+    }
+    __pipeline_commit();
     // thread t's wall nodes in the wall pass: t < 2 kFmW a row wall's node in
     // this thread's column (the corners belong to the columns), the next 2 RH
     // threads a column wall's node
@@ -790,7 +833,7 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
         if (!P.periodic_y && t < 2 * kFmW) {
             const int side = t / kFmW, ly = (side ? P.ny - 1 : 0) - ry0;
             if (ly >= 0 && ly < RH && colx && (P.periodic_x || (gx > 0 && gx < P.nx - 1))) {
-                wrow = (ly + 1) * PW + lx + 1;
+                wrow = (ly + 1) * PW + lx + kFmB;
                 wside = 2 + side;
                 win = side ? -PW : PW;
                 rowS[t] = flow_wall_scalars<Store>(P, sc, (long long)(side ? P.ny - 2 : 1) * P.pitch + gx);
@@ -802,7 +845,7 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
             int yy = ry0 + ly;
             if (P.periodic_y) yy = wrap(yy, P.ny);
             if (cx >= 0 && cx < kFmW && yy >= 0 && yy < P.ny) {
-                wcol = (ly + 1) * PW + cx + 1;
+                wcol = (ly + 1) * PW + cx + kFmB;
                 wside = side;
                 win = side ? -1 : 1;
                 colS[r] = flow_wall_scalars<Store>(P, sc, (long long)yy * P.pitch + (side ? P.nx - 2 : 1));
@@ -818,6 +861,7 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
 #pragma unroll
         for (int i = 0; i < 9; ++i) s[i * PP + w] = flow_enc<Store>(hb[i] * Store::kSF);
     };
+    __pipeline_wait_prior(0);
     __syncthreads();
 
     for (int k = 0;; ++k) {
@@ -834,7 +878,7 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
 #pragma unroll
             for (int i = 0; i < 9; ++i)
                 h[i].v = make_float2(flow_dec<Store>(own[i * PP + PJ * j]), flow_dec<Store>(own[i * PP + PJ * (j + 1)]));
-            flow_collide2<Store>(P, {make_float2(ph[j], ph[j + 1])}, {make_float2(fy[j], fy[j + 1])}, h, ho[j / 2]);
+            flow_collide2<Store>(P, {make_float2(nw[j], nw[j + 1])}, {make_float2(hfy[j], hfy[j + 1])}, h, ho[j / 2]);
         }
         __syncthreads();
 #pragma unroll
@@ -851,14 +895,21 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
         __syncthreads();
         if (k + 1 == ks) break;
     }
-    const bool outx = lx >= K && lx < kFmW - K && rx0 + lx < P.nx;
+    using V = typename VecOf<GB>::V;
+    constexpr int GO = (kFmW - 2 * KX) / VW, RO = RH - 2 * K;
+    for (int q = t; q < GO * RO; q += kFmW * kFmY) {
+        const int ly = K + q / GO, c = KX + VW * (q % GO), x = rx0 + c, y = ry0 + ly;
+        if (x >= P.nx || y >= P.ny) continue;
+        const T* e = s + (ly + 1) * PW + c + kFmB;
+        T* d = (T*)dst + block_index((long long)y * P.pitch + x, 9);
+        if (x + VW <= P.nx) {
 #pragma unroll
-    for (int j = 0; j < NR; ++j) {
-        const int ly = ty + kFmY * j;
-        if (!outx || ly < K || ly >= RH - K || ry0 + ly >= P.ny) continue;
-        const long long e = block_index((long long)(ry0 + ly) * P.pitch + rx0 + lx, 9);
+            for (int i = 0; i < 9; ++i) *(V*)(d + 32 * i) = *(const V*)(e + i * PP);
+        } else {
+            for (int k = 0; x + k < P.nx; ++k)
 #pragma unroll
-        for (int i = 0; i < 9; ++i) ((T*)dst)[e + 32 * i] = own[i * PP + PJ * j];
+                for (int i = 0; i < 9; ++i) d[32 * i + k] = e[i * PP + k];
+        }
     }
 }
 
@@ -866,7 +917,7 @@ template <class Store, int K>
 cudaError_t launch_flow_multi(const StepParams& P, const void* src, void* dst, const float* phi, int phi_np,
                               const float* fb, const void* sc, int ks, int repair, cudaStream_t s)
 {
-    constexpr int ow = kFmW - 2 * K, oh = kFmH - 2 * K, smem = flow_multi_smem<Store>();
+    constexpr int ow = kFmW - 2 * fm_kx(K), oh = kFmH - 2 * K, smem = flow_multi_smem<Store>();
     if (smem > 48 * 1024) {
         const cudaError_t e =
             cudaFuncSetAttribute(k_flow_multi<Store, K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -877,17 +928,23 @@ cudaError_t launch_flow_multi(const StepParams& P, const void* src, void* dst, c
                       repair);
 }
 
-// Steps per launch for n >= 2 flow steps: a launch costs about its steps plus
-// 8 of them for loading, the walls' scalars and storing (1.12 M nodes, FP32:
-// 49 us for 4 steps; one step per launch took 16 us), over the share of the
-// region that a ring of K nodes leaves to write.
-inline int flow_multi_k(int n)
+// Steps per launch for n >= 2 flow steps on an nx x ny grid: a launch costs about
+// its steps plus 8 of them for loading, the walls' scalars and storing, once for
+// each wave of two CTAs per SM that the regions fill (15 flow steps at 1024^2: K =
+// 4 fills 3 waves and K = 5 four, 818 and 834 us per four coupled steps; at 100^2,
+// one wave, 222 and 205 us).
+inline int flow_multi_k(int n, int nx, int ny)
 {
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int best = 2;
-    double least = 0.0;
+    long long least = 0;
     for (int K : {2, 4, 5}) {
-        const double cost = (8.0 * ((n + K - 1) / K) + n) / ((kFmW - 2 * K) * (kFmH - 2 * K));
-        if (least == 0.0 || cost < least) {
+        const int ow = kFmW - 2 * fm_kx(K), oh = kFmH - 2 * K;
+        const long long tiles = (long long)((nx + ow - 1) / ow) * ((ny + oh - 1) / oh);
+        const long long cost = (tiles + 2 * sms - 1) / (2 * sms) * (8 * ((n + K - 1) / K) + n);
+        if (least == 0 || cost < least) {
             least = cost;
             best = K;
         }
@@ -909,7 +966,7 @@ cudaError_t flow_chain(const StepParams& P, int n, const void* sc, void* const f
         *cf = 1 - *cf;
         return cudaGetLastError();
     }
-    const int K = flow_multi_k(n);
+    const int K = flow_multi_k(n, P.nx, P.ny);
     int repair = 0;
     for (int left = (n + K - 1) / K; left > 0 && e == cudaSuccess; --left) {
         const int ks = (n + left - 1) / left;
