@@ -382,7 +382,7 @@ __global__ void k_maxpool_bwd8(const bf16* __restrict__ X, int B, int H, int W, 
 // pooled layer and the rounding for the next GEMM in one pass (as k_maxpool_bwd8
 // and k_mask_cast8, which write and read the FP32 sum in between: 86 + 46 us at
 // 1 M pixels of 32 channels against 48).  Thread layout of k_maxpool_bwd8.
-__global__ void k_pool_mask_bwd8(const bf16* __restrict__ X, int B, int H, int W, int C, int xpitch,
+__global__ void __launch_bounds__(256, 3) k_pool_mask_bwd8(const bf16* __restrict__ X, int B, int H, int W, int C, int xpitch,
                                  const float* __restrict__ dY, const float* __restrict__ skip, int spitch,
                                  bf16* __restrict__ out)
 {
@@ -504,40 +504,57 @@ __global__ void k_proj_fwd(const bf16* __restrict__ X, int P, int C, int xpitch,
 }
 
 // The same with 16-byte loads of X (C and xpitch multiples of 8) and the
-// weights staged in shared memory: one thread per pixel.
-__global__ void k_proj_fwd_vec(const bf16* __restrict__ X, int P, int C, int xpitch, const float* __restrict__ Wt,
-                               const float* __restrict__ bias, int O, const float* __restrict__ R,
-                               float* __restrict__ Y)
+// weights staged in shared memory: one thread per pixel.  The block's outputs go
+// through shared memory, so that they are stored contiguously; with y, the
+// prediction y = x + Y / inv_out is formed from them on the way.
+__global__ void __launch_bounds__(128) k_proj_fwd_vec(const bf16* __restrict__ X, int P, int C, int xpitch,
+                                                      const float* __restrict__ Wt, const float* __restrict__ bias,
+                                                      int O, const float* __restrict__ R, float* __restrict__ Y,
+                                                      const float* x, const float* __restrict__ inv_out, float* y)
 {
     extern __shared__ float wsh[];  // O * C weights, then O biases
+    __shared__ float out[128 * 8];
+    __shared__ float so[8];
     for (int i = threadIdx.x; i < O * C; i += blockDim.x) wsh[i] = Wt[i];
     for (int i = threadIdx.x; i < O; i += blockDim.x) wsh[O * C + i] = bias[i];
+    if (y && threadIdx.x < O) so[threadIdx.x] = 1.0f / inv_out[threadIdx.x];
     __syncthreads();
-    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (p >= P) return;
-    float acc[8];
+    const int p0 = blockIdx.x * 128, p = p0 + threadIdx.x;
+    if (p < P) {
+        float acc[8];
 #pragma unroll
-    for (int o = 0; o < 8; ++o) acc[o] = o < O ? wsh[O * C + o] + (R ? R[p * O + o] : 0.0f) : 0.0f;
-    const uint4* xp = (const uint4*)(X + p * xpitch);
-    for (int c8 = 0; c8 < C / 8; ++c8) {
-        const uint4 q = xp[c8];
-        const __nv_bfloat162* h = (const __nv_bfloat162*)&q;
-        float xv[8];
+        for (int o = 0; o < 8; ++o) acc[o] = o < O ? wsh[O * C + o] + (R ? R[(long long)p * O + o] : 0.0f) : 0.0f;
+        const uint4* xp = (const uint4*)(X + (long long)p * xpitch);
+        for (int c8 = 0; c8 < C / 8; ++c8) {
+            const uint4 q = xp[c8];
+            const __nv_bfloat162* h = (const __nv_bfloat162*)&q;
+            float xv[8];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float2 f = __bfloat1622float2(h[j]);
-            xv[2 * j] = f.x;
-            xv[2 * j + 1] = f.y;
+            for (int j = 0; j < 4; ++j) {
+                const float2 f = __bfloat1622float2(h[j]);
+                xv[2 * j] = f.x;
+                xv[2 * j + 1] = f.y;
+            }
+#pragma unroll
+            for (int o = 0; o < 8; ++o) {
+                if (o >= O) break;
+                const float* w = wsh + o * C + c8 * 8;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[o] += xv[j] * w[j];
+            }
         }
 #pragma unroll
-        for (int o = 0; o < 8; ++o) {
-            if (o >= O) break;
-            const float* w = wsh + o * C + c8 * 8;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[o] += xv[j] * w[j];
-        }
+        for (int o = 0; o < 8; ++o)
+            if (o < O) out[threadIdx.x * O + o] = acc[o];
     }
-    for (int o = 0; o < O; ++o) Y[p * O + o] = acc[o];
+    __syncthreads();
+    const int n = min(128, P - p0) * O;
+    const long long e0 = (long long)p0 * O;
+    for (int i = threadIdx.x; i < n; i += 128) {
+        const float v = out[i];
+        Y[e0 + i] = v;
+        if (y) y[e0 + i] = x[e0 + i] + v * so[i % O];
+    }
 }
 
 // dX[p][c] = sum_o dY[p][o] Wt[o][c] (FP32, pitch dpitch).
@@ -846,13 +863,10 @@ __global__ void k_colsum_part8(const bf16* __restrict__ g, long long rows, int C
 #pragma unroll
     for (int k = 0; k < 8; ++k) sm[threadIdx.x][k] = acc[k];
     __syncthreads();
-    if (threadIdx.x < G) {
-        float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int l = 0; l < lanes; ++l)
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] += sm[l * G + threadIdx.x][k];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) part[(long long)blockIdx.x * C + 8 * threadIdx.x + k] = v[k];
+    for (int c = threadIdx.x; c < C; c += 128) {  // a thread per column
+        float v = 0.0f;
+        for (int l = 0; l < lanes; ++l) v += sm[l * G + (c >> 3)][c & 7];
+        part[(long long)blockIdx.x * C + c] = v;
     }
 }
 
@@ -909,32 +923,53 @@ __global__ void __launch_bounds__(1024) k_sum_one(const float* __restrict__ part
     if (threadIdx.x == 0) out[0] = sm[0];
 }
 
-// Weighted squared error: d[i] = pred - target, weight w = 1 + alpha max(0,
-// 1 - phi^2) with phi = x[pixel * F] the phase field of the input at the
-// element's pixel (w = 1 without x); per-block partial sums of w d^2 and the
-// gradient 2 w d / n.
+// Squared error: d[i] = pred - target; per-block partial sums of w d^2 and the
+// gradient 2 w d / n, with w = 1.  INC: target holds the fields K steps on, and
+// the error is taken against the increment (target - x) * inv_out[field] in output
+// units, rounded as if it were stored; where alpha != 0 its weight is w = 1 +
+// alpha max(0, 1 - phi^2) with phi = x[pixel * F] the phase field of the input.
+template <bool INC>
 __global__ void k_mse(const float* __restrict__ pred, const float* __restrict__ target, long long n,
-                      const float* __restrict__ x, int F, float alpha, float* __restrict__ grad,
-                      float* __restrict__ part)
+                      const float* __restrict__ x, int F, float alpha, const float* __restrict__ inv_out,
+                      float* __restrict__ grad, float* __restrict__ part)
 {
     __shared__ float sm[256];
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    float d = 0.0f, w = 1.0f;
-    if (i < n) {
-        d = pred[i] - target[i];
-        if (x) {
-            const float phi = x[(i / F) * F];
-            w = 1.0f + alpha * fmaxf(0.0f, 1.0f - phi * phi);
-        }
-        grad[i] = 2.0f * w * d / (float)n;
-    }
-    sm[threadIdx.x] = w * d * d;
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-        if (threadIdx.x < s) sm[threadIdx.x] += sm[threadIdx.x + s];
+    __shared__ float io[8];
+    if (INC) {
+        if (threadIdx.x < F) io[threadIdx.x] = inv_out[threadIdx.x];
         __syncthreads();
     }
-    if (threadIdx.x == 0) part[blockIdx.x] = sm[0];
+    const long long i0 = blockIdx.x * 256LL, i = i0 + threadIdx.x;
+    float d = 0.0f, w = 1.0f;
+    if (i < n) {
+        float t = target[i];
+        if (INC) {
+            const long long p0 = i0 / F;  // the block's first pixel; the division below is short
+            const int r = (int)(i0 - p0 * F) + threadIdx.x, dp = r / F;
+            t = __fmul_rn(t - x[i], io[r - dp * F]);
+            if (alpha != 0.0f) {
+                const float phi = x[(p0 + dp) * F];
+                w = 1.0f + alpha * fmaxf(0.0f, 1.0f - phi * phi);
+            }
+        }
+        d = pred[i] - t;
+        grad[i] = 2.0f * w * d / (float)n;
+    }
+    // a tree over the block's values: 128, 64 and 32 apart through shared
+    // memory, then by shuffles
+    float v = w * d * d;
+    sm[threadIdx.x] = v;
+    __syncthreads();
+#pragma unroll
+    for (int s = 128; s >= 32; s >>= 1) {
+        if (threadIdx.x < s) sm[threadIdx.x] = v = v + sm[threadIdx.x + s];
+        __syncthreads();
+    }
+    if (threadIdx.x < 32) {
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
+        if (threadIdx.x == 0) part[blockIdx.x] = v;
+    }
 }
 
 // Adam with bias correction on FP32 master weights; writes the BF16 copy.
@@ -988,12 +1023,17 @@ __global__ void k_adam4(float4* __restrict__ w, const float4* __restrict__ g, fl
 __global__ void k_pack_px(const float* __restrict__ f, long long P, int F, const float* __restrict__ mean,
                           const float* __restrict__ inv_std, bf16* __restrict__ X, int cpitch)
 {
-    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    // the block's fields are read contiguously, then taken pixel by pixel
+    __shared__ float in[256 * 8];
+    const long long p0 = blockIdx.x * 256LL, p = p0 + threadIdx.x;
+    const int n = (int)(P - p0 < 256 ? P - p0 : 256) * F;
+    for (int i = threadIdx.x; i < n; i += 256) in[i] = f[p0 * F + i];
+    __syncthreads();
     if (p >= P) return;
     __nv_bfloat162 h[4];
     float v[8];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) v[c] = c < F ? (f[p * F + c] - mean[c]) * inv_std[c] : 0.0f;
+    for (int c = 0; c < 8; ++c) v[c] = c < F ? (in[threadIdx.x * F + c] - mean[c]) * inv_std[c] : 0.0f;
 #pragma unroll
     for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
     uint4* dst = (uint4*)(X + p * cpitch);
@@ -1024,16 +1064,6 @@ __global__ void k_cast_bf16(const float* __restrict__ a, long long rows, int C, 
     const long long r = i / C;
     const int c = (int)(i - r * C);
     b[r * bpitch + c] = __float2bfloat16(a[r * apitch + c]);
-}
-
-// T[p][c] = (t[p][c] - x[p][c]) * inv_out[c]: the K-step increment in the
-// network's output units.
-__global__ void k_increment(const float* __restrict__ t, const float* __restrict__ x, long long P, int F,
-                            const float* __restrict__ inv_out, float* __restrict__ T)
-{
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= P * F) return;
-    T[i] = (t[i] - x[i]) * inv_out[(int)(i % F)];
 }
 
 // y[p][c] = x[p][c] + Y[p][c] / inv_out[c]; a block covers a contiguous run
@@ -1168,14 +1198,16 @@ cudaError_t shuffle_bwd(const void* dY, bool dy_fp32, int ypitch, int c0, int B,
 }
 
 cudaError_t proj_fwd(const void* X, int P, int C, int xpitch, const float* Wt, const float* bias, int O,
-                     const float* R, float* Y, cudaStream_t s)
+                     const float* R, float* Y, cudaStream_t s, const float* x, const float* inv_out, float* y)
 {
     if (O > 8) return cudaErrorInvalidValue;
     const size_t sh = (size_t)(O * C + O) * sizeof(float);
-    if (C % 8 == 0 && xpitch % 8 == 0 && ((uintptr_t)X & 15) == 0 && sh <= 48 * 1024)
-        k_proj_fwd_vec<<<blocks(P, 128), 128, sh, s>>>((const bf16*)X, P, C, xpitch, Wt, bias, O, R, Y);
-    else
+    if (C % 8 == 0 && xpitch % 8 == 0 && ((uintptr_t)X & 15) == 0 && sh <= 43 * 1024)
+        k_proj_fwd_vec<<<blocks(P, 128), 128, sh, s>>>((const bf16*)X, P, C, xpitch, Wt, bias, O, R, Y, x, inv_out, y);
+    else {
         k_proj_fwd<<<blocks(P), 256, 0, s>>>((const bf16*)X, P, C, xpitch, Wt, bias, O, R, Y);
+        if (y) return add_increment(Y, x, P, O, inv_out, y, s);
+    }
     return cudaGetLastError();
 }
 
@@ -1317,10 +1349,20 @@ cudaError_t colsum_part(const void* g, bool g_fp32, long long rows, int C, int p
 }
 
 cudaError_t mse(const float* pred, const float* target, long long n, float* grad, float* loss, float* part,
-                cudaStream_t s, const float* x, int F, float alpha)
+                cudaStream_t s)
 {
     const int nb = (int)((n + 255) / 256);
-    k_mse<<<nb, 256, 0, s>>>(pred, target, n, x, F, alpha, grad, part);
+    k_mse<false><<<nb, 256, 0, s>>>(pred, target, n, nullptr, 1, 0.0f, nullptr, grad, part);
+    k_sum_one<<<1, 1024, 0, s>>>(part, nb, loss);
+    return cudaGetLastError();
+}
+
+cudaError_t mse_increment(const float* Y, const float* t, const float* x, long long P, int F, const float* inv_out,
+                          float alpha, float* grad, float* loss, float* part, cudaStream_t s)
+{
+    const long long n = P * F;
+    const int nb = (int)((n + 255) / 256);
+    k_mse<true><<<nb, 256, 0, s>>>(Y, t, n, x, F, alpha, inv_out, grad, part);
     k_sum_one<<<1, 1024, 0, s>>>(part, nb, loss);
     return cudaGetLastError();
 }
@@ -1352,13 +1394,6 @@ cudaError_t unpack(const float* Y, long long P, int F, const float* mean, const 
                    cudaStream_t s)
 {
     k_unpack<<<blocks(P * F), 256, 0, s>>>(Y, P, F, mean, inv_std, f);
-    return cudaGetLastError();
-}
-
-cudaError_t increment(const float* t, const float* x, long long P, int F, const float* inv_out, float* T,
-                      cudaStream_t s)
-{
-    k_increment<<<blocks(P * F), 256, 0, s>>>(t, x, P, F, inv_out, T);
     return cudaGetLastError();
 }
 

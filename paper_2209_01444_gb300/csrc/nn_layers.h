@@ -21,7 +21,8 @@ cudaError_t shuffle_fwd(const void* U, int B, int H, int W, int C, void* Y, int 
 cudaError_t shuffle_bwd(const void* dY, bool dy_fp32, int ypitch, int c0, int B, int H, int W, int C, void* dU,
                         cudaStream_t s);
 cudaError_t proj_fwd(const void* X, int P, int C, int xpitch, const float* Wt, const float* bias, int O,
-                     const float* R, float* Y, cudaStream_t s);
+                     const float* R, float* Y, cudaStream_t s, const float* x = nullptr,
+                     const float* inv_out = nullptr, float* y = nullptr);  // y: also x + Y / inv_out
 cudaError_t proj_bwd(const float* dY, const void* X, int P, int C, int xpitch, const float* Wt, int O, float* dX,
                      int dpitch, float* dW, float* db, float* part, int part_blocks, cudaStream_t s,
                      void* dXb = nullptr);  // dXb: BF16 [P][C], dX masked by X > 0 (dX is then scratch)
@@ -47,19 +48,20 @@ cudaError_t colsum(const void* g, bool g_fp32, long long rows, int C, int pitch,
 // columns are then added over the blocks in k_sum_parts' order.
 cudaError_t colsum_part(const void* g, bool g_fp32, long long rows, int C, int pitch, float* part, int part_blocks,
                         int* nblocks, cudaStream_t s);
-// Mean of w (pred - target)^2 over n elements and its gradient; with x (the
-// network input, F fields per pixel, phase field first) each pixel's
-// elements are weighted by w = 1 + alpha max(0, 1 - phi^2), else w = 1.
+// Mean of (pred - target)^2 over n elements and its gradient.
 cudaError_t mse(const float* pred, const float* target, long long n, float* grad, float* loss, float* part,
-                cudaStream_t s, const float* x = nullptr, int F = 1, float alpha = 0.0f);
+                cudaStream_t s);
+// The same against the increment (t - x) * inv_out of P pixels of F fields (phase
+// field first); where alpha != 0 a pixel's elements are weighted by
+// 1 + alpha max(0, 1 - phi^2), phi of x.
+cudaError_t mse_increment(const float* Y, const float* t, const float* x, long long P, int F, const float* inv_out,
+                          float alpha, float* grad, float* loss, float* part, cudaStream_t s);
 cudaError_t adam(float* w, const float* g, float* m, float* v, long long n, float lr, float b1, float b2, float eps,
                  int t, void* wb, cudaStream_t s);
 cudaError_t pack(const float* f, long long P, int F, const float* mean, const float* inv_std, void* X, int cpitch,
                  float* R, cudaStream_t s);
 cudaError_t unpack(const float* Y, long long P, int F, const float* mean, const float* inv_std, float* f,
                    cudaStream_t s);
-cudaError_t increment(const float* t, const float* x, long long P, int F, const float* inv_out, float* T,
-                      cudaStream_t s);
 cudaError_t add_increment(const float* Y, const float* x, long long P, int F, const float* inv_out, float* y,
                           cudaStream_t s);
 cudaError_t cast_bf16(const float* a, long long rows, int C, int apitch, void* b, int bpitch, cudaStream_t s);

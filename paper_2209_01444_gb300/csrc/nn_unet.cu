@@ -98,7 +98,7 @@ struct lbm_unet {
     float iface_w = 0.0f;  // interface weight of the loss (lbm_unet_set_loss_weight)
     std::vector<float> norm_h;  // host copy: mean, std_in, std_out (F each)
     bf16* x0 = nullptr;
-    float *Y = nullptr, *T = nullptr, *G = nullptr;
+    float *Y = nullptr, *G = nullptr;
     float *loss = nullptr, *part = nullptr;
     bf16 *col = nullptr, *colT = nullptr, *tA = nullptr;
     bf16 *gA = nullptr, *gB = nullptr, *dU = nullptr;
@@ -259,7 +259,6 @@ cudaError_t allocate(lbm_unet* u)
     const long long P0 = u->P0;
     UN_ALLOC(u->x0, P0 * kX0Pitch);
     UN_ALLOC(u->Y, P0 * u->F);
-    UN_ALLOC(u->T, P0 * u->F);
     UN_ALLOC(u->G, P0 * u->F);
     UN_ALLOC(u->loss, 4);
     const long long part_n = std::max<long long>((long long)kPartBlocks * (u->base + 1) * 8, P0 * u->F / 256 + 2);
@@ -497,7 +496,8 @@ cudaError_t conv_bwd(lbm_unet* u, const Level& v, const Conv& cv, const bf16* in
 }
 
 
-cudaError_t forward(lbm_unet* u, const float* x)
+// The network's output for the fields x, and with y the prediction.
+cudaError_t forward(lbm_unet* u, const float* x, float* y = nullptr)
 {
     cudaError_t e;
     if ((e = nn::pack(x, u->P0, u->F, u->mean, u->inv_std, u->x0, kX0Pitch, nullptr, u->s))) return e;
@@ -528,7 +528,7 @@ cudaError_t forward(lbm_unet* u, const float* x)
     }
     const bf16* top = L > 1 ? u->lv[0].dD : u->lv[0].s;
     return nn::proj_fwd(top, (int)u->P0, u->base, u->base, u->w + u->out_w, u->w + u->out_b, u->F, nullptr, u->Y,
-                        u->s);
+                        u->s, x, u->inv_out, y);
 }
 
 // Loss and parameter gradients for the target t (physical units); forward(x) ran.
@@ -537,10 +537,7 @@ cudaError_t backward(lbm_unet* u, const float* x, const float* t)
     cudaError_t e;
     const long long P0 = u->P0;
     const int L = u->L, F = u->F, w0 = u->base;
-    if ((e = nn::increment(t, x, P0, F, u->inv_out, u->T, u->s))) return e;
-    if ((e = nn::mse(u->Y, u->T, P0 * F, u->G, u->loss, u->part, u->s, u->iface_w != 0.0f ? x : nullptr, F,
-                     u->iface_w)))
-        return e;
+    if ((e = nn::mse_increment(u->Y, t, x, P0, F, u->inv_out, u->iface_w, u->G, u->loss, u->part, u->s))) return e;
     const bf16* top = L > 1 ? u->lv[0].dD : u->lv[0].s;
     if ((e = nn::proj_bwd(u->G, top, (int)P0, w0, w0, u->w + u->out_w, F, u->g32, w0, u->g + u->out_w, u->g + u->out_b,
                           u->part, kPartBlocks, u->s, u->gA)))
@@ -802,8 +799,7 @@ int lbm_unet_forward(lbm_unet* u, const float* x, float* y)
 {
     trace::Range range("lbm_unet_forward");
     if (!u || !x) return LBM_EINVAL;
-    UN_CHECK(u, forward(u, x));
-    if (y) UN_CHECK(u, nn::add_increment(u->Y, x, u->P0, u->F, u->inv_out, y, u->s));
+    UN_CHECK(u, forward(u, x, y));
     return LBM_OK;
 }
 
