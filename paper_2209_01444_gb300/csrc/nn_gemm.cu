@@ -555,18 +555,10 @@ constexpr int kWsGemmThreads = 64 + 32 * kWsEpi;
 
 __device__ __forceinline__ bool mbar_wait_abort(uint64_t* bar, uint32_t parity, volatile int* abort_flag)
 {
-    const uint32_t addr = smem_u32(bar);
+    if (mbar_try(bar, parity)) return true;  // before the clock is read
     const unsigned long long t0 = global_ns();
     for (uint32_t it = 0;; ++it) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\t"
-            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(addr), "r"(parity)
-            : "memory");
-        if (done) return true;
+        if (mbar_try(bar, parity)) return true;
         if ((it & 63) == 63) {
             if (*abort_flag) return false;
             if (global_ns() - t0 > kWaitNs) {
@@ -603,6 +595,7 @@ __device__ __forceinline__ uint32_t elect_lane()
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
                                                unsigned long long lim = kWaitNs)
 {
+    if (lim != 0 && __all_sync(0xffffffffu, mbar_try(bar, parity))) return true;  // before the clock is read
     const unsigned long long t0 = global_ns();
     for (uint32_t it = 0;; ++it) {
         if (lim != 0 && __all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
@@ -669,6 +662,49 @@ __device__ __forceinline__ void tmem_wait32(uint32_t (&r)[32])
                    "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
                  :
                  : "memory");
+}
+
+// 32 columns from col on of output row `row`: the ReLU mask (mp null: none; mk
+// loaded where `all`, the columns lying inside the matrix), then the stores, of the
+// two halves at off0 and off1 of D.
+template <bool OUT_BF16>
+__device__ __forceinline__ void store_unit(float (&v)[32], const Mask16 (&mk)[2], const __nv_bfloat16* __restrict__ mp,
+                                           bool all, long long row, int col, int N, void* __restrict__ D,
+                                           long long off0, long long off1, const ShuffleGeo& sh)
+{
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        float(&w)[16] = *(float(*)[16])(v + 16 * k);
+        const int left = N - col - 16 * k;
+        const long long off = k ? off1 : off0;
+        if (left <= 0) break;
+        if (mp) apply_relu_mask(w, mk[k], mp + 16 * k, all, left);
+        if (!OUT_BF16 && sh.dU && col + 16 * k >= sh.c) {
+            const int x = (int)row % sh.Wf, y = ((int)row / sh.Wf) % sh.Hf, b = (int)row / (sh.Wf * sh.Hf);
+            const long long q = ((long long)b * (sh.Hf / 2) + y / 2) * (sh.Wf / 2) + x / 2;
+            __nv_bfloat162 h[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(w[2 * j], w[2 * j + 1]);
+            store32(sh.dU + (q * 4 + (y & 1) * 2 + (x & 1)) * sh.c + col + 16 * k - sh.c, (const uint32_t*)h);
+        } else if (left < 16) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                if (j >= left) break;
+                if (OUT_BF16)
+                    ((__nv_bfloat16*)D)[off + j] = __float2bfloat16_rn(w[j]);
+                else
+                    ((float*)D)[off + j] = w[j];
+            }
+        } else if (OUT_BF16) {
+            __nv_bfloat162 h[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(w[2 * j], w[2 * j + 1]);
+            store32((__nv_bfloat16*)D + off, (const uint32_t*)h);
+        } else {
+            store32((float*)D + off, (const uint32_t*)w);
+            store32((float*)D + off + 8, (const uint32_t*)(w + 8));
+        }
+    }
 }
 
 // Low and high words of a tile's descriptor; a tile `bytes` further has
@@ -912,38 +948,7 @@ __global__ void __launch_bounds__(kWsGemmThreads, 1)
                         off[k] = qq * ldd + sh.c0 + co;
                     }
                 }
-#pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    float(&w)[16] = *(float(*)[16])(v + 16 * k);
-                    const int left = N - col - 16 * k;
-                    if (left <= 0) break;
-                    if (mrow) apply_relu_mask(w, mk[k], mp + 16 * k, all, left);
-                    if (!OUT_BF16 && sh.dU && col + 16 * k >= sh.c) {
-                        const int x = row % sh.Wf, y = (row / sh.Wf) % sh.Hf, b = row / (sh.Wf * sh.Hf);
-                        const long long q = ((long long)b * (sh.Hf / 2) + y / 2) * (sh.Wf / 2) + x / 2;
-                        __nv_bfloat162 h[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(w[2 * j], w[2 * j + 1]);
-                        store32(sh.dU + (q * 4 + (y & 1) * 2 + (x & 1)) * sh.c + col + 16 * k - sh.c, (const uint32_t*)h);
-                    } else if (left < 16) {
-#pragma unroll
-                        for (int j = 0; j < 16; ++j) {
-                            if (j >= left) break;
-                            if (OUT_BF16)
-                                ((__nv_bfloat16*)D)[off[k] + j] = __float2bfloat16_rn(w[j]);
-                            else
-                                ((float*)D)[off[k] + j] = w[j];
-                        }
-                    } else if (OUT_BF16) {
-                        __nv_bfloat162 h[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) h[j] = __floats2bfloat162_rn(w[2 * j], w[2 * j + 1]);
-                        store32((__nv_bfloat16*)D + off[k], (const uint32_t*)h);
-                    } else {
-                        store32((float*)D + off[k], (const uint32_t*)w);
-                        store32((float*)D + off[k] + 8, (const uint32_t*)(w + 8));
-                    }
-                }
+                store_unit<OUT_BF16>(v, mk, mp, all, row, col, N, D, off[0], off[1], sh);
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             mbar_arrive(&acc_empty[acc]);
@@ -967,6 +972,7 @@ __global__ void __launch_bounds__(kWsGemmThreads, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
+#include "nn_conv_roll.cuh"
 #include "nn_wgrad.cuh"
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
@@ -1062,6 +1068,18 @@ cudaError_t launch_ws_mt(const CUtensorMap& a, const CUtensorMap& b, void* D, co
     const int grid = tiles < sms * per_sm ? tiles : sms * per_sm;
     k_gemm_ws<BN, OUT_BF16, BK, CONV, MT, ROW3><<<grid, kWsGemmThreads, smem, s>>>(a, b, D, bias, M, N, K, ldd, relu, geo,
                                                                                sh, tiles_m, tiles);
+    return cudaGetLastError();
+}
+
+template <int BN, bool OUT_BF16, int BK>
+cudaError_t launch_roll(const CUtensorMap& a, const CUtensorMap& b, void* D, const float* bias, int N, int ldd,
+                        int relu, int W, int H, int nx, int total, int ctas, const ShuffleGeo& sh, cudaStream_t s)
+{
+    constexpr int smem = 9 * BN * BK * 2 + roll_stages<BN, BK>() * roll_stage_bytes<BN, BK>() + 1024 + 256;
+    static_assert(smem <= 227 * 1024, "shared memory per CTA");
+    cudaError_t e = cudaFuncSetAttribute(k_conv_roll<BN, OUT_BF16, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k_conv_roll<BN, OUT_BF16, BK><<<ctas, kRollThreads, smem, s>>>(a, b, D, bias, N, ldd, relu, W, H, nx, total, sh);
     return cudaGetLastError();
 }
 
@@ -1661,7 +1679,18 @@ static cudaError_t conv3x3(const void* X, int B, int H, int W, int C, int cpitch
         bh = kBM / geo.tw;
         bb = 1;
     }
+    const long long nx = (W + kBM - 1) / kBM, total = nx * H * B;
+    // k_conv_roll where one channel block and one column tile hold everything, the
+    // last tile of a row is not mostly padding, and each SM has three tiles or more:
+    // fewer do not repay the two extra input rows and the weights each CTA loads
+    // (64 -> 64 channels, k_gemm_ws against it: 1 x 128 x 256 9.3 and 10.1 us, 1 x 256 x 256
+    // 12.3 and 12.3, 2 x 256 x 256 16.4 and 14.3; rows of 64 pixels, half a tile, 16 x 64 x
+    // 64 12.3 and 16.4; 160 pixels, 4 x 160 x 160 forward, 322 and 313)
+    const bool roll = N <= bn && bn <= 64 && C == bk && nx * kBM * 5 <= 8LL * W && total >= 3LL * sm_count() &&
+                      total <= 0x7fffffffLL;
+    row3 = row3 || roll;
     CUtensorMap ta, tb;
+    if (roll) bh = bn == 32 && bk == 32 ? roll_rows<32, 32>() : roll_rows<64, 64>();
     cudaError_t e = make_map_4d(&ta, X, B, H, W, C, cpitch, row3 ? kBM + 2 : bw, bh, bb, bk);
     if (e == cudaSuccess) e = make_map(&tb, Wm, N, 9 * C, ldw, bn, bk);
     if (e != cudaSuccess) return e;
@@ -1671,6 +1700,17 @@ static cudaError_t conv3x3(const void* X, int B, int H, int W, int C, int cpitch
     geo.cblocks = C / bk;
     geo.row3 = row3 ? 1 : 0;
     const int M = B * H * W, K = 9 * C;
+    if (roll) {
+        const int ctas = total < sm_count() ? (int)total : sm_count();
+#define NN_ROLL(BNV, BKV)                                                                                            \
+    return out_bf16 ? launch_roll<BNV, true, BKV>(ta, tb, D, bias, N, ldd, relu, W, H, (int)nx, (int)total, ctas, sh, s) \
+                    : launch_roll<BNV, false, BKV>(ta, tb, D, bias, N, ldd, relu, W, H, (int)nx, (int)total, ctas, sh, s)
+        if (bn == 32 && bk == 32) NN_ROLL(32, 32);
+        if (bn == 64 && bk == 32) NN_ROLL(64, 32);
+        if (bn == 32 && bk == 64) NN_ROLL(32, 64);
+        if (bn == 64 && bk == 64) NN_ROLL(64, 64);
+#undef NN_ROLL
+    }
     return bk == 64 ? dispatch<64, true>(bn, out_bf16, ta, tb, D, bias, M, N, K, ldd, relu ? 1 : 0, 1, 1 << 30, geo,
                                          sh, s)
                     : dispatch<32, true>(bn, out_bf16, ta, tb, D, bias, M, N, K, ldd, relu ? 1 : 0, 1, 1 << 30, geo,
