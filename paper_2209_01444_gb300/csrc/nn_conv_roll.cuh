@@ -101,6 +101,7 @@ __global__ void __launch_bounds__(kRollThreads, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
+    lbm::pdl_begin();  // after the tensor memory is taken, as in k_gemm_ws
 
     if (warp == 0) {  // ------------------------------------------- producer
         const uint32_t lead = elect_lane();

@@ -22,6 +22,7 @@
 
 #include "lbm.h"
 #include "nn_kernels.h"
+#include "pdl.cuh"
 
 namespace nn {
 
@@ -778,6 +779,8 @@ __global__ void __launch_bounds__(kWsGemmThreads, 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
+    // the next kernel may start only now: it takes tensor memory of its own, and waits
+    lbm::pdl_begin();
 
     if (warp == 0) {
         const uint32_t lead = elect_lane();
@@ -1066,8 +1069,8 @@ cudaError_t launch_ws_mt(const CUtensorMap& a, const CUtensorMap& b, void* D, co
     const int tiles_m = (Mt + kBM * MT - 1) / (kBM * MT);
     const int tiles = tiles_m * ((N + BN - 1) / BN);
     const int grid = tiles < sms * per_sm ? tiles : sms * per_sm;
-    k_gemm_ws<BN, OUT_BF16, BK, CONV, MT, ROW3><<<grid, kWsGemmThreads, smem, s>>>(a, b, D, bias, M, N, K, ldd, relu, geo,
-                                                                               sh, tiles_m, tiles);
+    lbm::launch_pdl(k_gemm_ws<BN, OUT_BF16, BK, CONV, MT, ROW3>, grid, kWsGemmThreads, smem, s, a, b, D, bias, M,
+                    N, K, ldd, relu, geo, sh, tiles_m, tiles);
     return cudaGetLastError();
 }
 
@@ -1079,7 +1082,8 @@ cudaError_t launch_roll(const CUtensorMap& a, const CUtensorMap& b, void* D, con
     static_assert(smem <= 227 * 1024, "shared memory per CTA");
     cudaError_t e = cudaFuncSetAttribute(k_conv_roll<BN, OUT_BF16, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    k_conv_roll<BN, OUT_BF16, BK><<<ctas, kRollThreads, smem, s>>>(a, b, D, bias, N, ldd, relu, W, H, nx, total, sh);
+    lbm::launch_pdl(k_conv_roll<BN, OUT_BF16, BK>, ctas, kRollThreads, smem, s, a, b, D, bias, N, ldd, relu, W, H,
+                    nx, total, sh);
     return cudaGetLastError();
 }
 
@@ -1235,6 +1239,7 @@ __global__ void k_split_reduce_t_tile(const float* __restrict__ part, int splits
 // order of the kernel named, so the results are the same bits.
 __global__ void __launch_bounds__(256) k_reduce_jobs(const ReduceJob* __restrict__ jobs, int njobs)
 {
+    lbm::pdl_begin();
     __shared__ float t[32][33];
     const int tx = threadIdx.x, ty = threadIdx.y;
     int lo = 0, hi = njobs - 1;  // the last job whose start is <= blockIdx.x
@@ -1335,7 +1340,8 @@ cudaError_t launch_wgrad(const void* X, int B, int W, int C, int cpitch, const v
     CUtensorMap tx, ty;
     if ((e = make_map_4d(&tx, X, B, g.H, W, C, cpitch, g.bk + 2, KYS, 1, CB)) != cudaSuccess) return e;
     if ((e = make_map_4d(&ty, dY, B, g.H, W, g.N, g.N, g.bk, 1, 1, BN)) != cudaSuccess) return e;
-    k_wgrad<CB, BN, KYS><<<dim3(g.ncb * g.nnb * (3 / KYS), splits), kWsThreads, smem, s>>>(tx, ty, part, g);
+    lbm::launch_pdl(k_wgrad<CB, BN, KYS>, dim3(g.ncb * g.nnb * (3 / KYS), splits), kWsThreads, smem, s, tx, ty,
+                    part, g);
     return cudaGetLastError();
 }
 
@@ -1352,7 +1358,7 @@ int reduce_job_blocks(const ReduceJob& j)
 cudaError_t reduce_jobs(const ReduceJob* jobs, int njobs, int blocks, cudaStream_t s)
 {
     if (njobs < 1) return cudaSuccess;
-    k_reduce_jobs<<<blocks, dim3(32, 8), 0, s>>>(jobs, njobs);
+    lbm::launch_pdl(k_reduce_jobs, blocks, dim3(32, 8), 0, s, jobs, njobs);
     return cudaGetLastError();
 }
 
@@ -1413,8 +1419,8 @@ static cudaError_t launch_tn(const void* A, const void* B, int M, int N, int P, 
     CUtensorMap ta, tb;
     if ((e = make_map(&ta, A, P, M, M, 64, 64)) != cudaSuccess) return e;
     if ((e = make_map(&tb, B, P, N, N, 64, BN > 32 ? 64 : 32)) != cudaSuccess) return e;
-    k_gemm_tn<BN><<<dim3((M + kBM - 1) / kBM, (N + BN - 1) / BN, splits), kWsThreads, smem, s>>>(
-        ta, tb, part, M, N, (P + 63) / 64, per);
+    lbm::launch_pdl(k_gemm_tn<BN>, dim3((M + kBM - 1) / kBM, (N + BN - 1) / BN, splits), kWsThreads, smem, s, ta,
+                    tb, part, M, N, (P + 63) / 64, per);
     return cudaGetLastError();
 }
 

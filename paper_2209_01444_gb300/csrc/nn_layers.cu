@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "nn_layers.h"
+#include "pdl.cuh"
 
 namespace nn {
 
@@ -241,6 +242,7 @@ __global__ void k_mask_cast8(const float* __restrict__ g, int gpitch, const bf16
 __global__ void k_transpose(const bf16* __restrict__ in, int rows, int cols, int ipitch, bf16* __restrict__ out,
                             int opitch)
 {
+    lbm::pdl_begin();
     __shared__ bf16 t[32][33];
     const int r0 = blockIdx.x * 32, c0 = blockIdx.y * 32;  // rows on x: up to 2^31 blocks
     for (int k = threadIdx.y; k < 32; k += 8) {
@@ -275,6 +277,7 @@ __global__ void k_maxpool_fwd(const bf16* __restrict__ X, int B, int H, int W, i
 __global__ void k_maxpool_fwd8(const bf16* __restrict__ X, int B, int H, int W, int C, int xpitch,
                                bf16* __restrict__ Y)
 {
+    lbm::pdl_begin();
     const int Ho = H / 2, Wo = W / 2, G = C / 8;
     const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;  // fewer than 2^31 groups
     if (i >= (unsigned)B * Ho * Wo * G) return;
@@ -386,6 +389,7 @@ __global__ void __launch_bounds__(256, 3) k_pool_mask_bwd8(const bf16* __restric
                                  const float* __restrict__ dY, const float* __restrict__ skip, int spitch,
                                  bf16* __restrict__ out)
 {
+    lbm::pdl_begin();
     const int Ho = H / 2, Wo = W / 2;
     const int c = 8 * threadIdx.x;
     const unsigned p = blockIdx.x * blockDim.y + threadIdx.y;  // fewer than 2^31 pixels
@@ -512,6 +516,7 @@ __global__ void __launch_bounds__(128) k_proj_fwd_vec(const bf16* __restrict__ X
                                                       int O, const float* __restrict__ R, float* __restrict__ Y,
                                                       const float* x, const float* __restrict__ inv_out, float* y)
 {
+    lbm::pdl_begin();
     extern __shared__ float wsh[];  // O * C weights, then O biases
     __shared__ float out[128 * 8];
     __shared__ float so[8];
@@ -663,6 +668,7 @@ __global__ void __launch_bounds__(256) k_proj_bwd_w8(const float* __restrict__ d
                                                      int C, int xpitch, int chunk, float* __restrict__ part,
                                                      const float* __restrict__ Wt, bf16* __restrict__ dXb)
 {
+    lbm::pdl_begin();
     __shared__ float sm[8][8][O * 9];  // [warp][group][o * 9 + k], k = 8: the bias
     __shared__ float wsh[O * 64];      // the weights (C <= 64)
     if (dXb) {
@@ -764,6 +770,7 @@ __global__ void k_flip3x3(const bf16* __restrict__ W, int cout, int cin, bf16* _
 // jobs, scanned in order).
 __global__ void k_flip3x3_many(const FlipJob* __restrict__ jobs, int njobs)
 {
+    lbm::pdl_begin();
     __shared__ bf16 t[32][33];
     const long long i = blockIdx.x;
     int j = 0;
@@ -791,6 +798,7 @@ __global__ void k_flip3x3_many(const FlipJob* __restrict__ jobs, int njobs)
 // kernel of a convolution whose input carries cin_pad channels, the extra ones zero.
 __global__ void k_pad_conv3x3(const bf16* __restrict__ W, int cout, int cin, int cin_pad, bf16* __restrict__ Wp)
 {
+    lbm::pdl_begin();
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= (long long)cout * 9 * cin_pad) return;
     const int ci = (int)(i % cin_pad);
@@ -835,6 +843,7 @@ __global__ void k_colsum_part(const G* __restrict__ g, long long rows, int C, in
 __global__ void k_colsum_part8(const bf16* __restrict__ g, long long rows, int C, int pitch, int chunk,
                                float* __restrict__ part)
 {
+    lbm::pdl_begin();
     __shared__ float sm[128][8];
     const int G = C >> 3;
     const int lanes = 128 / G;
@@ -875,6 +884,7 @@ __global__ void k_colsum_part8(const bf16* __restrict__ g, long long rows, int C
 __global__ void k_proj_sum(const float* __restrict__ part, int nb, int O, int C, float* __restrict__ dW,
                            float* __restrict__ db)
 {
+    lbm::pdl_begin();
     const int s = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     const int slots = O * (C + 1);
@@ -911,6 +921,7 @@ __global__ void k_sum_parts(const float* __restrict__ part, int nb, int slots, f
 // reproducible).
 __global__ void __launch_bounds__(1024) k_sum_one(const float* __restrict__ part, int nb, float* __restrict__ out)
 {
+    lbm::pdl_begin();
     __shared__ float sm[1024];
     float acc = 0.0f;
     for (int b = threadIdx.x; b < nb; b += 1024) acc += part[b];
@@ -933,6 +944,7 @@ __global__ void k_mse(const float* __restrict__ pred, const float* __restrict__ 
                       const float* __restrict__ x, int F, float alpha, const float* __restrict__ inv_out,
                       float* __restrict__ grad, float* __restrict__ part)
 {
+    lbm::pdl_begin();
     __shared__ float sm[256];
     __shared__ float io[8];
     if (INC) {
@@ -994,6 +1006,7 @@ __global__ void k_adam4(float4* __restrict__ w, const float4* __restrict__ g, fl
                         float4* __restrict__ v, long long n4, float lr, float b1, float b2, float eps, float c1,
                         float c2, uint2* __restrict__ wb)
 {
+    lbm::pdl_begin();
     const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (i >= n4) return;
     const float4 g4 = g[i];
@@ -1023,6 +1036,7 @@ __global__ void k_adam4(float4* __restrict__ w, const float4* __restrict__ g, fl
 __global__ void k_pack_px(const float* __restrict__ f, long long P, int F, const float* __restrict__ mean,
                           const float* __restrict__ inv_std, bf16* __restrict__ X, int cpitch)
 {
+    lbm::pdl_begin();
     // the block's fields are read contiguously, then taken pixel by pixel
     __shared__ float in[256 * 8];
     const long long p0 = blockIdx.x * 256LL, p = p0 + threadIdx.x;
@@ -1119,7 +1133,7 @@ cudaError_t transpose(const void* in, int rows, int cols, int ipitch, void* out,
 {
     if ((cols + 31) / 32 > 65535) return cudaErrorInvalidValue;
     dim3 grid((rows + 31) / 32, (cols + 31) / 32), block(32, 8);
-    k_transpose<<<grid, block, 0, s>>>((const bf16*)in, rows, cols, ipitch, (bf16*)out, opitch);
+    lbm::launch_pdl(k_transpose, grid, block, 0, s, (const bf16*)in, rows, cols, ipitch, (bf16*)out, opitch);
     return cudaGetLastError();
 }
 
@@ -1128,8 +1142,8 @@ cudaError_t maxpool_fwd(const void* X, int B, int H, int W, int C, int xpitch, v
     if (H % 2 || W % 2) return cudaErrorInvalidValue;
     if (C % 8 == 0 && xpitch % 8 == 0 && (((uintptr_t)X | (uintptr_t)Y) & 15) == 0 &&
         (long long)B * (H / 2) * (W / 2) * (C / 8) < 0x7fffffffLL - 256)
-        k_maxpool_fwd8<<<blocks((long long)B * (H / 2) * (W / 2) * (C / 8)), 256, 0, s>>>((const bf16*)X, B, H, W, C,
-                                                                                        xpitch, (bf16*)Y);
+        lbm::launch_pdl(k_maxpool_fwd8, blocks((long long)B * (H / 2) * (W / 2) * (C / 8)), 256, 0, s,
+                        (const bf16*)X, B, H, W, C, xpitch, (bf16*)Y);
     else
         k_maxpool_fwd<<<blocks((long long)B * (H / 2) * (W / 2) * C), 256, 0, s>>>((const bf16*)X, B, H, W, C, xpitch,
                                                                                  (bf16*)Y);
@@ -1163,8 +1177,8 @@ cudaError_t pool_mask_bwd(const void* X, int B, int H, int W, int C, int xpitch,
         return e != cudaSuccess ? e : mask_cast(skip, spitch, X, xpitch, (long long)B * H * W, C, out, C, s);
     }
     const dim3 b(C / 8, 256 / (C / 8));
-    k_pool_mask_bwd8<<<(unsigned)((Po + b.y - 1) / b.y), b, 0, s>>>((const bf16*)X, B, H, W, C, xpitch, dY, skip, spitch,
-                                                                    (bf16*)out);
+    lbm::launch_pdl(k_pool_mask_bwd8, (unsigned)((Po + b.y - 1) / b.y), b, 0, s, (const bf16*)X, B, H, W, C,
+                    xpitch, dY, skip, spitch, (bf16*)out);
     return cudaGetLastError();
 }
 
@@ -1203,7 +1217,8 @@ cudaError_t proj_fwd(const void* X, int P, int C, int xpitch, const float* Wt, c
     if (O > 8) return cudaErrorInvalidValue;
     const size_t sh = (size_t)(O * C + O) * sizeof(float);
     if (C % 8 == 0 && xpitch % 8 == 0 && ((uintptr_t)X & 15) == 0 && sh <= 43 * 1024)
-        k_proj_fwd_vec<<<blocks(P, 128), 128, sh, s>>>((const bf16*)X, P, C, xpitch, Wt, bias, O, R, Y, x, inv_out, y);
+        lbm::launch_pdl(k_proj_fwd_vec, blocks(P, 128), 128, sh, s, (const bf16*)X, P, C, xpitch, Wt, bias, O, R,
+                        Y, x, inv_out, y);
     else {
         k_proj_fwd<<<blocks(P), 256, 0, s>>>((const bf16*)X, P, C, xpitch, Wt, bias, O, R, Y);
         if (y) return add_increment(Y, x, P, O, inv_out, y, s);
@@ -1232,7 +1247,8 @@ cudaError_t proj_bwd(const float* dY, const void* X, int P, int C, int xpitch, c
     if (vec) {
         switch (O) {
 #define NN_PROJ_W8(OV) \
-    case OV: k_proj_bwd_w8<OV><<<nb, 256, 0, s>>>(dY, (const bf16*)X, P, C, xpitch, chunk, part, Wt, (bf16*)dXb); break;
+    case OV: lbm::launch_pdl(k_proj_bwd_w8<OV>, nb, 256, 0, s, dY, (const bf16*)X, P, C, xpitch, chunk, part, Wt, \
+                             (bf16*)dXb); break;
             NN_PROJ_W8(1)
             NN_PROJ_W8(2)
             NN_PROJ_W8(3)
@@ -1249,7 +1265,7 @@ cudaError_t proj_bwd(const float* dY, const void* X, int P, int C, int xpitch, c
         k_proj_bwd_w<<<nb, 128, 0, s>>>(dY, (const bf16*)X, P, C, xpitch, O, chunk, part);
     }
     const int slots = O * (C + 1);
-    k_proj_sum<<<(unsigned)((slots + 7) / 8), 256, 0, s>>>(part, nb, O, C, dW, db);
+    lbm::launch_pdl(k_proj_sum, (unsigned)((slots + 7) / 8), 256, 0, s, part, nb, O, C, dW, db);
     if (dXb && !vec) return mask_cast(dX, dpitch, X, xpitch, P, C, dXb, C, s);
     return cudaGetLastError();
 }
@@ -1297,14 +1313,15 @@ cudaError_t mask_cast(const float* g, int gpitch, const void* y, int ypitch, lon
 cudaError_t pad_conv3x3(const void* W, int cout, int cin, int cin_pad, void* Wp, cudaStream_t s)
 {
     if (cin_pad < cin) return cudaErrorInvalidValue;
-    k_pad_conv3x3<<<blocks((long long)cout * 9 * cin_pad), 256, 0, s>>>((const bf16*)W, cout, cin, cin_pad, (bf16*)Wp);
+    lbm::launch_pdl(k_pad_conv3x3, blocks((long long)cout * 9 * cin_pad), 256, 0, s, (const bf16*)W, cout, cin,
+                    cin_pad, (bf16*)Wp);
     return cudaGetLastError();
 }
 
 cudaError_t flip3x3_many(const FlipJob* jobs, int njobs, long long total, cudaStream_t s)
 {
     if (njobs < 1 || total < 1) return cudaSuccess;
-    k_flip3x3_many<<<(unsigned)total, dim3(32, 8), 0, s>>>(jobs, njobs);
+    lbm::launch_pdl(k_flip3x3_many, (unsigned)total, dim3(32, 8), 0, s, jobs, njobs);
     return cudaGetLastError();
 }
 
@@ -1342,7 +1359,7 @@ cudaError_t colsum_part(const void* g, bool g_fp32, long long rows, int C, int p
     if (g_fp32)
         k_colsum_part<float><<<nb, 128, 0, s>>>((const float*)g, rows, C, pitch, (int)chunk, part);
     else if (vec)
-        k_colsum_part8<<<nb, 128, 0, s>>>((const bf16*)g, rows, C, pitch, (int)chunk, part);
+        lbm::launch_pdl(k_colsum_part8, nb, 128, 0, s, (const bf16*)g, rows, C, pitch, (int)chunk, part);
     else
         k_colsum_part<bf16><<<nb, 128, 0, s>>>((const bf16*)g, rows, C, pitch, (int)chunk, part);
     return cudaGetLastError();
@@ -1352,8 +1369,8 @@ cudaError_t mse(const float* pred, const float* target, long long n, float* grad
                 cudaStream_t s)
 {
     const int nb = (int)((n + 255) / 256);
-    k_mse<false><<<nb, 256, 0, s>>>(pred, target, n, nullptr, 1, 0.0f, nullptr, grad, part);
-    k_sum_one<<<1, 1024, 0, s>>>(part, nb, loss);
+    lbm::launch_pdl(k_mse<false>, nb, 256, 0, s, pred, target, n, nullptr, 1, 0.0f, nullptr, grad, part);
+    lbm::launch_pdl(k_sum_one, 1, 1024, 0, s, part, nb, loss);
     return cudaGetLastError();
 }
 
@@ -1362,8 +1379,8 @@ cudaError_t mse_increment(const float* Y, const float* t, const float* x, long l
 {
     const long long n = P * F;
     const int nb = (int)((n + 255) / 256);
-    k_mse<true><<<nb, 256, 0, s>>>(Y, t, n, x, F, alpha, inv_out, grad, part);
-    k_sum_one<<<1, 1024, 0, s>>>(part, nb, loss);
+    lbm::launch_pdl(k_mse<true>, nb, 256, 0, s, Y, t, n, x, F, alpha, inv_out, grad, part);
+    lbm::launch_pdl(k_sum_one, 1, 1024, 0, s, part, nb, loss);
     return cudaGetLastError();
 }
 
@@ -1372,8 +1389,8 @@ cudaError_t adam(float* w, const float* g, float* m, float* v, long long n, floa
 {
     const float c1 = 1.0f - powf(b1, (float)t), c2 = 1.0f - powf(b2, (float)t);
     if (n % 4 == 0 && (((uintptr_t)w | (uintptr_t)g | (uintptr_t)m | (uintptr_t)v | (uintptr_t)wb) & 15) == 0)
-        k_adam4<<<blocks(n / 4), 256, 0, s>>>((float4*)w, (const float4*)g, (float4*)m, (float4*)v, n / 4, lr, b1, b2,
-                                              eps, c1, c2, (uint2*)wb);
+        lbm::launch_pdl(k_adam4, blocks(n / 4), 256, 0, s, (float4*)w, (const float4*)g, (float4*)m, (float4*)v,
+                        n / 4, lr, b1, b2, eps, c1, c2, (uint2*)wb);
     else
         k_adam<<<blocks(n), 256, 0, s>>>(w, g, m, v, n, lr, b1, b2, eps, c1, c2, (bf16*)wb);
     return cudaGetLastError();
@@ -1384,7 +1401,7 @@ cudaError_t pack(const float* f, long long P, int F, const float* mean, const fl
 {
     if (F > cpitch) return cudaErrorInvalidValue;
     if (X && !R && F <= 8 && cpitch % 8 == 0 && ((uintptr_t)X & 15) == 0)
-        k_pack_px<<<blocks(P), 256, 0, s>>>(f, P, F, mean, inv_std, (bf16*)X, cpitch);
+        lbm::launch_pdl(k_pack_px, blocks(P), 256, 0, s, f, P, F, mean, inv_std, (bf16*)X, cpitch);
     else
         k_pack<<<blocks(P * cpitch), 256, 0, s>>>(f, P, F, mean, inv_std, (bf16*)X, cpitch, R);
     return cudaGetLastError();

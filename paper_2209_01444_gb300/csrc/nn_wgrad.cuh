@@ -110,6 +110,7 @@ __global__ void __launch_bounds__(kWsThreads, KYS == 1 ? 2 : 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
+    lbm::pdl_begin();  // after the tensor memory is taken, as in k_gemm_ws
 
     if (warp == 0) {  // ------------------------------------------- producer
         const uint32_t lead = elect_lane();
@@ -269,6 +270,7 @@ __global__ void __launch_bounds__(kWsThreads, BN <= 64 ? 2 : 1)
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = *tmem_slot;
+    lbm::pdl_begin();  // after the tensor memory is taken, as in k_gemm_ws
 
     if (warp == 0) {
         const uint32_t lead = elect_lane();
