@@ -1237,7 +1237,7 @@ __global__ void k_split_reduce_t_tile(const float* __restrict__ part, int splits
 // x 8 threads per start .. next start): one kernel after the other they were 44
 // launches of 4 to 15 us, most of a few blocks.  Each job adds its terms in the
 // order of the kernel named, so the results are the same bits.
-__global__ void __launch_bounds__(256) k_reduce_jobs(const ReduceJob* __restrict__ jobs, int njobs)
+__global__ void __launch_bounds__(256, 8) k_reduce_jobs(const ReduceJob* __restrict__ jobs, int njobs)
 {
     lbm::pdl_begin();
     __shared__ float t[32][33];
