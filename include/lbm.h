@@ -182,8 +182,8 @@ LBM_API int lbm_init_fields(lbm_handle* h, const double* fields, const double* o
 /* Queue `nsteps` coupled time steps (the fused stream-collide kernel of all
  * four models, then the wall kernels, then n_sub - 1 flow-only sub-steps) on
  * the handle's stream and return without waiting.  Long runs are replayed
- * from captured 16-step CUDA graphs; inside one, and inside the
- * remainder of a call, walls (n_sub = 1; on grids of more than 2^20 nodes the
+ * from captured 16-step CUDA graphs; inside one, and in FP32 storage inside
+ * the remainder of a call, walls (n_sub = 1; on grids of more than 2^20 nodes the
  * left/right ones) are updated by the next step as it loads them, and the last
  * step runs the wall kernels in full, so the state seen between calls is always
  * complete.  The graph is captured,
@@ -626,14 +626,15 @@ LBM_API int lbm_reduce_noalloc(const lbm_params* p, const void* scalar_pops, con
 /* Kernel timing for roofline measurements: while enabled, lbm_step launches
  * every coupled step directly (no graph) and brackets kernels with CUDA events
  * on the handle's stream.  enable = 1: the fused stream-collide kernel of each
- * coupled step; enable = 2: the n_sub - 1 flow sub-step kernels of each
+ * coupled step; enable = 2: the launches of the n_sub - 1 flow sub-steps of each
  * coupled step (two-time-scaling, Sec. 4; LBM_EINVAL when n_sub = 1), their
  * final wall pass excluded; 0 disables.  Enabling or disabling resets the
  * accumulated time. */
 LBM_API int lbm_set_profiling(lbm_handle* h, int enable);
 
 /* Total device time (ms) of the kernel launches timed since profiling was
- * enabled, and their number (fused kernels, or flow sub-step kernels).
+ * enabled, and their number (fused kernels, or flow sub-steps, several of
+ * which may share a launch).
  * Synchronises the pending events. */
 LBM_API int lbm_kernel_time(lbm_handle* h, double* total_ms, long long* launches);
 

@@ -359,9 +359,12 @@ int run_steps_direct(lbm_handle* h, int n)
             h->B.ev_end = h->ev[h->ev_used++];
             h->B.ev_substeps = h->prof_substeps;
         }
-        // (a profiled step runs its wall passes: its fused kernel is timed alone)
-        cudaError_t e = lbm::launch_coupled_step(h->P, h->storage, h->prm.n_sub, h->B, h->stream,
-                                                 !h->profiling && i > 0, !h->profiling && i + 1 < n);
+        // walls updated by the next step as it loads them, in FP32: with 16-bit
+        // storage a column left to the next step is not rounded, as the pass
+        // rounds it (a profiled step runs its passes: its kernel is timed alone)
+        const bool fold = !h->profiling && h->storage == LBM_FP32;
+        cudaError_t e = lbm::launch_coupled_step(h->P, h->storage, h->prm.n_sub, h->B, h->stream, fold && i > 0,
+                                                 fold && i + 1 < n);
         h->B.ev_begin = h->B.ev_end = nullptr;
         if (e != cudaSuccess) return cuda_fail(h, e, "coupled step");
     }
@@ -1479,8 +1482,9 @@ int batch_run_direct(lbm_batch* b, int n)
             T.ev_begin = b->ev[b->ev_used++];
             T.ev_end = b->ev[b->ev_used++];
         }
+        const bool fold = !b->profiling && b->storage == LBM_FP32;  // as for a single domain
         LBM_BCUDA(b, lbm::launch_batch_step(T, b->storage, b->ty, b->run, b->parity, b->ctas[tyk(b->ty)], b->stream,
-                                            !b->profiling && i > 0, !b->profiling && i + 1 < n));
+                                            fold && i > 0, fold && i + 1 < n));
         b->parity = 1 - b->parity;
     }
     return LBM_OK;

@@ -476,7 +476,7 @@ __device__ __forceinline__ void coupled_tile(const StepParams& P, const void* __
             float sum = 0.0f;
 #pragma unroll
             for (int i = 0; i < 5; ++i) {
-                const float v = side >= 2 ? stored<Store>(kF + i, fbw[i]) : fbw[i];
+                const float v = ROWS && side >= 2 ? stored<Store>(kF + i, fbw[i]) : fbw[i];
                 fs[i][hy][hx] = v;
                 sum += v;
             }

@@ -12,10 +12,12 @@
 //   output: the K-step increment proj1x1(d_0) in output units, so that the
 //   prediction is y = x + std_out * proj1x1(d_0), with the inputs normalised
 //   as (x - mean) / std_in.
-// A 3 x 3 convolution is an im2col gather followed by a GEMM with the bias and
-// ReLU in its epilogue; its input gradient is the same gather of the output
-// gradient times the 180-degree-rotated kernel; its weight gradient is a
-// split-K GEMM over all pixels.  s_l is written straight into the first half
+// A 3 x 3 convolution is an implicit GEMM with the bias and ReLU in its epilogue
+// (an im2col gather only for widths that are no multiple of 32 channels); its input
+// gradient is the same convolution of the output gradient with the
+// 180-degree-rotated kernel, the ReLU mask in the epilogue; its weight gradient
+// contracts input and output gradient over all pixels as they lie in memory
+// (nn_wgrad.cuh), in slices whose partial sums one launch adds at the end.  s_l is written straight into the first half
 // of the concatenation buffer cat_l and u_l into the second half, so the
 // concatenation costs nothing.
 #include <cuda_bf16.h>
