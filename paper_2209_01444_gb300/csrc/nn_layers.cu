@@ -385,7 +385,8 @@ __global__ void k_maxpool_bwd8(const bf16* __restrict__ X, int B, int H, int W, 
 // pooled layer and the rounding for the next GEMM in one pass (as k_maxpool_bwd8
 // and k_mask_cast8, which write and read the FP32 sum in between: 86 + 46 us at
 // 1 M pixels of 32 channels against 48).  Thread layout of k_maxpool_bwd8.
-__global__ void __launch_bounds__(256, 3) k_pool_mask_bwd8(const bf16* __restrict__ X, int B, int H, int W, int C, int xpitch,
+__global__ void __launch_bounds__(256, 3) k_pool_mask_bwd8(const bf16* __restrict__ X, int B, int H, int W, int C,
+                                                           int xpitch,
                                  const float* __restrict__ dY, const float* __restrict__ skip, int spitch,
                                  bf16* __restrict__ out)
 {
@@ -520,45 +521,66 @@ __global__ void __launch_bounds__(128) k_proj_fwd_vec(const bf16* __restrict__ X
     extern __shared__ float wsh[];  // O * C weights, then O biases
     __shared__ float out[128 * 8];
     __shared__ float so[8];
+    const int p0 = blockIdx.x * 128, p = p0 + threadIdx.x;
+    const int n = min(128, P - p0) * O;
+    const long long e0 = (long long)p0 * O;
+    // the pixel's first 32 channels and the fields are on their way while the
+    // weights arrive (1M pixels with the prediction: 35 us one after the other, 32 here)
+    const uint4* xp = (const uint4*)(X + (long long)p * xpitch);
+    uint4 q[4];
+    float xf[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) q[j] = p < P && j < C / 8 ? xp[j] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+        const int i = threadIdx.x + 128 * o;
+        xf[o] = y && i < n ? x[e0 + i] : 0.0f;
+    }
     for (int i = threadIdx.x; i < O * C; i += blockDim.x) wsh[i] = Wt[i];
     for (int i = threadIdx.x; i < O; i += blockDim.x) wsh[O * C + i] = bias[i];
     if (y && threadIdx.x < O) so[threadIdx.x] = 1.0f / inv_out[threadIdx.x];
     __syncthreads();
-    const int p0 = blockIdx.x * 128, p = p0 + threadIdx.x;
     if (p < P) {
         float acc[8];
 #pragma unroll
         for (int o = 0; o < 8; ++o) acc[o] = o < O ? wsh[O * C + o] + (R ? R[(long long)p * O + o] : 0.0f) : 0.0f;
-        const uint4* xp = (const uint4*)(X + (long long)p * xpitch);
-        for (int c8 = 0; c8 < C / 8; ++c8) {
-            const uint4 q = xp[c8];
-            const __nv_bfloat162* h = (const __nv_bfloat162*)&q;
-            float xv[8];
+        for (int c0 = 0; c0 < C / 8; c0 += 4) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 f = __bfloat1622float2(h[j]);
-                xv[2 * j] = f.x;
-                xv[2 * j + 1] = f.y;
+            for (int cj = 0; cj < 4; ++cj) {
+                const int c8 = c0 + cj;
+                if (c8 >= C / 8) break;
+                const __nv_bfloat162* h = (const __nv_bfloat162*)&q[cj];
+                float xv[8];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 f = __bfloat1622float2(h[j]);
+                    xv[2 * j] = f.x;
+                    xv[2 * j + 1] = f.y;
+                }
+#pragma unroll
+                for (int o = 0; o < 8; ++o) {
+                    if (o >= O) break;
+                    const float* w = wsh + o * C + c8 * 8;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) acc[o] += xv[j] * w[j];
+                }
             }
 #pragma unroll
-            for (int o = 0; o < 8; ++o) {
-                if (o >= O) break;
-                const float* w = wsh + o * C + c8 * 8;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) acc[o] += xv[j] * w[j];
-            }
+            for (int j = 0; j < 4; ++j)
+                if (c0 + 4 + j < C / 8) q[j] = xp[c0 + 4 + j];
         }
 #pragma unroll
         for (int o = 0; o < 8; ++o)
             if (o < O) out[threadIdx.x * O + o] = acc[o];
     }
     __syncthreads();
-    const int n = min(128, P - p0) * O;
-    const long long e0 = (long long)p0 * O;
-    for (int i = threadIdx.x; i < n; i += 128) {
+#pragma unroll
+    for (int o = 0; o < 8; ++o) {
+        const int i = threadIdx.x + 128 * o;
+        if (i >= n) break;
         const float v = out[i];
         Y[e0 + i] = v;
-        if (y) y[e0 + i] = x[e0 + i] + v * so[i % O];
+        if (y) y[e0 + i] = xf[o] + v * so[i % O];
     }
 }
 
@@ -1049,29 +1071,42 @@ __global__ void k_adam4(float4* __restrict__ w, const float4* __restrict__ g, fl
 
 // FP32 [P][F] fields -> BF16 NHWC [P][cpitch] with (x - mean) / std per field
 // and zero extra channels.
-// One thread per pixel: F <= 8 fields in, cpitch BF16 channels out as
-// 16-byte stores (cpitch a multiple of 8, X 16-byte aligned).
-__global__ void k_pack_px(const float* __restrict__ f, long long P, int F, const float* __restrict__ mean,
-                          const float* __restrict__ inv_std, bf16* __restrict__ X, int cpitch)
+// A block takes 256 pixels of F <= 8 fields, read contiguously, and writes their
+// cpitch BF16 channels (a multiple of 8, X 16-byte aligned) as 16-byte chunks, a
+// warp's 32 chunks in a row; only a pixel's first chunk holds fields.  A thread
+// writing a whole pixel stored 16 of every 64 bytes at a time: 22 us for 1M pixels
+// of 32 channels, 19 here.
+__global__ void __launch_bounds__(256) k_pack_px(const float* __restrict__ f, long long P, int F,
+                                                 const float* __restrict__ mean, const float* __restrict__ inv_std,
+                                                 bf16* __restrict__ X, int cpitch)
 {
     lbm::pdl_begin();
-    // the block's fields are read contiguously, then taken pixel by pixel
     __shared__ float in[256 * 8];
-    const long long p0 = blockIdx.x * 256LL, p = p0 + threadIdx.x;
-    const int n = (int)(P - p0 < 256 ? P - p0 : 256) * F;
+    __shared__ float ms[16];
+    if (threadIdx.x < F) {
+        ms[threadIdx.x] = mean[threadIdx.x];
+        ms[8 + threadIdx.x] = inv_std[threadIdx.x];
+    }
+    const long long p0 = blockIdx.x * 256LL;
+    const int np = (int)(P - p0 < 256 ? P - p0 : 256), n = np * F;
     for (int i = threadIdx.x; i < n; i += 256) in[i] = f[p0 * F + i];
     __syncthreads();
-    if (p >= P) return;
-    __nv_bfloat162 h[4];
-    float v[8];
+    const int G = cpitch / 8;  // chunks per pixel
+    uint4* dst = (uint4*)(X + p0 * cpitch);
+    for (int i = threadIdx.x; i < np * G; i += 256) {
+        const int p = i / G;
+        uint4 q = make_uint4(0, 0, 0, 0);
+        if (i == p * G) {
+            float v[8];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) v[c] = c < F ? (in[threadIdx.x * F + c] - mean[c]) * inv_std[c] : 0.0f;
+            for (int c = 0; c < 8; ++c) v[c] = c < F ? (in[p * F + c] - ms[c]) * ms[8 + c] : 0.0f;
+            __nv_bfloat162 h[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
-    uint4* dst = (uint4*)(X + p * cpitch);
-    dst[0] = *(const uint4*)h;
-    const uint4 z = make_uint4(0, 0, 0, 0);
-    for (int g = 1; g < cpitch / 8; ++g) dst[g] = z;
+            for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(v[2 * j], v[2 * j + 1]);
+            q = make_uint4(*(uint32_t*)&h[0], *(uint32_t*)&h[1], *(uint32_t*)&h[2], *(uint32_t*)&h[3]);
+        }
+        dst[i] = q;
+    }
 }
 
 // R (optional) receives the same normalised fields in FP32 [P][F].
@@ -1387,7 +1422,8 @@ cudaError_t mse(const float* pred, const float* target, long long n, float* grad
                 cudaStream_t s)
 {
     const int nb = (int)((n + 255) / 256);
-    lbm::launch_pdl(k_mse<false>, (nb + kMseRuns - 1) / kMseRuns, 256, 0, s, pred, target, n, nullptr, 1, 0.0f, nullptr, grad, part);
+    lbm::launch_pdl(k_mse<false>, (nb + kMseRuns - 1) / kMseRuns, 256, 0, s, pred, target, n, nullptr, 1, 0.0f, nullptr,
+                    grad, part);
     lbm::launch_pdl(k_sum_one, 1, 1024, 0, s, part, nb, loss);
     return cudaGetLastError();
 }
