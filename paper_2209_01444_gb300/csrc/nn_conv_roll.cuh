@@ -9,7 +9,8 @@
 // 512^2: 774 cycles a tile).  An output still gets its products by input row, tap
 // and channel, as there, so the results are the same bits.  k_gemm_ws against this,
 // us at 4 x 512^2: 32 -> 32 channels 39 and 29, 64 -> 32 59 and 41, 32 -> 64 65 and 40;
-// 64 -> 64 at 4 x 256^2 22.7 and 19.8.  What is left is about 8 us of launch, set-up
+// 64 -> 64 at 4 x 256^2 22.7 and 19.8, 128 -> 64 there 36.4 and 28.4 (CBL = 2: two channel
+// blocks, whose products k_gemm_ws's row-reuse form adds in this order too).  What is left is about 8 us of launch, set-up
 // and last drain, and 19 us of DRAM for the 32 channels in and out.
 //
 // Warp 0 loads RT input rows a stage, warp 1 issues the MMAs, the others drain the
@@ -17,21 +18,22 @@
 // ReLU mask loaded one stage ahead.  Waits are bounded as in k_gemm_ws.
 
 // Input rows a stage: as many as the tensor memory's 512 columns allow (output rows
-// in the ring: two unfinished and RT of each of three stages).
-template <int BN, int BK>
+// in the ring: two unfinished and RT of each of three stages), and one where two
+// channel blocks (CBL) of weights leave no room for more.
+template <int BN, int BK, int CBL>
 constexpr int roll_rows()
 {
-    return BN == 32 && BK == 32 ? 4 : 2;
+    return CBL == 2 ? 1 : BN == 32 && BK == 32 ? 4 : 2;
 }
-template <int BN, int BK>
-constexpr int roll_stage_bytes()
+template <int BN, int BK, int CBL>
+constexpr int roll_block_bytes()  // a channel block of a stage's rows
 {
-    return (roll_rows<BN, BK>() * (kBM + 2) * BK * 2 + 1023) / 1024 * 1024;
+    return (roll_rows<BN, BK, CBL>() * (kBM + 2) * BK * 2 + 1023) / 1024 * 1024;
 }
-template <int BN, int BK>
+template <int BN, int BK, int CBL>
 constexpr int roll_stages()
 {
-    constexpr int n = (224 * 1024 - 9 * BN * BK * 2) / roll_stage_bytes<BN, BK>();
+    constexpr int n = (224 * 1024 - 9 * CBL * BN * BK * 2) / (CBL * roll_block_bytes<BN, BK, CBL>());
     return n > 6 ? 6 : n;
 }
 constexpr int kRollEpi = 8;  // epilogue warps: two groups of one per lane quarter
@@ -41,24 +43,25 @@ constexpr int kRollThreads = 64 + 32 * kRollEpi;
 __device__ __forceinline__ int uniform(int v) { return __reduce_max_sync(0xffffffffu, v); }
 
 // total: rows of tiles, nx to an image row, H to a column, columns image by image.
-template <int BN, bool OUT_BF16, int BK>
+template <int BN, bool OUT_BF16, int BK, int CBL>
 __global__ void __launch_bounds__(kRollThreads, 1)
     k_conv_roll(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, void* __restrict__ D,
                 const float* __restrict__ bias, int N, int ldd, int relu, int W, int H, int nx, int total, ShuffleGeo sh)
 {
-    constexpr int RT = roll_rows<BN, BK>(), S = roll_stages<BN, BK>(), STAGE = roll_stage_bytes<BN, BK>();
-    constexpr int ROW = (kBM + 2) * BK * 2;  // bytes of an input row
+    constexpr int RT = roll_rows<BN, BK, CBL>(), S = roll_stages<BN, BK, CBL>();
+    constexpr int BLK = roll_block_bytes<BN, BK, CBL>(), STAGE = CBL * BLK;
+    constexpr int ROW = (kBM + 2) * BK * 2;  // bytes of an input row's channel block
     constexpr int B_BYTES = BN * BK * 2;
     constexpr int NS = 512 / BN;  // output rows in tensor memory
     constexpr int G = 4;          // stages whose outputs are under way
-    static_assert(NS >= 2 + 3 * RT, "output rows of three stages");
+    static_assert(NS >= 2 + 3 * RT && S >= 2, "output rows of three stages");
     constexpr int KS = BK / 16;
     constexpr uint32_t HI = tile_desc_hi<BK>();
     constexpr int UN = BN / 32;                        // units per tile
     constexpr int MU = UN == 2 ? RT : (RT + 1) / 2;    // units a warp has of a stage
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* wts = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);  // [kx][2 - ky][BN][BK]
-    uint8_t* rows = wts + 9 * B_BYTES;
+    uint8_t* wts = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);  // [block][kx][2 - ky][BN][BK]
+    uint8_t* rows = wts + 9 * CBL * B_BYTES;
     uint64_t* full = (uint64_t*)(rows + S * STAGE);
     uint64_t* empty = full + S;
     uint64_t* acc_full = empty + S;
@@ -106,9 +109,11 @@ __global__ void __launch_bounds__(kRollThreads, 1)
     if (warp == 0) {  // ------------------------------------------- producer
         const uint32_t lead = elect_lane();
         if (lead) {
-            mbar_expect_tx(wfull, 9 * B_BYTES);
-            for (int t = 0; t < 9; ++t)
-                tma_load_2d(wts + (t % 3 * 3 + 2 - t / 3) * B_BYTES, &tmB, t * BK, 0, wfull);
+            mbar_expect_tx(wfull, 9 * CBL * B_BYTES);
+            for (int t = 0; t < 9 * CBL; ++t) {  // tap t / CBL, channel block t % CBL
+                const int ky = t / (3 * CBL), kx = t / CBL - 3 * ky;
+                tma_load_2d(wts + ((t % CBL * 3 + kx) * 3 + 2 - ky) * B_BYTES, &tmB, t * BK, 0, wfull);
+            }
         }
         int it = 0;
         bool ok = true;
@@ -119,8 +124,9 @@ __global__ void __launch_bounds__(kRollThreads, 1)
                 const int st = it % S;
                 if (it >= S && !(ok = mbar_wait_warp(&empty[st], (uint32_t)((it / S - 1) & 1), abort_flag))) break;
                 if (!lead) continue;
-                mbar_expect_tx(&full[st], RT * ROW);
-                tma_load_4d(rows + st * STAGE, &tmA, 0, x0 - 1, y + i - 1, b, &full[st]);
+                mbar_expect_tx(&full[st], CBL * RT * ROW);
+                for (int cb = 0; cb < CBL; ++cb)
+                    tma_load_4d(rows + st * STAGE + cb * BLK, &tmA, cb * BK, x0 - 1, y + i - 1, b, &full[st]);
                 counts[0] = it + 1;
             }
         }
@@ -131,10 +137,12 @@ __global__ void __launch_bounds__(kRollThreads, 1)
         const uint32_t ut = uniform(tmem);
         const uint32_t w0 = uniform(tile_desc_lo<BK>(smem_u32(wts))), a0 = uniform(tile_desc_lo<BK>(smem_u32(rows)));
         int st = 0, ph = 0, g = 0;
-        // nb blocks of BN columns from block b on: tap kx, channels 16 k .., rows at a
-        auto mma = [&](int slot, uint32_t a, int b, int nb, int kx, int k, uint32_t acc) {
-            umma_lead(lead, ut + (uint32_t)(slot * BN), a + ((kx * BK * 2 + k * 32) >> 4), HI,
-                      w0 + (((kx * 3 + b) * B_BYTES + k * 32) >> 4), HI, idesc_bf16(kBM, BN * nb), acc);
+        // nb blocks of BN columns from block b on, K step ks (channel block, tap kx, channels
+        // 16 k ..), rows at a
+        auto mma = [&](int slot, uint32_t a, int b, int nb, int ks, uint32_t acc) {
+            const int cb = ks / (3 * KS), kx = ks / KS % 3, k = ks % KS;
+            umma_lead(lead, ut + (uint32_t)(slot * BN), a + ((cb * BLK + kx * BK * 2 + k * 32) >> 4), HI,
+                      w0 + ((((cb * 3 + kx) * 3 + b) * B_BYTES + k * 32) >> 4), HI, idesc_bf16(kBM, BN * nb), acc);
         };
         bool ok = mbar_wait_warp(wfull, 0, abort_flag, lim);
         for (int r = u0, n; r < u1 && ok; r += n) {
@@ -155,26 +163,18 @@ __global__ void __launch_bounds__(kRollThreads, 1)
                     const int lo = i < 2 ? 2 - i : 0, hi = i < n ? 3 : n + 2 - i;
                     const int s0 = (r - u0 + i - 2) & (NS - 1);
                     if (lo == 0 && hi == 3 && s0 <= NS - 3) {
+                        mma(s0, a, 0, 2, 0, 1);
+                        mma(s0 + 2, a, 2, 1, 0, 0);
 #pragma unroll
-                        for (int kx = 0; kx < 3; ++kx)
-#pragma unroll
-                            for (int k = 0; k < KS; ++k)
-                                if (kx == 0 && k == 0) {
-                                    mma(s0, a, 0, 2, 0, 0, 1);
-                                    mma(s0 + 2, a, 2, 1, 0, 0, 0);
-                                } else {
-                                    mma(s0, a, 0, 3, kx, k, 1);
-                                }
+                        for (int ks = 1; ks < 3 * KS * CBL; ++ks) mma(s0, a, 0, 3, ks, 1);
                     } else {
                         // the rows of a segment's ends, and where the ring wraps: block by block
 #pragma unroll
-                        for (int kx = 0; kx < 3; ++kx)
+                        for (int ks = 0; ks < 3 * KS * CBL; ++ks)
 #pragma unroll
-                            for (int k = 0; k < KS; ++k)
-#pragma unroll
-                                for (int b = 0; b < 3; ++b)
-                                    if (b >= lo && b < hi)
-                                        mma((s0 + b) & (NS - 1), a, b, 1, kx, k, kx == 0 && k == 0 && b == 2 ? 0u : 1u);
+                            for (int b = 0; b < 3; ++b)
+                                if (b >= lo && b < hi)
+                                    mma((s0 + b) & (NS - 1), a, b, 1, ks, ks == 0 && b == 2 ? 0u : 1u);
                     }
                 }
                 if (lead) {

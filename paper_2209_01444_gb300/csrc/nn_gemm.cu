@@ -1074,16 +1074,17 @@ cudaError_t launch_ws_mt(const CUtensorMap& a, const CUtensorMap& b, void* D, co
     return cudaGetLastError();
 }
 
-template <int BN, bool OUT_BF16, int BK>
+template <int BN, bool OUT_BF16, int BK, int CBL>
 cudaError_t launch_roll(const CUtensorMap& a, const CUtensorMap& b, void* D, const float* bias, int N, int ldd,
                         int relu, int W, int H, int nx, int total, int ctas, const ShuffleGeo& sh, cudaStream_t s)
 {
-    constexpr int smem = 9 * BN * BK * 2 + roll_stages<BN, BK>() * roll_stage_bytes<BN, BK>() + 1024 + 256;
+    constexpr int smem = 9 * CBL * BN * BK * 2 +
+                         roll_stages<BN, BK, CBL>() * CBL * roll_block_bytes<BN, BK, CBL>() + 1024 + 256;
     static_assert(smem <= 227 * 1024, "shared memory per CTA");
-    cudaError_t e = cudaFuncSetAttribute(k_conv_roll<BN, OUT_BF16, BK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    auto kernel = k_conv_roll<BN, OUT_BF16, BK, CBL>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    lbm::launch_pdl(k_conv_roll<BN, OUT_BF16, BK>, ctas, kRollThreads, smem, s, a, b, D, bias, N, ldd, relu, W, H,
-                    nx, total, sh);
+    lbm::launch_pdl(kernel, ctas, kRollThreads, smem, s, a, b, D, bias, N, ldd, relu, W, H, nx, total, sh);
     return cudaGetLastError();
 }
 
@@ -1689,17 +1690,18 @@ static cudaError_t conv3x3(const void* X, int B, int H, int W, int C, int cpitch
         bb = 1;
     }
     const long long nx = (W + kBM - 1) / kBM, total = nx * H * B;
-    // k_conv_roll where one channel block and one column tile hold everything, the
-    // last tile of a row is not mostly padding, and each SM has three tiles or more:
+    // k_conv_roll where one channel block (or two of 64, whose order of products is the
+    // row-reuse form's) and one column tile hold everything, the last tile of a row is not mostly padding, and each SM has three tiles or more:
     // fewer do not repay the two extra input rows and the weights each CTA loads
     // (64 -> 64 channels, k_gemm_ws against it: 1 x 128 x 256 9.3 and 10.1 us, 1 x 256 x 256
     // 12.3 and 12.3, 2 x 256 x 256 16.4 and 14.3; rows of 64 pixels, half a tile, 16 x 64 x
     // 64 12.3 and 16.4; 160 pixels, 4 x 160 x 160 forward, 322 and 313)
-    const bool roll = N <= bn && bn <= 64 && C == bk && nx * kBM * 5 <= 8LL * W && total >= 3LL * sm_count() &&
-                      total <= 0x7fffffffLL;
+    const bool roll = N <= bn && bn <= 64 && (C == bk || (C == 128 && bn == 64 && row3)) && nx * kBM * 5 <= 8LL * W &&
+                      total >= 3LL * sm_count() && total <= 0x7fffffffLL;
     row3 = row3 || roll;
     CUtensorMap ta, tb;
-    if (roll) bh = bn == 32 && bk == 32 ? roll_rows<32, 32>() : roll_rows<64, 64>();
+    if (roll)
+        bh = C == 128 ? roll_rows<64, 64, 2>() : bn == 32 && bk == 32 ? roll_rows<32, 32, 1>() : roll_rows<64, 64, 1>();
     cudaError_t e = make_map_4d(&ta, X, B, H, W, C, cpitch, row3 ? kBM + 2 : bw, bh, bb, bk);
     if (e == cudaSuccess) e = make_map(&tb, Wm, N, 9 * C, ldw, bn, bk);
     if (e != cudaSuccess) return e;
@@ -1711,13 +1713,16 @@ static cudaError_t conv3x3(const void* X, int B, int H, int W, int C, int cpitch
     const int M = B * H * W, K = 9 * C;
     if (roll) {
         const int ctas = total < sm_count() ? (int)total : sm_count();
-#define NN_ROLL(BNV, BKV)                                                                                            \
-    return out_bf16 ? launch_roll<BNV, true, BKV>(ta, tb, D, bias, N, ldd, relu, W, H, (int)nx, (int)total, ctas, sh, s) \
-                    : launch_roll<BNV, false, BKV>(ta, tb, D, bias, N, ldd, relu, W, H, (int)nx, (int)total, ctas, sh, s)
-        if (bn == 32 && bk == 32) NN_ROLL(32, 32);
-        if (bn == 64 && bk == 32) NN_ROLL(64, 32);
-        if (bn == 32 && bk == 64) NN_ROLL(32, 64);
-        if (bn == 64 && bk == 64) NN_ROLL(64, 64);
+#define NN_ROLL(BNV, BKV, CBLV)                                                                                      \
+    return out_bf16 ? launch_roll<BNV, true, BKV, CBLV>(ta, tb, D, bias, N, ldd, relu, W, H, (int)nx, (int)total,    \
+                                                        ctas, sh, s)                                                 \
+                    : launch_roll<BNV, false, BKV, CBLV>(ta, tb, D, bias, N, ldd, relu, W, H, (int)nx, (int)total,   \
+                                                         ctas, sh, s)
+        if (C == 128) NN_ROLL(64, 64, 2);
+        if (bn == 32 && bk == 32) NN_ROLL(32, 32, 1);
+        if (bn == 64 && bk == 32) NN_ROLL(64, 32, 1);
+        if (bn == 32 && bk == 64) NN_ROLL(32, 64, 1);
+        if (bn == 64 && bk == 64) NN_ROLL(64, 64, 1);
 #undef NN_ROLL
     }
     return bk == 64 ? dispatch<64, true>(bn, out_bf16, ta, tb, D, bias, M, N, K, ldd, relu ? 1 : 0, 1, 1 << 30, geo,

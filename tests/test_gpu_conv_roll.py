@@ -12,10 +12,11 @@ from paper_2209_01444_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
-# runs that cross images and columns of tiles and end anywhere in one; images of one and two rows; 32 and 64 channels in and out, ragged N
+# runs that cross images and columns of tiles and end anywhere in one; images of one and two rows; 32 to 128 channels in, 32 and 64 out, ragged N
 @pytest.mark.parametrize("B,H,width,C,N", [
     (1, 230, 256, 32, 32), (230, 1, 256, 32, 64), (120, 2, 256, 64, 32), (3, 100, 256, 64, 64), (2, 79, 384, 32, 40),
-    (1, 300, 384, 64, 24), (1, 61, 1024, 32, 8), (4, 127, 128, 64, 56)])
+    (1, 300, 384, 64, 24), (1, 61, 1024, 32, 8), (4, 127, 128, 64, 56),
+    (3, 100, 256, 128, 64), (2, 79, 384, 128, 40)])
 @pytest.mark.parametrize("fp32", [0, 1])
 def test_outputs_match_fp64(B, H, width, C, N, fp32):
     import torch
