@@ -699,9 +699,10 @@ __global__ void __launch_bounds__(256, 8) k_flow_substep(const StepParams P, con
 // move VW = 4 (K = 5: 2) nodes of a plane at a time, the loads straight into
 // shared memory (cp.async): loading and storing took two thirds of a launch with
 // a register and an instruction per value (1.12 M nodes, four steps: 46.5
-// against 44 us; FP16 2.4 M nodes, 32 steps: 778 against 643 us).
-// Per step and node, each thread reads its own populations, collides (its rows
-// in pairs, packed FP32), and after a barrier pushes them to the neighbours'
+// against 44 us; FP16 2.4 M nodes, 32 steps: 778 against 643 us, 697 with the
+// single step's collision).
+// Per step and node, each thread reads its own populations, collides (FP32: its rows
+// in pairs, packed), and after a barrier pushes them to the neighbours'
 // places, in the storage type (16-bit storage rounds at every step as a store
 // to memory would).  Wall nodes take the values of the flow-only wall pass
 // (rows, then columns) at the start of every step but the first (there when
@@ -783,7 +784,10 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
                        (!P.periodic_y && (ry0 <= 0 || ry0 + RH >= P.ny));
 
     pdl_begin();
-    float nw[NR], hfy[NR];
+    // FP32 collides two rows at once; with 16-bit storage each node does as in
+    // k_flow_substep, to the bit: a rounding that falls the other way is 1e-4 of a field
+    constexpr bool PACKED = std::is_same<Store, StoreF32>::value;
+    float nw[NR], hfy[NR];  // PACKED: q~ - 1 and half the force; else phi and the force
     bool on[NR];
 #pragma unroll
     for (int j = 0; j < NR; ++j) {
@@ -796,8 +800,9 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
             rowy = gy >= 0 && gy < P.ny;
         on[j] = colx && rowy && ly >= margin && ly < RH - margin;
         const long long o = on[j] ? (long long)gy * P.pitch + gx : 0;
-        nw[j] = -0.5f * (phi[block_index(o, phi_np)] + 1.0f);
-        hfy[j] = 0.5f * fb[o];
+        const float ph = phi[block_index(o, phi_np)], fy = fb[o];
+        nw[j] = PACKED ? -0.5f * (ph + 1.0f) : ph;
+        hfy[j] = PACKED ? 0.5f * fy : fy;
     }
     // the region's populations, groups of VW nodes of a row and plane; rx0 is a
     // multiple of VW, so a group inside the row lies in one node block
@@ -874,11 +879,23 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
         F2 ho[NR / 2][9];
 #pragma unroll
         for (int j = 0; j < NR; j += 2) {
-            F2 h[9];
+            if constexpr (PACKED) {
+                F2 h[9];
 #pragma unroll
-            for (int i = 0; i < 9; ++i)
-                h[i].v = make_float2(flow_dec<Store>(own[i * PP + PJ * j]), flow_dec<Store>(own[i * PP + PJ * (j + 1)]));
-            flow_collide2<Store>(P, {make_float2(nw[j], nw[j + 1])}, {make_float2(hfy[j], hfy[j + 1])}, h, ho[j / 2]);
+                for (int i = 0; i < 9; ++i) h[i].v = make_float2(own[i * PP + PJ * j], own[i * PP + PJ * (j + 1)]);
+                flow_collide2<Store>(P, {make_float2(nw[j], nw[j + 1])}, {make_float2(hfy[j], hfy[j + 1])}, h,
+                                     ho[j / 2]);
+            } else {
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    float h[9], o9[9];
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) h[i] = flow_dec<Store>(own[i * PP + PJ * (j + r)]);
+                    flow_collide<Store>(P, nw[j + r], hfy[j + r], h, o9);
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) (r ? ho[j / 2][i].v.y : ho[j / 2][i].v.x) = o9[i];
+                }
+            }
         }
         __syncthreads();
 #pragma unroll

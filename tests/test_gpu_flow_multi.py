@@ -62,6 +62,21 @@ def test_16_bit_storage(gpu_lib, storage, walls):
         assert np.abs(fa[name] - fb[name]).max() <= TOL[storage] * speed, name
 
 
+# away from walls 16-bit storage steps to the bit as one step at a time does: the
+# collision is the single step's, whatever the steps of a launch (2, 4 and 5)
+@pytest.mark.parametrize("storage", ["fp16", "bf16"])
+@pytest.mark.parametrize("n", [2, 8, 15])
+def test_16_bit_steps_are_the_single_steps_bits(gpu_lib, storage, n):
+    L, W = gpu_lib
+    a, b = _sim(L, W, 109, 45, "periodic", storage), _sim(L, W, 109, 45, "periodic", storage)
+    a.step_flow(n)
+    for _ in range(n):
+        b.step_flow(1)
+    fa, fb = a.fields(("ux", "uy", "p")), b.fields(("ux", "uy", "p"))
+    for name in fa:
+        assert np.array_equal(fa[name], fb[name]), name
+
+
 @pytest.fixture(scope="module")
 def gpu_lib():
     torch = pytest.importorskip("torch")
