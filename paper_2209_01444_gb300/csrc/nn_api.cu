@@ -96,7 +96,7 @@ int lbm_nn_conv3x3(const void* X, int B, int H, int W, int C, int cpitch, const 
                    const float* bias, int N, int out_fp32, int relu, void* stream)
 {
     // (ragged images stay refused here; the network runs them in other tiles)
-    if (B < 1 || H < 1 || W < 1 || !nn::conv3x3_whole_rows(B, H, W)) return LBM_EINVAL;
+    if (B < 1 || H < 1 || W < 1 || !nn::conv3x3_whole_rows(B, H, W)) return nn_status(cudaErrorNotSupported);
     return nn_status(nn::conv3x3_bf16(X, B, H, W, C, cpitch, Wm, ldw, D, ldd, bias, N, out_fp32 == 0, relu != 0,
                                       NN_S(stream)));
 }
