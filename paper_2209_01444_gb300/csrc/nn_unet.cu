@@ -678,11 +678,17 @@ static int get_vec(lbm_unet* u, const float* dev, float* host)
 {
     if (!u || !host) return LBM_EINVAL;
     const long long chunk = 2 * (long long)lbm::kPinHalf / (long long)sizeof(float);
-    std::lock_guard<std::mutex> hold(lbm::g_pinned.mu);
+    // The wait for this network's queued work comes before the buffer is taken, and
+    // where another call holds it this one does without: neither waits for the
+    // other's stream.
+    UN_CHECK(u, cudaStreamSynchronize(u->s));
+    std::unique_lock<std::mutex> hold(lbm::g_pinned.mu, std::try_to_lock);
     cudaError_t e = cudaSuccess;
-    float* pin = lbm::pinned_staging((size_t)std::min(u->n_padded, chunk) * sizeof(float), &e);
-    if (!pin) {  // no page-locked memory: tensor by tensor
-        UN_CHECK(u, cudaStreamSynchronize(u->s));
+    float* pin = nullptr;
+    if (hold.owns_lock() &&
+        !(pin = lbm::pinned_staging((size_t)std::min(u->n_padded, chunk) * sizeof(float), &e)))
+        hold.unlock();
+    if (!pin) {  // no page-locked memory, or in use: tensor by tensor
         for (const Tensor& t : u->tensors)
             UN_CHECK(u, cudaMemcpy(host + t.packed, dev + t.padded, (size_t)t.n * sizeof(float), cudaMemcpyDeviceToHost));
         return LBM_OK;
