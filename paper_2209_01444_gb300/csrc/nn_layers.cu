@@ -683,17 +683,20 @@ __global__ void k_proj_bwd_x4(const float* __restrict__ dY, int P, int O, const 
 // 8 (t % G) .. + 7 of every (256 / G)-th pixel of the block's chunk from one
 // 16-byte load; the threads of one channel group are added by shuffles within
 // each warp and then over the warps through shared memory, in a fixed order.
-// dXb (or null): also the input gradient, masked by X > 0 (X the output of a
-// ReLU) and rounded to BF16 [P][C], from the same loads.
-template <int O>
+// DX: also the input gradient dXb, masked by X > 0 (X the output of a ReLU) and
+// rounded to BF16 [P][C], from the same loads.  One pixel at a time: four pixels'
+// loads at once beside 9 O sums leave fewer warps resident (weights and bias alone,
+// 1M pixels of 32 channels: 30 against 49 us with 5 fields, 43 against 89 with 6;
+// with the input gradient 67 either way).
+template <int O, bool DX>
 __global__ void __launch_bounds__(256) k_proj_bwd_w8(const float* __restrict__ dY, const bf16* __restrict__ X, int P,
                                                      int C, int xpitch, int chunk, float* __restrict__ part,
                                                      const float* __restrict__ Wt, bf16* __restrict__ dXb)
 {
     lbm::pdl_begin();
     __shared__ float sm[8][8][O * 9];  // [warp][group][o * 9 + k], k = 8: the bias
-    __shared__ float wsh[O * 64];      // the weights (C <= 64)
-    if (dXb) {
+    __shared__ float wsh[DX ? O * 64 : 1];  // the weights (C <= 64)
+    if constexpr (DX) {
         for (int i = threadIdx.x; i < O * C; i += 256) wsh[i] = Wt[i];
         __syncthreads();
     }
@@ -706,45 +709,31 @@ __global__ void __launch_bounds__(256) k_proj_bwd_w8(const float* __restrict__ d
     for (int o = 0; o < O; ++o)
 #pragma unroll
         for (int k = 0; k < 9; ++k) acc[o][k] = 0.0f;
-    // four pixels' loads in flight; their products are added in pixel order
-    for (int pb = p0 + pl; pb < p1; pb += 4 * lanes) {
-        uint4 v4[4];
-        float d4[4][O];
+    for (int p = p0 + pl; p < p1; p += lanes) {
+        const uint4 v = *(const uint4*)(X + (long long)p * xpitch + 8 * cg);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+        float x[8];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int p = min(pb + j * lanes, p1 - 1);
-            v4[j] = *(const uint4*)(X + (long long)p * xpitch + 8 * cg);
-#pragma unroll
-            for (int o = 0; o < O; ++o) d4[j][o] = dY[(long long)p * O + o];
+        for (int k = 0; k < 4; ++k) {
+            x[2 * k] = __uint_as_float(w[k] << 16);
+            x[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
         }
+        float dx[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int p = pb + j * lanes;
-            if (p >= p1) break;
-            const uint32_t w[4] = {v4[j].x, v4[j].y, v4[j].z, v4[j].w};
-            float x[8];
+        for (int o = 0; o < O; ++o) {
+            const float d = dY[(long long)p * O + o];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                x[2 * k] = __uint_as_float(w[k] << 16);
-                x[2 * k + 1] = __uint_as_float(w[k] & 0xffff0000u);
-            }
-            float dx[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            for (int k = 0; k < 8; ++k) acc[o][k] += d * x[k];
+            acc[o][8] += d;
+            if constexpr (DX)
 #pragma unroll
-            for (int o = 0; o < O; ++o) {
-                const float d = d4[j][o];
+                for (int k = 0; k < 8; ++k) dx[k] += d * wsh[o * C + 8 * cg + k];
+        }
+        if constexpr (DX) {
+            __align__(16) bf16 b[8];
 #pragma unroll
-                for (int k = 0; k < 8; ++k) acc[o][k] += d * x[k];
-                acc[o][8] += d;
-                if (dXb)
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) dx[k] += d * wsh[o * C + 8 * cg + k];
-            }
-            if (dXb) {
-                __align__(16) bf16 b[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) b[k] = __float2bfloat16(x[k] > 0.0f ? dx[k] : 0.0f);
-                *(uint4*)(dXb + (long long)p * C + 8 * cg) = *(const uint4*)b;
-            }
+            for (int k = 0; k < 8; ++k) b[k] = __float2bfloat16(x[k] > 0.0f ? dx[k] : 0.0f);
+            *(uint4*)(dXb + (long long)p * C + 8 * cg) = *(const uint4*)b;
         }
     }
     // lanes with the same group differ in the bits above log2(G)
@@ -1300,8 +1289,8 @@ cudaError_t proj_bwd(const float* dY, const void* X, int P, int C, int xpitch, c
     if (vec) {
         switch (O) {
 #define NN_PROJ_W8(OV) \
-    case OV: lbm::launch_pdl(k_proj_bwd_w8<OV>, nb, 256, 0, s, dY, (const bf16*)X, P, C, xpitch, chunk, part, Wt, \
-                             (bf16*)dXb); break;
+    case OV: lbm::launch_pdl(dXb ? k_proj_bwd_w8<OV, true> : k_proj_bwd_w8<OV, false>, nb, 256, 0, s, dY,          \
+                             (const bf16*)X, P, C, xpitch, chunk, part, Wt, (bf16*)dXb); break;
             NN_PROJ_W8(1)
             NN_PROJ_W8(2)
             NN_PROJ_W8(3)
