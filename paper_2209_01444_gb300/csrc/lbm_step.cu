@@ -769,7 +769,7 @@ __global__ void __launch_bounds__(256, 8) k_flow_substep(const StepParams P, con
 // to memory would).  Wall nodes take the values of the flow-only wall pass
 // (rows, then columns) at the start of every step but the first (there when
 // `repair` is set: the launch before left them out); the last step leaves them
-// to the next launch or the pass.
+// to the next launch or the pass.  more: another launch of the chain follows.
 constexpr int kFmW = 64;   // region width: two warps
 constexpr int kFmY = 8;    // rows of threads
 constexpr int kFmR = 4;    // rows per thread
@@ -815,7 +815,7 @@ template <class Store, int K>
 __global__ void __launch_bounds__(kFmW* kFmY, 2)
     k_flow_multi(const StepParams P, const void* __restrict__ src, void* __restrict__ dst,
                  const float* __restrict__ phi, int phi_np, const float* __restrict__ fb, const void* __restrict__ sc,
-                 int ks, int repair)
+                 int ks, int repair, int more)
 {
     static_assert(kFmR % 2 == 0, "rows in pairs");
     constexpr int KX = fm_kx(K);
@@ -845,7 +845,8 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
     const bool walls = (!P.periodic_x && (rx0 <= 0 || rx0 + kFmW >= P.nx)) ||
                        (!P.periodic_y && (ry0 <= 0 || ry0 + RH >= P.ny));
 
-    pdl_begin();
+    pdl_wait();
+    if (more) pdl_release();  // the chain's next launch, of as many CTAs, at once; the wall pass at the end
     // FP32 collides two rows at once; with 16-bit storage each node does as in
     // k_flow_substep, to the bit: a rounding that falls the other way is 1e-4 of a field
     constexpr bool PACKED = std::is_same<Store, StoreF32>::value;
@@ -974,6 +975,7 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
         __syncthreads();
         if (k + 1 == ks) break;
     }
+    if (!more) pdl_release();
     using V = typename VecOf<GB>::V;
     constexpr int GO = (kFmW - 2 * KX) / VW, RO = RH - 2 * K;
     for (int q = t; q < GO * RO; q += kFmW * kFmY) {
@@ -994,7 +996,7 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
 
 template <class Store, int K>
 cudaError_t launch_flow_multi(const StepParams& P, const void* src, void* dst, const float* phi, int phi_np,
-                              const float* fb, const void* sc, int ks, int repair, cudaStream_t s)
+                              const float* fb, const void* sc, int ks, int repair, int more, cudaStream_t s)
 {
     constexpr int ow = kFmW - 2 * fm_kx(K), oh = kFmH - 2 * K, smem = flow_multi_smem<Store>();
     if (smem > 48 * 1024) {
@@ -1004,7 +1006,7 @@ cudaError_t launch_flow_multi(const StepParams& P, const void* src, void* dst, c
     }
     const dim3 grid((P.nx + ow - 1) / ow, (P.ny + oh - 1) / oh);
     return launch_pdl(k_flow_multi<Store, K>, grid, dim3(kFmW, kFmY), smem, s, P, src, dst, phi, phi_np, fb, sc, ks,
-                      repair);
+                      repair, more);
 }
 
 // Steps per launch for n >= 2 flow steps on an nx x ny grid: a launch costs about
@@ -1052,7 +1054,7 @@ cudaError_t flow_chain(const StepParams& P, int n, const void* sc, void* const f
         const auto launch = K == 2   ? launch_flow_multi<Store, 2>
                             : K == 4 ? launch_flow_multi<Store, 4>
                                      : launch_flow_multi<Store, 5>;
-        e = launch(P, fl[*cf], fl[1 - *cf], phi, phi_np, fb, sc, ks, repair, s);
+        e = launch(P, fl[*cf], fl[1 - *cf], phi, phi_np, fb, sc, ks, repair, left > 1, s);
         n -= ks;
         repair = 1;
         *cf = 1 - *cf;

@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(128) k_proj_fwd_vec(const bf16* __restrict__ X
                                                       int O, const float* __restrict__ R, float* __restrict__ Y,
                                                       const float* x, const float* __restrict__ inv_out, float* y)
 {
-    lbm::pdl_begin();
+    lbm::pdl_wait();
     extern __shared__ float wsh[];  // O * C weights, then O biases
     __shared__ float out[128 * 8];
     __shared__ float so[8];
@@ -574,6 +574,7 @@ __global__ void __launch_bounds__(128) k_proj_fwd_vec(const bf16* __restrict__ X
             if (o < O) out[threadIdx.x * O + o] = acc[o];
     }
     __syncthreads();
+    lbm::pdl_release();
 #pragma unroll
     for (int o = 0; o < 8; ++o) {
         const int i = threadIdx.x + 128 * o;

@@ -56,3 +56,47 @@ def test_projection_weight_gradients_of_six_fields(env, P, C):
         return fn
 
     assert _ratio(torch, call(6), call(3)) < 2.3
+
+
+# calls queued one behind the other take no longer than a call alone, launch and all;
+# 1.3 where the CTAs of kernels that wait for their turn lie on few SMs
+def test_projections_queued_one_behind_the_other(env):
+    torch, lib = env
+    P, C, O = 100003, 256, 8
+    X, Wt = torch.randn(P, C, device="cuda").bfloat16(), torch.randn(O, C, device="cuda")
+    bias, Y = torch.randn(O, device="cuda"), torch.empty(P, O, device="cuda")
+
+    def fn():
+        assert lib.lbm_nn_proj_fwd(X.data_ptr(), P, C, C, Wt.data_ptr(), bias.data_ptr(), O, None, Y.data_ptr(),
+                                   torch.cuda.current_stream().cuda_stream) == 0
+
+    e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+
+    def time(reps):
+        torch.cuda.synchronize()
+        e[0].record()
+        for _ in range(reps):
+            fn()
+        e[1].record()
+        torch.cuda.synchronize()
+        return e[0].elapsed_time(e[1]) / reps
+
+    time(20)
+    queued, alone = (float(np.median([time(n) for _ in range(25)])) for n in (30, 1))
+    assert queued < 1.15 * alone
+
+
+# a second flow step in the same launch costs less than the first, which takes the
+# wall passes and the frozen fields' pass with it; 3.0 where the wall pass's CTAs were
+# resident before the step had finished, on the few SMs that it left free
+@pytest.mark.parametrize("walls", [("noslip", "noslip", "periodic", "periodic"),
+                                   ("inflow", "outflow", "symmetry", "symmetry")])
+@pytest.mark.parametrize("nx", [4, 32])
+def test_two_flow_steps_of_a_long_strip(env, nx, walls):
+    from paper_2209_01444_gb300 import lbm as L, workloads as W
+
+    torch, _ = env
+    p = W.thermosolutal_params(nx, 8000, bc=walls, u_in=(0.5, 0.0))
+    sim = L.Simulation(p, stream=torch.cuda.current_stream())
+    sim.init_seeds(np.array([[0.5 * nx, 4000.0, 1.0, 0.0]]), 0.0, -0.55)
+    assert _ratio(torch, lambda: sim.step_flow(2), lambda: sim.step_flow(1)) < 2.0
