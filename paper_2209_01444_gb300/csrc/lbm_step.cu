@@ -725,14 +725,44 @@ __device__ __forceinline__ void flow_collide2(const StepParams& P, F2 nw, F2 hFy
     out[8] = g - t;
 }
 
+// The flow populations that the flow-only wall pass (rows, then columns) would have
+// left at wall node (x, y) after the flow step before, which skipped it: a row node's
+// from its interior node, a column node's from its interior node, which in a corner
+// is itself a row node, as the row pass would store it.
+template <class Store>
+__device__ __forceinline__ void flow_wall_repair(const StepParams& P, const void* __restrict__ sc,
+                                                 const void* __restrict__ src, int x, int y, bool column, bool row,
+                                                 float (&h)[9])
+{
+    const int xi = !column ? x : (x == 0 ? 1 : P.nx - 2);
+    const int yi = !row ? y : (y == 0 ? 1 : P.ny - 2);
+    const long long oi = (long long)yi * P.pitch + xi;
+    float hi[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) h[i] = Store::load(nullptr, src, kH + i, oi, P);
+#pragma unroll 1
+    for (int axis = row ? 1 : 0; axis >= (column ? 0 : 1); --axis) {
+        // the column's own step reads the scalars of the node beside it
+        const long long os = axis ? oi : (long long)y * P.pitch + xi;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) hi[i] = h[i];
+        flow_wall_from(P, axis, axis ? (y == 0 ? 2 : 3) : (x == 0 ? 0 : 1), flow_wall_scalars<Store>(P, sc, os), hi, h);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) h[i] = stored<Store>(kH + i, h[i]);
+    }
+}
+
 // One flow sub-step (two-time-scaling of Sec. 4): collide and stream h with phi
 // and the force frozen at time n.
 // phi: plane 0 of a node-block array of phi_np planes (the history, or the
-// frozen phi of flow-only steps, phi_np = 1: a plain plane).
-template <class Store>
+// frozen phi of flow-only steps, phi_np = 1: a plain plane).  REPAIR: the flow step
+// before left the flow-only wall pass out; wall nodes first take what it would have
+// given them (sc: the newest scalar populations, whose macros it uses).
+template <class Store, bool REPAIR>
 __global__ void __launch_bounds__(256, 8) k_flow_substep(const StepParams P, const void* __restrict__ src,
                                                       void* __restrict__ dst, const float* __restrict__ phi,
-                                                      int phi_np, const float* __restrict__ fb)
+                                                      int phi_np, const float* __restrict__ fb,
+                                                      const void* __restrict__ sc)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -741,6 +771,11 @@ __global__ void __launch_bounds__(256, 8) k_flow_substep(const StepParams P, con
     float h[9], ho[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) h[i] = Store::load(nullptr, src, kH + i, o, P);
+    if constexpr (REPAIR) {
+        const bool column = !P.periodic_x && (x == 0 || x == P.nx - 1);
+        const bool row = !P.periodic_y && (y == 0 || y == P.ny - 1);
+        if (column || row) flow_wall_repair<Store>(P, sc, src, x, y, column, row, h);
+    }
     flow_collide<Store>(P, phi[block_index(o, phi_np)], fb[o], h, ho);
     const int xp = (x + 1 == P.nx) ? 0 : x + 1, xm = (x == 0) ? P.nx - 1 : x - 1;
     const int yp = (y + 1 == P.ny) ? 0 : y + 1, ym = (y == 0) ? P.ny - 1 : y - 1;
@@ -1009,18 +1044,26 @@ cudaError_t launch_flow_multi(const StepParams& P, const void* src, void* dst, c
                       repair, more);
 }
 
-// Steps per launch for n >= 2 flow steps on an nx x ny grid: a launch costs about
-// its steps plus 8 of them for loading, the walls' scalars and storing, once for
-// each wave of two CTAs per SM that the regions fill (15 flow steps at 1024^2: K =
-// 4 fills 3 waves and K = 5 four, 818 and 834 us per four coupled steps; at 100^2,
-// one wave, 222 and 205 us).
-inline int flow_multi_k(int n, int nx, int ny)
+// Steps per launch for n >= 2 flow steps on an nx x ny grid, or 1 for node by node.
+// In us: a launch of several steps costs about its steps plus 8 of them for loading,
+// the walls' scalars and storing, once for each wave of two CTAs per SM that the
+// regions fill (15 flow steps at 1024^2: K = 4 fills 3 waves and K = 5 four, 818 and
+// 834 us per four coupled steps; at 100^2, one wave, 222 and 205 us).  Node by node a
+// step costs about 4 for its launch and 3.2 for each 64 warps per SM (3 and 2.8 with
+// 16-bit storage).  Where a region covers little more than half its nodes of the grid
+// that is the faster (14 steps of 262140 x 4 nodes, no walls: 190 us against 572 in
+// regions, FP16 180 against 704; of 4 x 262140 FP16 1260 and 1840); not on tall strips with walls
+// at their sides, whose nodes a warp of a step finds one to a row (16 x 65536, FP32: 32
+// steps 1477 and 1086).
+template <class Store>
+int flow_multi_k(const StepParams& P, int n)
 {
+    const int nx = P.nx, ny = P.ny;
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     int best = 2;
-    long long least = 0;
+    long long least = 0, regions = 1;
     for (int K : {2, 4, 5}) {
         const int ow = kFmW - 2 * fm_kx(K), oh = kFmH - 2 * K;
         const long long tiles = (long long)((nx + ow - 1) / ow) * ((ny + oh - 1) / oh);
@@ -1028,7 +1071,13 @@ inline int flow_multi_k(int n, int nx, int ny)
         if (least == 0 || cost < least) {
             least = cost;
             best = K;
+            regions = tiles;
         }
+    }
+    if (regions > 2 * sms && 1.8 * nx * ny < (double)(regions * kFmW * kFmH) && (P.periodic_x || nx >= ny)) {
+        constexpr bool F32 = std::is_same<Store, StoreF32>::value;
+        const double waves = (double)ny * ((nx + 31) / 32) / (64.0 * sms);
+        if (n * ((F32 ? 4.0 : 3.0) + (F32 ? 3.2 : 2.8) * waves) < (double)least) return 1;
     }
     return best;
 }
@@ -1041,13 +1090,17 @@ cudaError_t flow_chain(const StepParams& P, int n, const void* sc, void* const f
                        int phi_np, const float* fb, cudaStream_t s)
 {
     cudaError_t e = cudaSuccess;
-    if (n == 1) {
+    const int K = n == 1 ? 1 : flow_multi_k<Store>(P, n);
+    if (K == 1) {
         const dim3 block(64, 4), grid((P.nx + 63) / 64, (P.ny + 3) / 4);
-        k_flow_substep<Store><<<grid, block, 0, s>>>(P, fl[*cf], fl[1 - *cf], phi, phi_np, fb);
-        *cf = 1 - *cf;
-        return cudaGetLastError();
+        for (int k = 0; k < n && e == cudaSuccess; ++k) {
+            const auto step = k > 0 && !(P.periodic_x && P.periodic_y) ? k_flow_substep<Store, true> : k_flow_substep<Store, false>;
+            step<<<grid, block, 0, s>>>(P, fl[*cf], fl[1 - *cf], phi, phi_np, fb, sc);
+            *cf = 1 - *cf;
+            e = cudaGetLastError();
+        }
+        return e;
     }
-    const int K = flow_multi_k(n, P.nx, P.ny);
     int repair = 0;
     for (int left = (n + K - 1) / K; left > 0 && e == cudaSuccess; --left) {
         const int ks = (n + left - 1) / left;

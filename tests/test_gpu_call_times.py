@@ -58,8 +58,8 @@ def test_projection_weight_gradients_of_six_fields(env, P, C):
     assert _ratio(torch, call(6), call(3)) < 2.3
 
 
-# calls queued one behind the other take no longer than a call alone, launch and all;
-# 1.3 where the CTAs of kernels that wait for their turn lie on few SMs
+# calls queued one behind the other take less than a call alone with its launch
+# (0.75 as it stands) and 1.1 to 1.2 where the CTAs of kernels that wait for their turn lie on few SMs
 def test_projections_queued_one_behind_the_other(env):
     torch, lib = env
     P, C, O = 100003, 256, 8
@@ -83,7 +83,7 @@ def test_projections_queued_one_behind_the_other(env):
 
     time(20)
     queued, alone = (float(np.median([time(n) for _ in range(25)])) for n in (30, 1))
-    assert queued < 1.15 * alone
+    assert queued < 0.95 * alone
 
 
 # a second flow step in the same launch costs less than the first, which takes the
@@ -100,3 +100,18 @@ def test_two_flow_steps_of_a_long_strip(env, nx, walls):
     sim = L.Simulation(p, stream=torch.cuda.current_stream())
     sim.init_seeds(np.array([[0.5 * nx, 4000.0, 1.0, 0.0]]), 0.0, -0.55)
     assert _ratio(torch, lambda: sim.step_flow(2), lambda: sim.step_flow(1)) < 2.0
+
+
+# fourteen flow steps of a long strip in one call cost no more than one by one, wall
+# pass and frozen fields' pass each time; 2 to 4 where they run in regions of which the
+# strip fills a small part
+@pytest.mark.parametrize("storage", ["fp32", "fp16"])
+def test_flow_steps_of_a_long_strip(env, storage):
+    from paper_2209_01444_gb300 import lbm as L, workloads as W
+
+    torch, _ = env
+    p = W.thermosolutal_params(262140, 4)
+    sim = L.Simulation(p, storage, stream=torch.cuda.current_stream())
+    sim.init_seeds(np.array([[1000.0, 2.0, 1.0, 0.0]]), 0.0, -0.55)
+    one = lambda: [sim.step_flow(1) for _ in range(14)]  # noqa: E731
+    assert _ratio(torch, lambda: sim.step_flow(14), one, reps=5) < 1.15

@@ -1,8 +1,9 @@
-"""Flow steps taken four to a launch next to walls, launches after the first
+"""Flow steps next to walls: four to a launch, launches after the first
 (which update the walls that the launch before left out) and launches of fewer
 steps than the region's rings allow among them, against the same steps one at a
 time.  On grids of one wave 3, 7 and 8 steps are launches of 3, 4 + 3 and 4 + 4; at
-1024^2, several waves, 14 steps are launches of 4, 4, 3 and 3.
+1024^2, several waves, 14 steps are launches of 4, 4, 3 and 3.  And steps of long strips,
+which go node by node.
 
 FP32 differs by rounding: a few units (2^-23 of populations of order one, against
 speeds of order 0.1: 1.2e-6 each) per step, two of them allowed.  16-bit storage:
@@ -60,3 +61,12 @@ def test_four_steps_a_launch_16_bit(walls, storage, tol, n):
 
 def test_several_waves():
     _compare(1024, 1024, "channel", "fp32", 14, 2.4e-6 * 14)
+
+
+# strips of which a region covers a small part go node by node, each step but the
+# first updating the walls that the step before left out; corners among them
+@pytest.mark.parametrize("nx,ny,walls", [(20000, 4, "channel"), (20001, 5, "noslip"), (20000, 6, "tube"),
+                                         (4, 9000, "noslip")])
+@pytest.mark.parametrize("storage,tol", [("fp32", 2.4e-6 * 3), ("fp16", 2e-3), ("bf16", 3e-2)])
+def test_long_strips(nx, ny, walls, storage, tol):
+    _compare(nx, ny, walls, storage, 3, tol)
