@@ -31,8 +31,8 @@ float* pinned_staging(size_t bytes, cudaError_t* e);
 template <class Fn>
 void parallel_range(long long n, long long least, Fn fn)
 {
-    const int nt = (int)std::max<long long>(
-        1, std::min({(long long)std::thread::hardware_concurrency(), 16LL, n / std::max(1LL, least)}));
+    static const long long most = std::min(std::thread::hardware_concurrency(), 16u);  // (a read of /sys each time)
+    const int nt = (int)std::max<long long>(1, std::min(most, n / std::max(1LL, least)));
     if (nt == 1) {
         fn(0LL, n);
         return;

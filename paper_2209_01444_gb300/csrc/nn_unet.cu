@@ -28,6 +28,8 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <memory>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -670,10 +672,15 @@ int lbm_unet_set_params(lbm_unet* u, const float* host)
     return LBM_OK;
 }
 
-// The packed tensors of a padded device vector to host memory: through the
+// Up to this many values a read goes through plain host memory: the staged form gains
+// from two host threads on (parallel_range below), one is the slower for the copy out
+// of page-locked memory (407,109 values 100 us against 118, 911,717 values 259 and 151).
+constexpr long long kPlainRead = 1 << 19;
+
+// The packed tensors of a padded device vector to host memory.  Large ones through the
 // page-locked staging buffer at the host link's rate, then on up to 16 threads
-// into the caller's (pageable, often untouched) memory.  A zeroed vector as the
-// way-station of a pageable copy took 2.4 ms for the five-level network's 31 MB.
+// into the caller's (pageable, often untouched) memory: 1.08 ms for the five-level
+// network's 31 MB, 2.15 through plain memory.
 static int get_vec(lbm_unet* u, const float* dev, float* host)
 {
     if (!u || !host) return LBM_EINVAL;
@@ -682,15 +689,21 @@ static int get_vec(lbm_unet* u, const float* dev, float* host)
     // where another call holds it this one does without: neither waits for the
     // other's stream.
     UN_CHECK(u, cudaStreamSynchronize(u->s));
-    std::unique_lock<std::mutex> hold(lbm::g_pinned.mu, std::try_to_lock);
+    std::unique_lock<std::mutex> hold(lbm::g_pinned.mu, std::defer_lock);
     cudaError_t e = cudaSuccess;
     float* pin = nullptr;
-    if (hold.owns_lock() &&
+    if (u->n_padded > kPlainRead && hold.try_lock() &&
         !(pin = lbm::pinned_staging((size_t)std::min(u->n_padded, chunk) * sizeof(float), &e)))
         hold.unlock();
-    if (!pin) {  // no page-locked memory, or in use: tensor by tensor
-        for (const Tensor& t : u->tensors)
-            UN_CHECK(u, cudaMemcpy(host + t.packed, dev + t.padded, (size_t)t.n * sizeof(float), cudaMemcpyDeviceToHost));
+    if (!pin) {
+        const std::unique_ptr<float[]> pad(new (std::nothrow) float[(size_t)u->n_padded]);
+        if (pad) UN_CHECK(u, cudaMemcpy(pad.get(), dev, (size_t)u->n_padded * sizeof(float), cudaMemcpyDeviceToHost));
+        for (const Tensor& t : u->tensors) {
+            if (pad)
+                std::memcpy(host + t.packed, &pad[t.padded], (size_t)t.n * sizeof(float));
+            else
+                UN_CHECK(u, cudaMemcpy(host + t.packed, dev + t.padded, (size_t)t.n * sizeof(float), cudaMemcpyDeviceToHost));
+        }
         return LBM_OK;
     }
     for (long long c0 = 0; c0 < u->n_padded; c0 += chunk) {

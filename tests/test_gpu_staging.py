@@ -12,8 +12,10 @@ from paper_2209_01444_gb300 import workloads as W
 pytestmark = pytest.mark.gpu
 
 
+# 103,205 and 1,927,845 parameters: read through plain memory and through the buffer
+@pytest.mark.parametrize("levels", [2, 4])
 @pytest.mark.parametrize("busy", ["network", "fields"])
-def test_a_busy_stream_holds_up_its_own_read_alone(busy):
+def test_a_busy_stream_holds_up_its_own_read_alone(busy, levels):
     import torch
 
     from paper_2209_01444_gb300 import lbm as L, surrogate as S
@@ -21,7 +23,7 @@ def test_a_busy_stream_holds_up_its_own_read_alone(busy):
     case = W.single_seed_periodic(n=48, steps=1, R=6.0)
     sim = L.Simulation(case.params)
     sim.init_seeds(case.seeds, case.U0, case.theta0)
-    net = S.UNet(1, 32, 32, levels=2)
+    net = S.UNet(2, 32, 32, levels=levels)
     vec = np.random.Generator(np.random.PCG64(1)).normal(size=net.param_count).astype(np.float32)
     net.set_params(vec)
     reads = {"network": lambda: np.concatenate([v.reshape(-1) for v in net.params().values()]),
