@@ -1133,20 +1133,17 @@ cudaError_t launch_ws(const CUtensorMap& a, const CUtensorMap& b, void* D, const
     return launch_ws_rows<BN, OUT_BF16, BK, CONV, false>(a, b, D, bias, M, N, K, ldd, relu, geo, sh, s);
 }
 
-#ifndef LBM_BN_FILL
-#define LBM_BN_FILL 0.5
-#endif
 // Widest tile that N allows: narrower tiles with more CTAs re-read A and
 // measured slower even where the wide tiles leave SMs idle.
 int bn_for(int N) { return N >= 256 ? 256 : N > 64 ? 128 : N > 32 ? 64 : 32; }
 
 // The same for a persistent GEMM of `tiles_m` row tiles: narrowed to 64 columns at
-// least while that leaves SMs without a tile.  A CTA's loads per K block, not the
-// MMAs, set its pace, and fewer columns are fewer weights to load.
+// least while that leaves more than half the SMs without a tile.  A CTA's loads per K
+// block, not the MMAs, set its pace, and fewer columns are fewer weights to load.
 int bn_fill(int N, long long tiles_m)
 {
     int bn = bn_for(N);
-    while (bn > 64 && tiles_m * ((N + bn - 1) / bn) < LBM_BN_FILL * sm_count()) bn /= 2;
+    while (bn > 64 && 2 * tiles_m * ((N + bn - 1) / bn) < sm_count()) bn /= 2;
     return bn;
 }
 
@@ -1691,13 +1688,20 @@ static cudaError_t conv3x3(const void* X, int B, int H, int W, int C, int cpitch
     }
     const long long nx = (W + kBM - 1) / kBM, total = nx * H * B;
     // k_conv_roll where one channel block (or two of 64, whose order of products is the
-    // row-reuse form's) and one column tile hold everything, the last tile of a row is not mostly padding, and each SM has three tiles or more:
-    // fewer do not repay the two extra input rows and the weights each CTA loads
-    // (64 -> 64 channels, k_gemm_ws against it: 1 x 128 x 256 9.3 and 10.1 us, 1 x 256 x 256
-    // 12.3 and 12.3, 2 x 256 x 256 16.4 and 14.3; rows of 64 pixels, half a tile, 16 x 64 x
-    // 64 12.3 and 16.4; 160 pixels, 4 x 160 x 160 forward, 322 and 313)
+    // row-reuse form's) and one column tile hold everything, the last tile of a row is
+    // not mostly padding, and each SM has three tiles or more: fewer do not repay the two
+    // extra input rows and the weights each CTA loads.  Where columns of tiles end within
+    // CTAs' runs (their number does not divide the SMs'), a run of three or four rows comes
+    // in two parts with two extra rows each, and it takes more than four tiles; 32 -> 64
+    // channels, the most gained, from three on all the same.  k_gemm_ws against it, us:
+    //   tiles per SM         32 -> 32      64 -> 32      32 -> 64      64 -> 64      128 -> 64
+    //   3.2 (1 x 240 x 256)  5.8 and 5.6   7.1 and 7.3   7.8 and 6.9   8.8 and 8.8   12.8 and 12.3
+    //   3.2 (1 x 160 x 384)  5.7 and 6.5   7.1 and 9.0   7.9 and 8.0   8.8 and 10.3  12.8 and 15.1
+    //   6.7 (2 x 256 x 256)  8.5 and 6.9   10.8 and 8.7  11.5 and 8.9  13.5 and 10.8 21.2 and 16.5
+    // and rows of 64 pixels, half a tile, 64 -> 64 channels, 16 x 64 x 64 12.3 and 16.4
+    const bool whole = sm_count() % (nx * B) == 0 || (bn == 64 && bk == 32);
     const bool roll = N <= bn && bn <= 64 && (C == bk || (C == 128 && bn == 64 && row3)) && nx * kBM * 5 <= 8LL * W &&
-                      total >= 3LL * sm_count() && total <= 0x7fffffffLL;
+                      (whole ? total >= 3LL * sm_count() : total > 4LL * sm_count()) && total <= 0x7fffffffLL;
     row3 = row3 || roll;
     CUtensorMap ta, tb;
     if (roll)
@@ -1712,7 +1716,7 @@ static cudaError_t conv3x3(const void* X, int B, int H, int W, int C, int cpitch
     geo.row3 = row3 ? 1 : 0;
     const int M = B * H * W, K = 9 * C;
     if (roll) {
-        const int ctas = total < sm_count() ? (int)total : sm_count();
+        const int ctas = sm_count();
 #define NN_ROLL(BNV, BKV, CBLV)                                                                                      \
     return out_bf16 ? launch_roll<BNV, true, BKV, CBLV>(ta, tb, D, bias, N, ldd, relu, W, H, (int)nx, (int)total,    \
                                                         ctas, sh, s)                                                 \

@@ -134,3 +134,23 @@ def test_packing_few_channels(env):
         return fn
 
     assert _ratio(torch, call(8), call(32)) < 0.55
+
+
+# two images of as many pixels and tiles, whose columns of tiles end at the ends of
+# CTAs' runs (two columns) and within them (three): 1.0, and 1.2 where the
+# column-walking kernel took the second on three tiles per SM as well
+@pytest.mark.parametrize("C,N", [(64, 64), (128, 64)])
+def test_convolutions_of_three_columns(env, C, N):
+    torch, lib = env
+    W = torch.randn(N, 9 * C, device="cuda").bfloat16()
+
+    def call(H, width):
+        X = torch.randn(H, width, C, device="cuda").bfloat16()
+        D = torch.empty(H, width, N, dtype=torch.bfloat16, device="cuda")
+
+        def fn():
+            assert lib.lbm_nn_conv3x3(X.data_ptr(), 1, H, width, C, C, W.data_ptr(), 9 * C, D.data_ptr(), N, None, N, 0,
+                                      1, torch.cuda.current_stream().cuda_stream) == 0
+        return fn
+
+    assert _ratio(torch, call(160, 384), call(240, 256)) < 1.09
