@@ -1225,13 +1225,19 @@ cudaError_t coupled_step(const StepParams& P, int n_sub, StepBuffers& B, cudaStr
     // walls: with skip_walls wall passes are left out and the next step,
     // launched with `repair`, updates the walls as it loads them
     // (coupled_tile); only steps with one flow step per coupled step do that:
-    // flow sub-steps start from updated walls.  Up to kFoldNodes every pass is
-    // left out: two launches of few threads cost more than the wall code in the
-    // step (100^2 forced flow 5.9 -> 4.4 us per step, 777 x 500 16.0 -> 14.7);
-    // on larger grids, where the row pass is under 4 us of a step and the step's
-    // own speed counts for more (1500^2 FP16 69.4 against 70.6 us), only the
-    // columns' strided pass.
-    const bool all = !wfb && !(P.periodic_x && P.periodic_y) && (long long)P.nx * P.ny <= kFoldNodes;
+    // flow sub-steps start from updated walls.  With walls at the bottom and top every
+    // pass is left out up to kFoldNodes: two launches of few threads cost more than the
+    // wall code in the step (100^2 forced flow 5.9 -> 4.4 us per step, 777 x 500 16.0 ->
+    // 14.7); otherwise only the columns' strided pass.  The line is where FP16 stops
+    // gaining: rows left to the step against the row pass, us per step with walls all round
+    //          724^2              1024^2             1448^2             2048^2
+    //   FP32   21.0 and 22.0      40.7 and 42.1      77.5 and 78.7      148.2 and 149.3
+    //   FP16   17.5 and 17.8      35.1 and 35.6      65.8 and 65.4      122.6 and 120.2
+    //   BF16   17.6 and 18.2      34.6 and 35.7      65.4 and 66.4      121.3 and 122.3
+    // (at 4096^2 FP32 is 3.5 % slower with them).  Without walls at the bottom and top
+    // there is no row pass to save, and the columns alone are the faster, 600 x 500 nodes
+    // 10.4 us a step against 10.8.
+    const bool all = !wfb && !P.periodic_y && (long long)P.nx * P.ny <= kFoldNodes;
     const bool columns = !wfb && !P.periodic_x && !all;
     const int wfix = all || columns ? repair : 0;
     if (all && grain)
