@@ -183,12 +183,15 @@ LBM_API int lbm_init_fields(lbm_handle* h, const double* fields, const double* o
  * four models, then the wall kernels, then n_sub - 1 flow-only sub-steps) on
  * the handle's stream and return without waiting.  Long runs are replayed
  * from captured 16-step CUDA graphs; inside one, and in FP32 storage inside
- * the remainder of a call, walls (n_sub = 1; on grids of more than 2^20 nodes the
- * left/right ones) are updated by the next step as it loads them, and the last
- * step runs the wall kernels in full, so the state seen between calls is always
- * complete.  The graph is captured,
- * instantiated and uploaded when a state is set (lbm_init_seeds,
- * lbm_init_fields, lbm_load_state), so the first lbm_step pays none of it. */
+ * the remainder of a call, walls (n_sub = 1; on grids of more than 2^20 nodes or
+ * periodic in y the left/right ones) are updated by the next step as it loads them,
+ * and the last step runs the wall kernels in full, so the state seen between calls is
+ * always complete.  In 16-bit storage left and right walls updated so are not rounded
+ * to the storage type in between, as the wall kernels round them: with such walls the
+ * last bits of a 16-bit result depend on how many of its steps were replayed, that is
+ * on how the steps were split into calls.  The graph is captured, instantiated and
+ * uploaded when a state is set (lbm_init_seeds, lbm_init_fields, lbm_load_state), so
+ * the first lbm_step pays none of it. */
 LBM_API int lbm_step(lbm_handle* h, int nsteps);
 
 /* Wait for all queued work of h; reports an asynchronous CUDA error. */
@@ -308,7 +311,8 @@ LBM_API int lbm_batch_set_stream(lbm_batch* b, void* stream);
 /* Seeded start of one domain (lbm_init_seeds semantics). */
 LBM_API int lbm_batch_init_seeds(lbm_batch* b, int dom, const lbm_seed* seeds, int n_seeds, double U0,
                                  double theta0);
-/* Queue nsteps coupled steps of every domain; all must be initialised. */
+/* Queue nsteps coupled steps of every domain; all must be initialised.  Left and right
+ * walls inside a replayed sequence as for lbm_step. */
 LBM_API int lbm_batch_step(lbm_batch* b, int nsteps);
 LBM_API int lbm_batch_synchronize(lbm_batch* b);
 LBM_API int lbm_batch_get_fields(lbm_batch* b, int dom, unsigned mask, double* out);

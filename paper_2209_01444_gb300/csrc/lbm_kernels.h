@@ -32,10 +32,10 @@ struct StepBuffers {
 };
 
 // One coupled step.  skip_walls: leave out wall passes (n_sub = 1; ignored
-// otherwise): all of them on a grid of up to kFoldNodes nodes (lbm_step.cu), the
-// left/right walls' on a larger one; the next step must then be launched with
-// `repair`, which applies that update to the wall cells as they are loaded.  A
-// state read or kept between calls must come from a step without skip_walls.
+// otherwise): all of them on a grid of up to kFoldNodes nodes (lbm_step.cu) with walls
+// at the bottom and top, the left/right walls' on any other; the next step must then
+// be launched with `repair`, which applies that update to the wall cells as they are
+// loaded.  A state read or kept between calls must come from a step without skip_walls.
 cudaError_t launch_coupled_step(const StepParams& P, int storage, int n_sub, StepBuffers& B, cudaStream_t s,
                                 int repair = 0, int skip_walls = 0);
 

@@ -344,7 +344,11 @@ __device__ __forceinline__ void coupled_node(const StepParams& P, void* __restri
 // the left and right walls; kAllWalls, the bottom and top walls too (rows
 // first: the corners belong to the columns).  Extrapolation depends on the first
 // interior node alone, and the tile and its halo hold that node for every wall
-// cell they hold, so the result is the passes'.
+// cell they hold, so the result is the passes' in FP32.  With 16-bit storage row
+// values are rounded as the row pass stores them, column values (corners among them)
+// are used as they are: the passes' but for that rounding.  (wall_node states the same
+// update for the passes, wall_values and phi_cell for kAllWalls, the code under
+// kColumns for the columns alone: what changes in one changes in all.)
 enum Walls { kNoWalls, kColumns, kAllWalls };
 template <class Store, bool GRAIN, bool WRITE_FB, int TYV, int WALLS = kNoWalls>
 __device__ __forceinline__ void coupled_tile(const StepParams& P, const void* __restrict__ src,

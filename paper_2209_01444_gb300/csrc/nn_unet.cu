@@ -13,13 +13,16 @@
 //   prediction is y = x + std_out * proj1x1(d_0), with the inputs normalised
 //   as (x - mean) / std_in.
 // A 3 x 3 convolution is an implicit GEMM with the bias and ReLU in its epilogue
-// (an im2col gather only for widths that are no multiple of 32 channels); its input
+// (an im2col gather for channels that are no multiple of 32, and for the first layer of
+// images whose rows fit no run of 128 pixels); its input
 // gradient is the same convolution of the output gradient with the
 // 180-degree-rotated kernel, the ReLU mask in the epilogue; its weight gradient
 // contracts input and output gradient over all pixels as they lie in memory
-// (nn_wgrad.cuh), in slices whose partial sums one launch adds at the end.  s_l is written straight into the first half
-// of the concatenation buffer cat_l and u_l into the second half, so the
-// concatenation costs nothing.
+// (nn_wgrad.cuh) on levels whose rows are a multiple of 32 pixels, and from transposed
+// copies on the others, in slices whose partial sums one launch adds at the end.  (Five
+// levels are all of the first kind where the image's rows are a multiple of 512 pixels.)
+// s_l is written straight into the first half of the concatenation buffer cat_l and u_l
+// into the second half, so the concatenation costs nothing.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -292,7 +295,7 @@ cudaError_t allocate(lbm_unet* u)
         if (v.up.cout) UN_ALLOC(v.up.wt, 8LL * c * c);
     }
     // gathered-copy buffer for the convolutions the implicit kernel does not
-    // take (the first one, 8 input channels; channels no multiple of 32)
+    // take (the first one without wpad, 8 input channels; channels no multiple of 32)
     long long col_n = 9LL * P0 * kInPitch;
     for (const Level& v : u->lv)
         for (const Conv* cv : {&v.ea, &v.eb, &v.da, &v.db})
