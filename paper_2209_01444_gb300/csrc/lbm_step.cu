@@ -679,50 +679,61 @@ __device__ __forceinline__ void flow_collide(const StepParams& P, float phi, flo
     collide_flow<1, Store::kSF>(h, m, P.s2u, ho);
 }
 
-// The same for two nodes at once, in packed FP32 (one instruction for both), with
-// the sums that directions share taken once: of flow_macros and collide_flow
-// 68 operations are left of 94 (their packed form runs at half rate, so the FMA
-// pipe, not the issue slots, sets the pace of a collision).
+// The same with FP32 storage, with the sums that directions share taken once: of
+// flow_macros and collide_flow 68 operations are left of 94.  F2: two nodes at once, in
+// packed FP32 (one instruction for both; the packed form runs at half rate, so the FMA
+// pipe, not the issue slots, sets the pace of a collision).  F1: one node, by the same
+// operations in the same order, so that a step alone and several to a launch give the
+// same bits.
 struct F2 {
     float2 v;
+    static __device__ __forceinline__ F2 of(float a) { return {make_float2(a, a)}; }
 };
-__device__ __forceinline__ F2 f2(float a) { return {make_float2(a, a)}; }
+struct F1 {
+    float v;
+    static __device__ __forceinline__ F1 of(float a) { return {a}; }
+};
 __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) { return {__ffma2_rn(a.v, b.v, c.v)}; }
 __device__ __forceinline__ F2 operator+(F2 a, F2 b) { return {__fadd2_rn(a.v, b.v)}; }
-__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return fma2(b, f2(-1.0f), a); }
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) { return fma2(b, F2::of(-1.0f), a); }
 __device__ __forceinline__ F2 operator*(F2 a, F2 b) { return {__fmul2_rn(a.v, b.v)}; }
+__device__ __forceinline__ F1 fma2(F1 a, F1 b, F1 c) { return {__fmaf_rn(a.v, b.v, c.v)}; }
+__device__ __forceinline__ F1 operator+(F1 a, F1 b) { return {__fadd_rn(a.v, b.v)}; }
+__device__ __forceinline__ F1 operator-(F1 a, F1 b) { return {__fsub_rn(a.v, b.v)}; }
+__device__ __forceinline__ F1 operator*(F1 a, F1 b) { return {__fmul_rn(a.v, b.v)}; }
 
 // nw: q~ - 1 = -(1 + phi)/2; hFy: half the body force along y.
-template <class Store>
-__device__ __forceinline__ void flow_collide2(const StepParams& P, F2 nw, F2 hFy, const F2 (&h)[9], F2 (&out)[9])
+template <class Store, class F>
+__device__ __forceinline__ void flow_collide2(const StepParams& P, F nw, F hFy, const F (&h)[9], F (&out)[9])
 {
+    auto f2 = [](float a) { return F::of(a); };
     constexpr float SO = (float)Store::kSF;
-    const F2 half = f2(0.5f), ns2 = f2(-P.s2u), hFx = f2(0.5f * P.Fx);
-    const F2 a = h[5] - h[7], b = h[6] - h[8], e = h[5] + h[7], f = h[6] + h[8];
-    const F2 s13 = h[1] + h[3], s24 = h[2] + h[4], d = e + f;
-    const F2 usx = (h[1] - h[3]) + (a - b) + hFx, usy = (h[2] - h[4]) + (a + b) + hFy;  // u*
-    const F2 mxx = s13 + d, myy = s24 + d, mxy = e - f, rest = mxx + s24;
-    const F2 nt = nw * half;
-    const F2 u = fma2(nt, usx, usx), v = fma2(nt, usy, usy);
-    const F2 p = f2(0.6f) * fma2(f2(-(2.0f / 3.0f)), fma2(u, u, v * v), rest);
+    const F half = f2(0.5f), ns2 = f2(-P.s2u), hFx = f2(0.5f * P.Fx);
+    const F a = h[5] - h[7], b = h[6] - h[8], e = h[5] + h[7], f = h[6] + h[8];
+    const F s13 = h[1] + h[3], s24 = h[2] + h[4], d = e + f;
+    const F usx = (h[1] - h[3]) + (a - b) + hFx, usy = (h[2] - h[4]) + (a + b) + hFy;  // u*
+    const F mxx = s13 + d, myy = s24 + d, mxy = e - f, rest = mxx + s24;
+    const F nt = nw * half;
+    const F u = fma2(nt, usx, usx), v = fma2(nt, usy, usy);
+    const F p = f2(0.6f) * fma2(f2(-(2.0f / 3.0f)), fma2(u, u, v * v), rest);
     // r1 = u + F'_x / 2 with F' = F + (1 - q~) f, f = -u*, and likewise r2
-    const F2 r1 = u + fma2(nt, usx, hFx), r2 = v + fma2(nt, usy, hFy);
-    const F2 pu = fma2(u, u, p);
-    const F2 r3 = fma2(ns2, mxx - pu, mxx);
-    const F2 r4 = fma2(ns2, myy - fma2(v, v, p), myy);
-    const F2 r5 = fma2(ns2, fma2(u * f2(-1.0f), v, mxy), mxy);
-    const F2 r8 = fma2(v, v, pu) * f2(1.0f / 3.0f);
+    const F r1 = u + fma2(nt, usx, hFx), r2 = v + fma2(nt, usy, hFy);
+    const F pu = fma2(u, u, p);
+    const F r3 = fma2(ns2, mxx - pu, mxx);
+    const F r4 = fma2(ns2, myy - fma2(v, v, p), myy);
+    const F r5 = fma2(ns2, fma2(u * f2(-1.0f), v, mxy), mxy);
+    const F r8 = fma2(v, v, pu) * f2(1.0f / 3.0f);
     // (r1 - r7 along the axes, not its equal 2 r7: momentum is kept whatever the
     // rounding of 1/3)
-    const F2 r6 = r2 * f2(1.0f / 3.0f), r7 = r1 * f2(1.0f / 3.0f);
+    const F r6 = r2 * f2(1.0f / 3.0f), r7 = r1 * f2(1.0f / 3.0f);
     out[0] = f2(SO) * (r8 - (r3 + r4));
-    const F2 hO = f2(0.5f * SO), ax = hO * (r3 - r8), ay = hO * (r4 - r8), bx = hO * (r1 - r7), by = hO * (r2 - r6);
+    const F hO = f2(0.5f * SO), ax = hO * (r3 - r8), ay = hO * (r4 - r8), bx = hO * (r1 - r7), by = hO * (r2 - r6);
     out[1] = ax + bx;
     out[3] = ax - bx;
     out[2] = ay + by;
     out[4] = ay - by;
-    const F2 q = f2(0.25f * SO), s = q * (r6 + r7), t = q * (r6 - r7);
-    const F2 c = q * (r8 + r5), g = q * (r8 - r5);
+    const F q = f2(0.25f * SO), s = q * (r6 + r7), t = q * (r6 - r7);
+    const F c = q * (r8 + r5), g = q * (r8 - r5);
     out[5] = c + s;
     out[7] = c - s;
     out[6] = g + t;
@@ -780,7 +791,17 @@ __global__ void __launch_bounds__(256, 8) k_flow_substep(const StepParams P, con
         const bool row = !P.periodic_y && (y == 0 || y == P.ny - 1);
         if (column || row) flow_wall_repair<Store>(P, sc, src, x, y, column, row, h);
     }
-    flow_collide<Store>(P, phi[block_index(o, phi_np)], fb[o], h, ho);
+    const float ph = phi[block_index(o, phi_np)], fy = fb[o];
+    if constexpr (std::is_same<Store, StoreF32>::value) {
+        F1 h1[9], o1[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) h1[i].v = h[i];
+        flow_collide2<Store>(P, F1{-0.5f * (ph + 1.0f)}, F1{0.5f * fy}, h1, o1);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) ho[i] = o1[i].v;
+    } else {
+        flow_collide<Store>(P, ph, fy, h, ho);
+    }
     const int xp = (x + 1 == P.nx) ? 0 : x + 1, xm = (x == 0) ? P.nx - 1 : x - 1;
     const int yp = (y + 1 == P.ny) ? 0 : y + 1, ym = (y == 0) ? P.ny - 1 : y - 1;
     const long long rY = Store::flow_row(y, P), rP = Store::flow_row(yp, P), rM = Store::flow_row(ym, P);
@@ -985,7 +1006,7 @@ __global__ void __launch_bounds__(kFmW* kFmY, 2)
                 F2 h[9];
 #pragma unroll
                 for (int i = 0; i < 9; ++i) h[i].v = make_float2(own[i * PP + PJ * j], own[i * PP + PJ * (j + 1)]);
-                flow_collide2<Store>(P, {make_float2(nw[j], nw[j + 1])}, {make_float2(hfy[j], hfy[j + 1])}, h,
+                flow_collide2<Store>(P, F2{make_float2(nw[j], nw[j + 1])}, F2{make_float2(hfy[j], hfy[j + 1])}, h,
                                      ho[j / 2]);
             } else {
 #pragma unroll
