@@ -648,20 +648,25 @@ __device__ __forceinline__ void flow_wall_from(const StepParams& P, int axis, in
     wall_rest(P, axis, P.bc[side], m, none, none, hi, nb, gb, hb, 1);
 }
 
-// phi + 1 and F_y of the node at offset o, from its scalar populations.
+// phi + 1 and F_y of the node at offset o, from its scalar populations: node_macros'
+// operations, each rounded as written (the compiler may contract those otherwise from
+// kernel to kernel), so that every form of a flow step gives its walls the same bits.
 template <class Store>
 __device__ __forceinline__ float2 flow_wall_scalars(const StepParams& P, const void* __restrict__ sc, long long o)
 {
-    float f[5], n[5], g[5];
-    const float h[9] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    auto sum = [&](int q) {
+        float v = Store::load(sc, nullptr, q, o, P);
 #pragma unroll
-    for (int i = 0; i < 5; ++i) f[i] = Store::load(sc, nullptr, kF + i, o, P);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) n[i] = Store::load(sc, nullptr, kN + i, o, P);
-#pragma unroll
-    for (int i = 0; i < 5; ++i) g[i] = Store::load(sc, nullptr, kG + i, o, P);
-    const Macro m = node_macros(f, n, g, h, P);
-    return make_float2(m.p1, m.Fy);
+        for (int i = 1; i < 5; ++i) v = __fadd_rn(v, Store::load(sc, nullptr, q + i, o, P));
+        return v;
+    };
+    const float p1 = sum(kF), dC = sum(kN), dH = sum(kG);
+    float hp1 = p1;
+    if (P.h_kind == 1)  // h_plus_1
+        hp1 = __fmul_rn(__fmul_rn(__fmul_rn(__fmul_rn(1.875f, p1), p1), p1),
+                        __fmaf_rn(__fmul_rn(0.2f, p1), p1, __fsub_rn(4.0f / 3.0f, p1)));
+    const float dth = __fmaf_rn(P.latent, hp1, dH);
+    return make_float2(p1, __fmaf_rn(P.gbC, __fadd_rn(dC, P.dC_ref), __fmaf_rn(P.gbT, dth, P.Fy)));
 }
 
 // Collision of one flow step at a node: phi and the body force F_y frozen, h
@@ -1069,20 +1074,27 @@ cudaError_t launch_flow_multi(const StepParams& P, const void* src, void* dst, c
                       repair, more);
 }
 
-// Steps per launch for n >= 2 flow steps on an nx x ny grid, or 1 for node by node.
-// In us: a launch of several steps costs about its steps plus 8 of them for loading,
-// the walls' scalars and storing, once for each wave of two CTAs per SM that the
-// regions fill (15 flow steps at 1024^2: K = 4 fills 3 waves and K = 5 four, 818 and
-// 834 us per four coupled steps; at 100^2, one wave, 222 and 205 us).  Node by node a
-// step costs about 4 for its launch and 3.2 for each 64 warps per SM (3 and 2.8 with
-// 16-bit storage).  Where a region covers little more than half its nodes of the grid
-// that is the faster (14 steps of 262140 x 4 nodes, no walls: 190 us against 572 in
-// regions, FP16 180 against 704; of 4 x 262140 FP16 1260 and 1840); not on tall strips with walls
-// at their sides, whose nodes a warp of a step finds one to a row (16 x 65536, FP32: 32
-// steps 1477 and 1086).
+// Steps per launch for n >= 2 flow steps on an nx x ny grid, or 1 for node by node
+// (the same bits).  In us: a launch of several steps costs about its steps plus 8 of
+// them for loading, the walls' scalars and storing (5 where every region has an SM to itself),
+// once for each wave of two CTAs per SM that the regions fill (15 flow steps at 1024^2:
+// K = 4 fills 3 waves and K = 5 four, 818 and 834 us per four coupled steps; at 100^2,
+// one wave, 222 and 205 us).
+//
+// Node by node a step costs its launch and about 3 for each 64 warps per SM.  In a
+// replayed graph (`captured`) that launch is 1.6, and a step's wall repair 0.8 more with
+// rows and 1.5 with columns: the faster on small grids with few steps (coupled steps of
+// n_sub = 3 at 48^2, no walls, 6.3 us against 9.8 in regions, n_sub = 9 16.6 and 19.5).
+// With walls on both axes it gains little (n_sub = 3 19.3 and 20.8, n_sub = 9 36 and 33)
+// and an inflow's corners may round otherwise in the last bit.  Launched directly it is 4 (3 with
+// 16-bit storage), which pays only on long strips, of which a region covers little more than half
+// its nodes (14 steps of 262140 x 4 nodes, no walls: 190 us against 572 in regions, FP16
+// 180 against 704); not on tall strips with walls at their sides, whose nodes
+// a warp of a step finds one to a row (16 x 65536, FP32: 32 steps 1477 and 1086).
 template <class Store>
-int flow_multi_k(const StepParams& P, int n)
+int flow_multi_k(const StepParams& P, int n, bool captured)
 {
+    constexpr bool F32 = std::is_same<Store, StoreF32>::value;
     const int nx = P.nx, ny = P.ny;
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
@@ -1099,9 +1111,12 @@ int flow_multi_k(const StepParams& P, int n)
             regions = tiles;
         }
     }
-    if (regions > 2 * sms && 1.8 * nx * ny < (double)(regions * kFmW * kFmH) && (P.periodic_x || nx >= ny)) {
-        constexpr bool F32 = std::is_same<Store, StoreF32>::value;
-        const double waves = (double)ny * ((nx + 31) / 32) / (64.0 * sms);
+    const double waves = (double)ny * ((nx + 31) / 32) / (64.0 * sms);
+    if (captured && (P.periodic_x || P.periodic_y)) {
+        const double cost = regions <= sms ? 5.2 * ((n + best - 1) / best) + 0.9 * n : (double)least;
+        const double wall = !P.periodic_x ? 1.5 + 3e-4 * ny : !P.periodic_y ? 0.8 : 0.0;
+        if (n * (1.6 + 3.0 * waves) + (n - 1) * wall < 1.1 * cost) return 1;
+    } else if (regions > 2 * sms && 1.8 * nx * ny < (double)(regions * kFmW * kFmH) && (P.periodic_x || nx >= ny)) {
         if (n * ((F32 ? 4.0 : 3.0) + (F32 ? 3.2 : 2.8) * waves) < (double)least) return 1;
     }
     return best;
@@ -1115,7 +1130,9 @@ cudaError_t flow_chain(const StepParams& P, int n, const void* sc, void* const f
                        int phi_np, const float* fb, cudaStream_t s)
 {
     cudaError_t e = cudaSuccess;
-    const int K = n == 1 ? 1 : flow_multi_k<Store>(P, n);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (n > 1 && (e = cudaStreamIsCapturing(s, &cap)) != cudaSuccess) return e;
+    const int K = n == 1 ? 1 : flow_multi_k<Store>(P, n, cap == cudaStreamCaptureStatusActive);
     if (K == 1) {
         const dim3 block(64, 4), grid((P.nx + 63) / 64, (P.ny + 3) / 4);
         for (int k = 0; k < n && e == cudaSuccess; ++k) {

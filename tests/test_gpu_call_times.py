@@ -154,3 +154,17 @@ def test_convolutions_of_three_columns(env, C, N):
         return fn
 
     assert _ratio(torch, call(160, 384), call(240, 256)) < 1.09
+
+
+# coupled steps with three flow steps each, replayed from a graph on a small grid: 2.2
+# times the step with one, 3.5 where the two more went through a region's load and store
+def test_small_grid_with_two_time_scales(env):
+    from paper_2209_01444_gb300 import lbm as L, workloads as W
+
+    torch, _ = env
+    sims = []
+    for n_sub in (3, 1):
+        sim = L.Simulation(W.thermosolutal_params(48, 48, n_sub=n_sub), stream=torch.cuda.current_stream())
+        sim.init_seeds(np.array([[24.0, 24.0, 6.0, 0.0]]), 0.0, -0.55)
+        sims.append(sim)
+    assert _ratio(torch, lambda: sims[0].step(32), lambda: sims[1].step(32), reps=5) < 2.9
