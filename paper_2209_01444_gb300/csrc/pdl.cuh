@@ -23,7 +23,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 // flow steps of 4 x 8000 nodes with four walls 49 against 23 (31).  The same happens
 // on a smaller scale to a kernel released by one that leaves many slots free for long:
 // such a one waits here and releases near its end (k_proj_fwd_vec; k_flow_multi
-// before a wall pass).
+// before a wall pass).  k_conv_roll, which fills every SM, releases first.
 __device__ __forceinline__ void pdl_begin()
 {
     pdl_wait();
